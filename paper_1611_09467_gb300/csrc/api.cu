@@ -114,6 +114,7 @@ struct peps_ctx {
   peps_ctx* parent = nullptr;                        // set on clones (model buffers borrowed)
   DevBuf env, small, O, scratch, gsum, go;
   int chunk = 0;  // configurations per pass
+  int res_small = 0;   // resident CTAs of the one-warp boundary sweeps (0: the model is too large for them)
   int res_boundary = 0, res_row = 0, res_pair = 0, res_mc = 0;  // resident CTAs per kernel
   bool pair_tc = false;  // two-row step on the tensor cores (PEPS_MIXED_TF32, D = 8, Dc = 16)
   // kernel variants (peps_autotune): row_generic 1 takes the generic single-row
@@ -269,6 +270,18 @@ size_t slot_elems(const peps_ctx* c) {
   return (s + 31) / 32 * 32;
 }
 
+// Whether the boundary sweeps take the one-warp kernel.
+bool small_boundary(const peps_ctx* c) { return c->res_small > 0 && boundary_small_fits(c->g); }
+
+// Scratch of the persistent kernels: a slot per resident CTA; the one-warp
+// sweeps keep one boundary MPS each.
+size_t scratch_bytes(const peps_ctx* c, int slots) {
+  const Geometry& g = c->g;
+  size_t e = slot_elems(c) * slots;
+  if (small_boundary(c)) e = std::max(e, (size_t)c->res_small * g.Lx * g.Dc * g.D * g.Dc);
+  return e * c->elem;
+}
+
 peps_status ensure_workspace(peps_ctx* c, int n, bool want_O) {
   const Geometry& g = c->g;
   const double budget = (c->p.workspace_gb > 0 ? c->p.workspace_gb : 24.0) * 1e9;
@@ -281,7 +294,7 @@ peps_status ensure_workspace(peps_ctx* c, int n, bool want_O) {
   PEPS_CUDA(c->env.ensure(env_bytes_per_cfg(c) * chunk));
   PEPS_CUDA(c->small.ensure(Small::bytes(chunk, g.Ly)));
   if (want_O) PEPS_CUDA(c->O.ensure((size_t)chunk * g.N * D4 * c->elem));
-  PEPS_CUDA(c->scratch.ensure(slot_elems(c) * c->elem * c->nslots));
+  PEPS_CUDA(c->scratch.ensure(scratch_bytes(c, c->nslots)));
   const void* after[4] = {c->env.p, c->small.p, c->O.p, c->scratch.p};
   for (int i = 0; i < 4; ++i)
     if (before[i] != after[i]) ++c->ws_gen;   // captured graphs that read the old buffers are stale
@@ -391,9 +404,15 @@ peps_status evaluate_chunk(peps_ctx* c, const uint64_t* S, int n, bool need_env_
   PEPS_CUDA(cudaMemsetAsync(sm.flags, 0, (size_t)n * sizeof(int), c->stream));
   const int dirs = need_env_l ? 2 : 1;
   // persistent kernels: never more CTAs than can be resident at once
-  const int res = c->boundary_ctas > 0 ? std::min(c->boundary_ctas, c->res_boundary) : c->res_boundary;
-  int grid = std::min(n * dirs, std::min(c->nslots, res));
-  {
+  if (small_boundary(c)) {
+    const size_t slot = (size_t)c->g.Lx * c->g.Dc * c->g.D * c->g.Dc;
+    Prof pf(c, 0);
+    PEPS_CUDA(launch_boundary_small<R>(a, nullptr, nullptr, 0, dirs, a.scratch, slot,
+                                       boundary_small_smem(c->g, c->elem),
+                                       std::max(std::min(n * dirs, c->res_small), 1), c->stream));
+  } else {
+    const int res = c->boundary_ctas > 0 ? std::min(c->boundary_ctas, c->res_boundary) : c->res_boundary;
+    const int grid = std::min(n * dirs, std::min(c->nslots, res));
     Prof pf(c, 0);
     PEPS_CUDA(launch_boundary<R>(a, dirs, std::max(grid, 1), c->stream));
   }
@@ -676,8 +695,6 @@ peps_status packed_impl(peps_packer* pk, int nreq, peps_ctx* const* ctxs, const 
   const int dirs = any_env ? 2 : 1;
   std::vector<KArgs<R>> args(nreq);
   std::vector<Small> sms(nreq);
-  std::vector<int> start(nreq + 1, 0);
-  size_t slot = 0, smem = 0;
   for (int i = 0; i < nreq; ++i) {
     peps_ctx* c = ctxs[i];
     peps_status st = ensure_workspace(c, n[i], false);
@@ -689,21 +706,45 @@ peps_status packed_impl(peps_packer* pk, int nreq, peps_ctx* const* ctxs, const 
     c->cache_dirty = true;   // the packed launch writes this context's environments without the cache
     args[i].O = (O && O[i]) ? (R*)O[i] : nullptr;
     PEPS_CUDA(cudaMemsetAsync(sms[i].flags, 0, (size_t)n[i] * sizeof(int), pk->stream));
-    start[i + 1] = start[i] + n[i] * dirs;
-    slot = std::max(slot, boundary_slot_elems(c->g, c->wm_smem));
-    smem = std::max(smem, dyn_smem_bytes(c->g, sizeof(R), true, c->wm_smem));
   }
-  slot = (slot + 31) / 32 * 32;
-  const int total = start[nreq];
-  const int grid = std::max(1, std::min(total, max_blocks_boundary_packed<R>(smem)));
-  PEPS_CUDA(pk->scratch.ensure(slot * sizeof(R) * grid));
+  // one launch for the models swept by one warp each and one for the others;
+  // both tables go to the device in one copy each, the small models' first
+  std::vector<KArgs<R>> models;
+  std::vector<int> start;
+  int first1 = 0, nm[2] = {0, 0}, total[2] = {0, 0}, grid[2] = {0, 0};
+  size_t slot[2] = {0, 0}, smem[2] = {0, 0};
+  for (int cls = 0; cls < 2; ++cls) {
+    first1 = (int)models.size();   // after the last pass: where the second class begins
+    start.push_back(0);
+    for (int i = 0; i < nreq; ++i) {
+      const peps_ctx* c = ctxs[i];
+      const Geometry& g = c->g;
+      if (small_boundary(c) != (cls == 0)) continue;
+      models.push_back(args[i]);
+      total[cls] += n[i] * dirs;
+      start.push_back(total[cls]);
+      ++nm[cls];
+      slot[cls] = std::max(slot[cls], cls == 0 ? (size_t)g.Lx * g.Dc * g.D * g.Dc : boundary_slot_elems(g, c->wm_smem));
+      smem[cls] = std::max(smem[cls], cls == 0 ? boundary_small_smem(g, sizeof(R))
+                                               : dyn_smem_bytes(g, sizeof(R), true, c->wm_smem));
+    }
+    slot[cls] = (slot[cls] + 31) / 32 * 32;
+    if (nm[cls])
+      grid[cls] = std::max(1, std::min(total[cls], cls == 0 ? max_blocks_boundary_small<R>(smem[cls])
+                                                            : max_blocks_boundary_packed<R>(smem[cls])));
+  }
+  PEPS_CUDA(pk->scratch.ensure(sizeof(R) * std::max(slot[0] * grid[0], slot[1] * grid[1])));
   PEPS_CUDA(pk->models.ensure(sizeof(KArgs<R>) * nreq));
-  PEPS_CUDA(pk->start.ensure(sizeof(int) * (nreq + 1)));
+  PEPS_CUDA(pk->start.ensure(sizeof(int) * (nreq + 2)));
   // pageable sources: the copies have taken the data when the calls return
-  PEPS_CUDA(cudaMemcpyAsync(pk->models.p, args.data(), sizeof(KArgs<R>) * nreq, cudaMemcpyHostToDevice, pk->stream));
-  PEPS_CUDA(cudaMemcpyAsync(pk->start.p, start.data(), sizeof(int) * (nreq + 1), cudaMemcpyHostToDevice, pk->stream));
-  PEPS_CUDA(launch_boundary_packed<R>((const KArgs<R>*)pk->models.p, (const int*)pk->start.p, nreq, dirs,
-                                      (R*)pk->scratch.p, slot, smem, grid, pk->stream));
+  PEPS_CUDA(cudaMemcpyAsync(pk->models.p, models.data(), sizeof(KArgs<R>) * nreq, cudaMemcpyHostToDevice, pk->stream));
+  PEPS_CUDA(cudaMemcpyAsync(pk->start.p, start.data(), sizeof(int) * (nreq + 2), cudaMemcpyHostToDevice, pk->stream));
+  if (nm[0])
+    PEPS_CUDA(launch_boundary_small<R>(models[0], (const KArgs<R>*)pk->models.p, (const int*)pk->start.p, nm[0], dirs,
+                                       (R*)pk->scratch.p, slot[0], smem[0], grid[0], pk->stream));
+  if (nm[1])
+    PEPS_CUDA(launch_boundary_packed<R>((const KArgs<R>*)pk->models.p + first1, (const int*)pk->start.p + nm[0] + 1,
+                                        nm[1], dirs, (R*)pk->scratch.p, slot[1], smem[1], grid[1], pk->stream));
   for (int i = 0; i < nreq; ++i) {
     peps_ctx* c = ctxs[i];
     const bool want_e = eloc && eloc[i], want_O = O && O[i];
@@ -783,6 +824,7 @@ peps_ctx* ctx_clone(peps_ctx* c, cudaStream_t stream, double workspace_gb, int s
   k->wm_smem = c->wm_smem;
   // a worker that shares the GPU with `share` lanes sizes its persistent grids to its part
   auto part = [&](int r) { return std::max(std::min(r, c->nsm), r / std::max(share, 1)); };
+  k->res_small = part(c->res_small);
   k->res_boundary = part(c->res_boundary);
   k->res_row = part(c->res_row);
   k->res_pair = part(c->res_pair);
@@ -812,7 +854,7 @@ size_t ctx_footprint(peps_ctx* c, int n, double workspace_gb, int share) {
   size_t chunk = (size_t)std::max<double>(1.0, std::floor(budget / (double)per));
   chunk = std::min(chunk, (size_t)std::max(n, 1));
   const int part = std::max(std::min(c->nslots, c->nsm), c->nslots / std::max(share, 1));
-  return per * chunk + Small::bytes((int)chunk, c->g.Ly) + slot_elems(c) * c->elem * part;
+  return per * chunk + Small::bytes((int)chunk, c->g.Ly) + scratch_bytes(c, part);
 }
 
 size_t ctx_workspace_bytes(peps_ctx* c) {
@@ -888,6 +930,11 @@ peps_status peps_create(const peps_params* p, const double* A_host, void* stream
     return cuda_fail(e, "device query");
   }
   c->wm_smem = wm_fits_smem(c->g, c->elem);
+  if (boundary_small_fits(c->g)) {
+    const size_t smem = boundary_small_smem(c->g, c->elem);
+    c->res_small = c->elem == 8 ? max_blocks_boundary_small<double>(smem)
+                                : max_blocks_boundary_small<float>(smem);
+  }
   if (c->elem == 8) {
     c->res_boundary = max_blocks_boundary<double>(c->g);
     c->res_row = max_blocks_row<double>(c->g);

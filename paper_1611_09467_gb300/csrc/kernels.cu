@@ -25,6 +25,7 @@
 #include <mutex>
 
 #include "kernels_common.cuh"
+#include "boundary_item.cuh"
 
 namespace peps {
 
@@ -72,77 +73,6 @@ size_t mc_slot_elems(const Geometry& g, bool wm_in_smem) {
 }
 
 // ------------------------------------------------------------ k_boundary
-// One work item: the top-down (dir 0) or bottom-up (dir 1) boundary sweep of
-// configuration cfg.  The upper environments U_r go to envU (the last row's
-// MPS to `lastbuf`, then closed to psi), the lower ones L_r to envL.
-template <typename R>
-__device__ void boundary_item(const KArgs<R>& a, int cfg, int dir, R* lastbuf, ZipBufs<R>& zb, R* red,
-                              uint64_t* sp, const int* ones) {
-  const Geometry& g = a.g;
-  const int Lx = g.Lx, Ly = g.Ly, Dc = g.Dc, D = g.D;
-  const size_t envT = (size_t)Dc * D * Dc;
-  if (a.cache) {
-    // this sweep of this configuration is already in place (same bits, same
-    // tensors, same workspace): its outputs were kept, only its flag is raised again
-    const unsigned bits = a.cache[cfg];
-    if (bits & (1u << dir)) {
-      if ((bits & (4u << dir)) && threadIdx.x == 0) atomicOr(&a.flags[cfg], kFlagZeroW);
-      return;
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < g.nwords; i += blockDim.x) sp[i] = a.S[(size_t)cfg * g.nwords + i];
-  __syncthreads();
-  const R* Min = a.triv_mps;
-  double ls = 0.0;
-  bool zero = false;
-  for (int j = 0; j < Ly; ++j) {
-    const int r = dir == 0 ? j : Ly - 1 - j;
-    if (dir == 1 && r == 0) break;
-    R* Mout;
-    if (dir == 0) Mout = r <= Ly - 2 ? a.envU + ((size_t)cfg * Ly + r) * Lx * envT : lastbuf;
-    else Mout = a.envL + ((size_t)cfg * Ly + r) * Lx * envT;
-    const int* bdin = j == 0 ? ones : a.bd + ((size_t)dir * Ly + (j - 1)) * (Lx + 1);
-    const double nrm = absorb_row<R>(a, Min, Mout, r, dir, (j % 2) == 0, bdin, sp, zb, red);
-    if (!(nrm > 0.0)) zero = true;
-    else ls += log(nrm);
-    if (dir == 0 && a.lnU && threadIdx.x == 0) a.lnU[(size_t)cfg * Ly + r] = nrm > 0.0 ? log(nrm) : -INFINITY;
-    Min = Mout;
-  }
-  if (dir == 0) {
-    // All physical legs are one now: close the chain of matrices M_c[:, 0, :].
-    __shared__ R vec[kMaxDc], nv[kMaxDc];
-    if (threadIdx.x == 0) {
-      const int* bdl = a.bd + ((size_t)0 * Ly + (Ly - 1)) * (Lx + 1);
-      vec[0] = R(1);
-      int na = 1;
-      for (int c = 0; c < Lx; ++c) {
-        const int nb = bdl[c + 1];
-        const R* M = lastbuf + (size_t)c * envT;
-        for (int b = 0; b < nb; ++b) {
-          R s = R(0);
-          for (int x = 0; x < na; ++x) s += vec[x] * M[(size_t)x * D * Dc + b];
-          nv[b] = s;
-        }
-        for (int b = 0; b < nb; ++b) vec[b] = nv[b];
-        na = nb;
-      }
-      const R v = vec[0];
-      if (zero || v == R(0)) {
-        a.logabs[cfg] = -INFINITY;
-        a.sign[cfg] = 0;
-        atomicOr(&a.flags[cfg], kFlagZeroW);
-      } else {
-        a.logabs[cfg] = ls + log(fabs((double)v));
-        a.sign[cfg] = v > R(0) ? 1 : -1;
-      }
-    }
-  } else if (zero && threadIdx.x == 0) {
-    atomicOr(&a.flags[cfg], kFlagZeroW);
-  }
-  if (a.cache && threadIdx.x == 0) atomicOr(&a.cache[cfg], (1u << dir) | (zero ? (4u << dir) : 0u));
-}
-
 __global__ void k_cache_check(const uint64_t* S, uint64_t* Scache, unsigned* bits, int n, int nwords) {
   for (int cfg = blockIdx.x * blockDim.x + threadIdx.x; cfg < n; cfg += gridDim.x * blockDim.x) {
     bool same = true;
@@ -178,8 +108,11 @@ __global__ void __launch_bounds__(kThreads) k_boundary(KArgs<R> a, int dirs) {
   for (int i = threadIdx.x; i <= g.Lx; i += blockDim.x) ones[i] = 1;
   // items direction-major: consecutive items (one per CTA) share a direction,
   // so sweeps the environment cache skips do not leave half the CTAs idle
+  auto absorb = [&](const R* Min, R* Mout, int r, int dir, bool lr, const int* bdin) {
+    return absorb_row<R>(a, Min, Mout, r, dir, lr, bdin, sp, zb, red);
+  };
   for (int item = blockIdx.x; item < a.n * dirs; item += gridDim.x)
-    boundary_item<R>(a, item % a.n, item / a.n, p, zb, red, sp, ones);
+    boundary_item<R>(a, item % a.n, item / a.n, p, sp, ones, absorb);
 }
 
 // The boundary sweeps of several models (lattices, D, Dc of one precision) in
@@ -219,7 +152,10 @@ __global__ void __launch_bounds__(kThreads) k_boundary_packed(const KArgs<R>* __
       cur = m;
     }
     const int local = item - start[m];
-    boundary_item<R>(a, local % a.n, local / a.n, p, zb, red, sp, ones);
+    boundary_item<R>(a, local % a.n, local / a.n, p, sp, ones,
+                     [&](const R* Min, R* Mout, int r, int dir, bool lr, const int* bdin) {
+                       return absorb_row<R>(a, Min, Mout, r, dir, lr, bdin, sp, zb, red);
+                     });
   }
 }
 
@@ -496,7 +432,7 @@ cudaError_t launch_boundary_packed(const KArgs<R>* models_dev, const int* start_
 #define PEPS_INST(R)                                                                                    \
   template int max_blocks_boundary_packed<R>(size_t);                                                   \
   template cudaError_t launch_boundary_packed<R>(const KArgs<R>*, const int*, int, int, R*, size_t, size_t, \
-                                                 int, cudaStream_t);                                    \
+                                                 int, cudaStream_t);                                   \
   template int max_blocks_boundary<R>(const Geometry&);                                                 \
   template cudaError_t launch_boundary<R>(const KArgs<R>&, int, int, cudaStream_t);                     \
   template cudaError_t launch_grad_accum<R>(const GradArgs&, const R*, cudaStream_t);

@@ -77,6 +77,15 @@ template <typename R> cudaError_t launch_mc(const KArgs<R>& a, uint64_t* S, int 
                                             uint64_t chain0, uint64_t sweep0, long long* accepted,
                                             int grid, cudaStream_t st);
 template <typename R> int max_blocks_boundary(const Geometry& g);
+// Boundary sweeps with one warp per sweep (small.cuh), for the models
+// boundary_small_fits accepts: of one model (nm = 0) or packed as below; a slot
+// is one boundary MPS, the resident count is for smem bytes of shared memory.
+bool boundary_small_fits(const Geometry& g);
+size_t boundary_small_smem(const Geometry& g, size_t elem);
+template <typename R> int max_blocks_boundary_small(size_t smem);
+template <typename R> cudaError_t launch_boundary_small(const KArgs<R>& one, const KArgs<R>* models_dev,
+                                                        const int* start_dev, int nm, int dirs, R* scratch,
+                                                        size_t slot_elems, size_t smem, int grid, cudaStream_t st);
 // Boundary sweeps of several models in one launch (k_boundary_packed): models_dev
 // [nm] kernel arguments in device memory, start_dev [nm + 1] first work item of
 // each model (n * dirs items per model), one scratch slot of slot_elems reals
