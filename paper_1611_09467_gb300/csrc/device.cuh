@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "contract.cuh"
+#include "sturm64.cuh"
 
 // Phase markers inside the truncation.  Empty in the library; the
 // diagnostic build (-DPEPS_PHASE_TIMING, phase_timing.py) makes thread 0 of
@@ -35,6 +36,7 @@ namespace peps {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int kMaxT2Shared = 256;   // reals of TruncWork::wv
 
 template <typename R> struct Eps;
 template <> struct Eps<double> {
@@ -514,7 +516,6 @@ struct TruncWork {
   R* t;       // 2 * Qmax off-diagonal of the Golub-Kahan form
   R* t2;      // squares of t
   R* lam;     // Kmax
-  R* Z;       // Kmax x 2Qmax
   R* lu;      // Kmax x 6 x 2Qmax: inverse-iteration workspace when it is not in shared memory
   R* Ub;      // Qmax x Kmax (unused when Ubs is set)
   R* Uk;      // Pmax x Kmax compact copy of the result in global memory
@@ -525,6 +526,7 @@ struct TruncWork {
   R* gsm;     // GEMM shared scratch (may alias Wm: used only after the reflectors are dead)
   int* gism;
   int Qmax;
+  int Kmax;        // Ubs and Uks hold Qmax x Kmax
   int wm_shared;   // Wm is in shared memory
 };
 
@@ -535,7 +537,6 @@ PEPS_HD size_t trunc_ws_elems(int pq, int kmax, bool with_wm) {
   e += (size_t)pq * (pq + 1);             // Wg
   e += 4 * (size_t)pq + 2 * (size_t)pq * 2;   // tau + scale factors (4 pq), t, t2
   e += kmax;                              // lam
-  e += (size_t)kmax * 2 * pq;             // Z
   e += (size_t)kmax * 6 * 2 * pq;         // lu
   e += (size_t)pq * kmax * 2;             // Ub, Uk
   return e + 64;
@@ -571,55 +572,135 @@ __device__ __forceinline__ void householder_fast(float alpha, float ss, float& t
   }
 }
 
-// Division inside the Sturm counts and the inverse-iteration factorisation:
-// IEEE in FP64, the hardware approximation (2 ulp) in FP32, where it sits on
-// a long dependent chain.
+// Division inside the inverse-iteration factorisation: IEEE in FP64, the
+// hardware approximation (2 ulp) in FP32, where it sits on a long dependent
+// chain.
 __device__ __forceinline__ double sturm_div(double a, double b) { return a / b; }
 __device__ __forceinline__ float sturm_div(float a, float b) { return __fdividef(a, b); }
 
+// One FP32 Sturm step: the next pivot q of T - x (zero diagonal, squared
+// off-diagonal t2) and whether it is negative.  The quotient t2 / q is t2 times
+// the hardware reciprocal of q, fused with the subtraction; __fdividef's
+// scaling for |q| > 2^126 is not needed, as the clamp keeps
+// |q| >= pivmin >= 2^-116 tmax^2, so |t2 / q| stays below 2^117.
+__device__ __forceinline__ int sturm_count_step(float& q, float x, float t2, float pivmin) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
+  q = __fmaf_rn(-t2, r, -x);
+  if (fabsf(q) < pivmin) q = -pivmin;
+  return (int)(__float_as_uint(q) >> 31);
+}
+
 // Number of eigenvalues below x of the zero-diagonal symmetric tridiagonal
 // with squared off-diagonals t2 (pivots of the LDL^T factorisation of T - x).
-template <typename R>
-__device__ int sturm_count(const R* t2, int n2, R x, R pivmin) {
-  int cnt = 0;
-  R q = -x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  if (q < R(0)) ++cnt;
-  for (int i = 1; i < n2; ++i) {
-    q = -x - sturm_div(t2[i - 1], q);
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < R(0)) ++cnt;
-  }
+__device__ __forceinline__ int sturm_count(const float* t2, int n2, float x, float pivmin) {
+  float q = -x;
+  if (fabsf(q) < pivmin) q = -pivmin;
+  int cnt = q < 0.f ? 1 : 0;
+#pragma unroll 4
+  for (int i = 1; i < n2; ++i) cnt += sturm_count_step(q, x, t2[i - 1], pivmin);
   return cnt;
+}
+
+// The K largest eigenvalues by sections, with the whole CTA: G threads count at
+// G points of a value's interval per step.
+static __device__ __noinline__ void section_f32(const float* t2, int n2, int K, float bound, float pivmin, float* lam) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int G = K <= 16 ? 16 : 8;
+  const int nit = K <= 16 ? 7 : 9;   // (G + 1)^nit >= 2^26: the last interval is below a quarter ulp of the bound
+  const int gid = tid / G, gl = tid % G;
+  const int gbase = (lane / G) * G;
+  const int idx = n2 - 1 - gid;  // ascending index of the (gid+1)-th largest eigenvalue
+  float lo = 0.f, hi = bound;
+  for (int it = 0; it < nit; ++it) {
+    const float step = (hi - lo) / float(G + 1);
+    bool pred = true;
+    if (gid < K) {
+      const float x = lo + step * float(gl + 1);
+      pred = sturm_count(t2, n2, x, pivmin) <= idx;
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, pred);
+    const unsigned bits = (bal >> gbase) & ((1u << G) - 1u);
+    const int gstar = __popc(bits) - 1;
+    const float nlo = gstar >= 0 ? lo + step * float(gstar + 1) : lo;
+    const float nhi = gstar + 1 < G ? lo + step * float(gstar + 2) : hi;
+    lo = nlo;
+    hi = nhi;
+  }
+  if (gid < K && gl == 0) lam[gid] = 0.5f * (lo + hi);
 }
 
 // Inverse iteration for one eigenvalue of the n2 x n2 zero-diagonal
 // symmetric tridiagonal with off-diagonal t: Gaussian elimination with
 // partial pivoting on (T - lam I), two solves from a fixed pseudo-random
-// start vector.  Sequential, one thread per eigenvalue.  Five passes over
-// the vector: factorisation fused with the first forward elimination, back
-// substitution, the second forward elimination (which also applies the
-// scaling of the first iterate), back substitution, and the output pass.
-// Each iterate is scaled only by its largest entry (the solve can amplify by
-// 1/pivtiny); the caller normalises the vectors.  The recurrences carry their
-// running values in registers; memory only receives the factors and reads
-// back values that do not depend on the running recurrence, so loads can be
-// issued ahead.  Workspace: four real arrays (reciprocal pivots, first
-// super-diagonal of U, multipliers of L, right-hand side) and one byte per
-// row for the interchanges, each interleaved across the K threads (element i
-// of thread k at i * K + k) so lock-step accesses of a warp are contiguous.
-// The second super-diagonal of U is t[i+1] where rows i, i+1 were
-// interchanged and zero otherwise, so it is not stored.
+// start vector.  Sequential, one thread per eigenvalue, so it is bound by the
+// latency of its recurrences.  Four passes over the vector: factorisation
+// fused with the first forward elimination, back substitution, the second
+// forward elimination (which also applies the scaling of the first iterate),
+// back substitution; the last scaling is left to the reader of the vector
+// (the return value).  Each iterate is scaled only by its largest entry (the
+// solve can amplify by 1/pivtiny); the caller normalises the vectors.
+// Row interchanges are selects, not branches: lanes that differ would run both
+// sides one after the other, with a division in each.  One warp issues all of
+// it, so instructions count: a row's reciprocal pivot, first super-diagonal of
+// U, multiplier of L and right-hand side are one 16-byte group (32 in FP64),
+// row i of vector k at group i * K + k, and the interchange flag is the top
+// exponent bit of the multiplier (|l| <= 1 leaves it free).  The passes over
+// stored rows read them a block of four ahead, since the stores in between keep
+// the compiler from doing so.  FP32 has two approximate divisions per row; FP64
+// one (the multiplier is formed from the pivot's reciprocal).  The second
+// super-diagonal of U is t[i+1] where rows i, i+1 were interchanged and zero
+// otherwise, so it is not stored.  The iterate is left in the fourth entries.
 template <typename R>
-__device__ void inverse_iteration(const R* t, int n2, R lam, R pivtiny, R* wsR, unsigned char* wsP, int K, int k,
-                                  R* z, int zs, unsigned seed) {
-  const size_t st = (size_t)n2 * K;
-  R* rdd = wsR + k;      // reciprocal pivots of U
-  R* du = rdd + st;      // first super-diagonal of U
-  R* mult = du + st;     // multipliers of L
-  R* b = mult + st;      // right-hand side / solution
-  unsigned char* piv = wsP + k;   // 1 where rows i, i+1 were interchanged
-#define IX(i) ((size_t)(i) * K)
+struct InvRow {
+  R rdd, du, mult, b;
+};
+__device__ __forceinline__ InvRow<float> inv_load(const float* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ InvRow<double> inv_load(const double* p) {
+  const double2 u = *reinterpret_cast<const double2*>(p), v = *reinterpret_cast<const double2*>(p + 2);
+  return {u.x, u.y, v.x, v.y};
+}
+__device__ __forceinline__ void inv_store(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void inv_store(double* p, double a, double b, double c, double d) {
+  *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(c, d);
+}
+__device__ __forceinline__ float flag_set(float x, bool f) {
+  return __uint_as_float(__float_as_uint(x) | (f ? 0x40000000u : 0u));
+}
+__device__ __forceinline__ double flag_set(double x, bool f) {
+  return __hiloint2double(__double2hiint(x) | (f ? 0x40000000 : 0), __double2loint(x));
+}
+__device__ __forceinline__ bool flag_get(float x) { return __float_as_uint(x) & 0x40000000u; }
+__device__ __forceinline__ bool flag_get(double x) { return __double2hiint(x) & 0x40000000; }
+__device__ __forceinline__ float flag_clear(float x) { return __uint_as_float(__float_as_uint(x) & ~0x40000000u); }
+__device__ __forceinline__ double flag_clear(double x) {
+  return __hiloint2double(__double2hiint(x) & ~0x40000000, __double2loint(x));
+}
+// num / d as __fdividef computes it for normal d below 2^126: the product with
+// the hardware reciprocal, without its scaling steps.
+__device__ __forceinline__ float quick_div(float num, float d) {
+  if (fabsf(d) < 1.17549435e-38f) return __fdividef(num, d);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return __fmul_rn(num, r);
+}
+// The workspace start for `p`: the next multiple of 32 bytes.
+template <typename R>
+__device__ __forceinline__ R* inv_align(R* p) {
+  return reinterpret_cast<R*>((reinterpret_cast<size_t>(p) + 31) / 32 * 32);
+}
+
+template <typename R>
+static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R pivtiny, R* ws, int K, int k,
+                                                   unsigned seed) {
+  R* const w0 = ws + 4 * k;
+  const int st = 4 * K;
   unsigned h = seed * 2654435761u + 12345u;
   auto start = [&]() {
     h ^= h << 13; h ^= h >> 17; h ^= h << 5;
@@ -629,76 +710,115 @@ __device__ void inverse_iteration(const R* t, int n2, R lam, R pivtiny, R* wsR, 
   // du[i+1], with the forward elimination of the start vector (carrying b[i])
   R cur_d = -lam, cur_u = n2 > 1 ? t[0] : R(0);
   R bi = start();
-  for (int i = 0; i < n2 - 1; ++i) {
-    const R sub = t[i];
-    R next_d = -lam;
-    R next_u = i + 1 < n2 - 1 ? t[i + 1] : R(0);
+  R sub = cur_u;
+  R* w = w0;
+#pragma unroll 2
+  for (int i = 0; i < n2 - 1; ++i, w += st) {
+    const R tn = i + 1 < n2 - 1 ? t[i + 1] : R(0);
+    const R nd = -lam;
     const R bn = start();
-    R d_i, u_i, l;
-    if (fabs(cur_d) >= fabs(sub)) {
-      d_i = cur_d == R(0) ? pivtiny : cur_d;
-      l = sturm_div(sub, d_i);
-      u_i = cur_u;
-      next_d -= l * cur_u;
-      piv[IX(i)] = 0;
-      b[IX(i)] = bi;
-      bi = bn - l * bi;
+    const bool sw = !(fabs(cur_d) >= fabs(sub));
+    R d = sw ? sub : (cur_d == R(0) ? pivtiny : cur_d);
+    const R num = sw ? cur_d : sub;
+    R lm, rd;
+    if constexpr (sizeof(R) == 4) {
+      lm = quick_div(num, d);
+      if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
+      rd = quick_div(1.f, d);
     } else {
-      l = sturm_div(cur_d, sub);
-      d_i = sub;
-      u_i = next_d;
-      next_d = cur_u - l * next_d;
-      next_u = -l * next_u;
-      piv[IX(i)] = 1;
-      b[IX(i)] = bn;
-      bi = bi - l * bn;
+      if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
+      rd = R(1) / d;
+      lm = num * rd;
     }
-    if (fabs(d_i) < pivtiny) d_i = d_i < R(0) ? -pivtiny : pivtiny;
-    rdd[IX(i)] = sturm_div(R(1), d_i);
-    du[IX(i)] = u_i;
-    mult[IX(i)] = l;
-    cur_d = next_d;
-    cur_u = next_u;
+    const R u = sw ? nd : cur_u, y = sw ? cur_u : nd;
+    const R bs = sw ? bn : bi, bo = sw ? bi : bn;
+    inv_store(w, rd, u, flag_set(lm, sw), bs);
+    cur_d = fma(-lm, u, y);
+    cur_u = sw ? -lm * tn : tn;
+    bi = fma(-lm, bs, bo);
+    sub = tn;
   }
   if (fabs(cur_d) < pivtiny) cur_d = cur_d < R(0) ? -pivtiny : pivtiny;
-  rdd[IX(n2 - 1)] = sturm_div(R(1), cur_d);
-  du[IX(n2 - 1)] = R(0);
-  piv[IX(n2 - 1)] = 0;
-  b[IX(n2 - 1)] = bi;
+  inv_store(w, sturm_div(R(1), cur_d), R(0), R(0), bi);
+  R* const wl = w;   // the last row
+  constexpr int B = 4;
+  const int rem = n2 % B, nf = (n2 - 1) / B;
   R sc = R(1);   // scale of the current iterate still to be applied
+#pragma unroll 1
   for (int it = 0; it < 2; ++it) {
     if (it == 1) {
-      // ---- forward: row interchanges and L^-1 on the scaled iterate
-      R bf = b[IX(0)] * sc;
-#pragma unroll 4
-      for (int i = 0; i < n2 - 1; ++i) {
-        const R bn = b[IX(i + 1)] * sc;
-        const R l = mult[IX(i)];
-        if (piv[IX(i)] == 0) {
-          b[IX(i)] = bf;
-          bf = bn - l * bf;
-        } else {
-          b[IX(i)] = bn;
-          bf = bf - l * bn;
+      // ---- forward: row interchanges and L^-1 on the scaled iterate; row i
+      // needs its own multiplier and the next row's entry
+      R bf = w0[3] * sc;
+      auto step = [&](R* p, R mult, R bnext) {
+        const R bn = bnext * sc, lm = flag_clear(mult);
+        const bool sw = flag_get(mult);
+        const R bs = sw ? bn : bf, bo = sw ? bf : bn;
+        p[3] = bs;
+        bf = fma(-lm, bs, bo);
+      };
+      R nm[B], nb[B];
+      w = w0;
+      auto load = [&](const R* p) {
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+          nm[q] = p[q * st + 2];
+          nb[q] = p[(q + 1) * st + 3];
         }
+      };
+      if (nf > 0) load(w);
+      for (int blk = 0; blk < nf; ++blk, w += B * st) {
+        R cm[B], cb[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+          cm[q] = nm[q];
+          cb[q] = nb[q];
+        }
+        if (blk + 1 < nf) load(w + B * st);
+#pragma unroll
+        for (int q = 0; q < B; ++q) step(w + q * st, cm[q], cb[q]);
       }
-      b[IX(n2 - 1)] = bf;
+      for (; w != wl; w += st) step(w, w[2], w[st + 3]);
+      wl[3] = bf;
     }
     // ---- backward: U^-1, carrying y[i+1], y[i+2]; track max |y|
     R y1 = R(0), y2 = R(0), mx = R(0);
-#pragma unroll 4
-    for (int i = n2 - 1; i >= 0; --i) {
-      const R du2 = (piv[IX(i)] != 0 && i + 1 < n2 - 1) ? t[i + 1] : R(0);
-      const R y = (b[IX(i)] - du[IX(i)] * y1 - du2 * y2) * rdd[IX(i)];
-      b[IX(i)] = y;
+    auto step = [&](R* p, const InvRow<R>& v, R tn) {
+      const R d2 = flag_get(v.mult) ? tn : R(0);
+      const R y = fma(-d2, y2, fma(-v.du, y1, v.b)) * v.rdd;
+      p[3] = y;
       mx = fmax(mx, fabs(y));
       y2 = y1;
       y1 = y;
+    };
+    int i = n2 - 1;
+    w = wl;
+    for (; i >= n2 - rem; --i, w -= st) step(w, inv_load(w), i + 1 < n2 - 1 ? t[i + 1] : R(0));
+    InvRow<R> nv[B];
+    R nt[B];
+    auto load = [&](const R* p, int j) {   // rows j, j - 1, ..
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        nv[q] = inv_load(p - q * st);
+        nt[q] = j - q + 1 < n2 - 1 ? t[j - q + 1] : R(0);
+      }
+    };
+    if (i >= 0) load(w, i);
+    for (; i >= 0; i -= B, w -= B * st) {
+      InvRow<R> cv[B];
+      R ct[B];
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        cv[q] = nv[q];
+        ct[q] = nt[q];
+      }
+      if (i >= B) load(w - B * st, i - B);
+#pragma unroll
+      for (int q = 0; q < B; ++q) step(w - q * st, cv[q], ct[q]);
     }
     sc = mx > R(0) ? R(1) / mx : R(1);
   }
-  for (int i = 0; i < n2; ++i) z[(size_t)i * zs] = b[IX(i)] * sc;
-#undef IX
+  return sc;
 }
 
 // v[k] for a run-time k
@@ -975,6 +1095,49 @@ static __device__ __noinline__ void bidiag_tiles_f32(const float* X, int n, bool
   __syncthreads();
 }
 
+// The reflectors j = jtop, jtop - 1, .. whose first row j + off lies in rows
+// 16 R0 .. 16 R0 + 15, applied to a column of U (u[r]: row l + 16 r) by a
+// half-warp; returns the next j.  The next reflector's entries are read while
+// the current dot product is reduced.
+template <int R0>
+__device__ __forceinline__ int apply_reflectors(const float* W, int ld, bool tall, int rows, int l, int off, int jtop,
+                                                const float* taus, const float* scs, float (&u)[8]) {
+  const int jlo = max(16 * R0 - off, 0);
+  if (jtop < jlo) return jtop;
+  const int rs = 16 * (tall ? ld : 1), js = tall ? 1 : ld;
+  const float* p = W + (l + 16 * R0) * (tall ? ld : 1) + jtop * js;
+  float w[8];
+  auto load = [&](const float* q) {
+#pragma unroll
+    for (int r = R0; r < 8; ++r) w[r] = l + 16 * r < rows ? q[(r - R0) * rs] : 0.f;
+  };
+  load(p);
+  float tj = taus[jtop], sj = scs[jtop];
+  for (int j = jtop; j >= jlo; --j) {
+    const int i0 = l + 16 * R0, pv = j + off;
+    float v[8], d = 0.f;
+#pragma unroll
+    for (int r = R0; r < 8; ++r) {
+      v[r] = sj * w[r];
+      if (r == R0) v[r] = i0 < pv ? 0.f : (i0 == pv ? 1.f : v[r]);
+      d = fmaf(v[r], u[r], d);
+    }
+    const float tc = tj;
+    if (j > jlo) {
+      p -= js;
+      load(p);
+      tj = taus[j - 1];
+      sj = scs[j - 1];
+    }
+#pragma unroll
+    for (int o = 8; o >= 1; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    const float cf = -tc * d;
+#pragma unroll
+    for (int r = R0; r < 8; ++r) u[r] = fmaf(cf, v[r], u[r]);
+  }
+  return jlo - 1;
+}
+
 // Writes U_K (m x K) through (uo_r, uo_c) and C' = U_K^T X (K x n) through
 // (co_r, co_c).  X is not modified.  K <= min(m, n), K <= 32.
 template <typename R>
@@ -1166,68 +1329,62 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
     __syncthreads();
   }   // !tiled
   PEPS_PHASE(1);
-  // ---------------- Sturm bisection for the K largest singular values
+  // ---------------- Sturm sections for the K largest singular values
   const int n2 = 2 * Q;
   R tmax = R(0);
-  for (int i = tid; i < n2 - 1; i += blockDim.x) {
-    const R v = w.t[i];
-    w.t2[i] = v * v;
-    tmax = fmax(tmax, fabs(v));
-  }
+  for (int i = tid; i < n2 - 1; i += blockDim.x) tmax = fmax(tmax, fabs(w.t[i]));
   tmax = warp_max(tmax);
   if (lane == 0) red[8 + warp] = tmax;
   __syncthreads();
   tmax = R(0);
   for (int i = 0; i < kWarps; ++i) tmax = fmax(tmax, red[8 + i]);
-  __syncthreads();
-  const R bound = R(2) * tmax * (R(1) + R(4) * Eps<R>::eps) + Eps<R>::tiny;
-  const R pivmin = Eps<R>::tiny * R(1024) * fmax(R(1), tmax * tmax);
-  {
-    const int G = K <= 16 ? 16 : 8;
-    const int gid = tid / G, gl = tid % G;
-    const int gbase = (lane / G) * G;
-    const double lg = log((double)(G + 1));
-    // (G+1)^nit >= 2^(bits+2): the final interval is below a quarter ulp of the bound
-    const int nit = (int)((Eps<R>::bits + 2) * 0.6931471805599453 / lg) + 1;
-    const int idx = n2 - 1 - gid;  // ascending index of the (gid+1)-th largest eigenvalue
-    R lo = R(0), hi = bound;
-    for (int it = 0; it < nit; ++it) {
-      const R step = (hi - lo) / R(G + 1);
-      bool pred = true;
-      if (gid < K) {
-        const R x = lo + step * R(gl + 1);
-        pred = sturm_count(w.t2, n2, x, pivmin) <= idx;
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, pred);
-      const unsigned bits = (bal >> gbase) & ((G == 32) ? 0xffffffffu : ((1u << G) - 1u));
-      const int gstar = __popc(bits) - 1;
-      const R nlo = gstar >= 0 ? lo + step * R(gstar + 1) : lo;
-      const R nhi = gstar + 1 < G ? lo + step * R(gstar + 2) : hi;
-      lo = nlo;
-      hi = nhi;
+  if constexpr (sizeof(R) == 4) {
+    // the squares in shared memory (wv is free here) where they fit
+    R* t2 = n2 <= kMaxT2Shared ? w.wv : w.t2;
+    for (int i = tid; i < n2 - 1; i += blockDim.x) t2[i] = w.t[i] * w.t[i];
+    __syncthreads();
+    const R bound = R(2) * tmax * (R(1) + R(4) * Eps<R>::eps) + Eps<R>::tiny;
+    const R pivmin = Eps<R>::tiny * R(1024) * fmax(R(1), tmax * tmax);
+    section_f32(t2, n2, K, bound, pivmin, w.lam);
+  } else {
+    const int e2 = pow2_exponent(tmax);
+    const R down = pow2<R>(-e2);
+    float* t2f = reinterpret_cast<float*>(w.wv);       // >= 512 floats
+    float* lamf = reinterpret_cast<float*>(red + 24);
+    for (int i = tid; i < n2 - 1; i += blockDim.x) {
+      const R v = w.t[i] * down;
+      w.t2[i] = v * v;
+      t2f[i] = (float)(v * v);
     }
-    if (gid < K && gl == 0) w.lam[gid] = R(0.5) * (lo + hi);
+    __syncthreads();
+    section_f32(t2f, n2, K, 4.001f, Eps<float>::tiny * 4096.f, lamf);
+    __syncthreads();
+    if (warp == 0) refine_values_f64(w.t2, n2, K, lamf, pow2<R>(e2), w.lam);
   }
   __syncthreads();
   PEPS_PHASE(2);
   // ---------------- inverse iteration, one thread per vector
   const R pivtiny = Eps<R>::eps * fmax(tmax, Eps<R>::tiny * R(1e10));
-  {
-    // in shared memory (the matrix buffer, free on the register-tiled path,
-    // and the Ub buffer for the interchange bytes) when it fits
-    const bool in_smem = tiled && (size_t)4 * n2 * K <= (size_t)w.Qmax * w.ldw;
-    R* wsR = in_smem ? w.Wm : w.lu;
-    unsigned char* wsP = in_smem ? reinterpret_cast<unsigned char*>(w.Ubs)
-                                 : reinterpret_cast<unsigned char*>(w.lu + (size_t)4 * n2 * K);
-    if (tid < K) inverse_iteration(w.t, n2, w.lam[tid], pivtiny, wsR, wsP, K, tid, w.Z + tid, K, (unsigned)(tid + 1));
-  }
-  __syncthreads();
-  PEPS_PHASE(3);
-  // extract u-parts (odd positions) for a tall matrix, v-parts (even) for a wide one
   R* Ub = w.Ubs;
-  for (int e = tid; e < Q * K; e += blockDim.x) {
-    const int i = e / K, k = e % K;
-    Ub[e] = w.Z[(size_t)(2 * i + (tall ? 1 : 0)) * K + k];
+  {
+    // in shared memory (the matrix buffer, free on the register-tiled path)
+    // when it fits; t in the Ub buffer
+    const bool in_smem = tiled && (size_t)4 * n2 * K <= (size_t)w.Qmax * w.ldw;
+    R* wsR = in_smem ? w.Wm : inv_align(w.lu);
+    const R* tv = w.t;
+    if (n2 <= w.Qmax * w.Kmax) {
+      for (int i = tid; i < n2 - 1; i += blockDim.x) Ub[i] = w.t[i];
+      tv = Ub;
+    }
+    __syncthreads();
+    if (tid < K) red[tid] = inverse_iteration(tv, n2, w.lam[tid], pivtiny, wsR, K, tid, (unsigned)(tid + 1));
+    __syncthreads();
+    PEPS_PHASE(3);
+    // u-parts (odd positions) for a tall matrix, v-parts (even) for a wide one, scaled
+    for (int e = tid; e < Q * K; e += blockDim.x) {
+      const int i = e / K, k = e % K;
+      Ub[e] = wsR[((2 * i + (tall ? 1 : 0)) * K + k) * 4 + 3] * red[k];
+    }
   }
   __syncthreads();
   // ---------------- orthonormal basis of the kept vectors: CholeskyQR2
@@ -1244,6 +1401,7 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
         const int a = e / K, b = e % K;
         if (b < a) continue;
         R sacc = R(0);
+#pragma unroll 8
         for (int i = 0; i < Q; ++i) sacc += Ub[i * K + a] * Ub[i * K + b];
         G[e] = sacc;
       }
@@ -1265,8 +1423,17 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
           __syncwarp();
           if (lane == j) G[j * K + j] = r;
           if (lane > j && lane < K) {
+            // rows in blocks of four, loaded before the block's stores
             const R gjl = G[j * K + lane];
-            for (int mm = j + 1; mm <= lane; ++mm) G[mm * K + lane] -= G[j * K + mm] * gjl;
+            for (int m0 = j + 1; m0 <= lane; m0 += 4) {
+              R x[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (m0 + q <= lane) x[q] = fma(-G[j * K + m0 + q], gjl, G[(m0 + q) * K + lane]);
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (m0 + q <= lane) G[(m0 + q) * K + lane] = x[q];
+            }
           }
           __syncwarp();
         }
@@ -1279,10 +1446,23 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
       }
       // Ub <- Ub R^-1, one thread per row (forward substitution in place)
       for (int i = tid; i < Q; i += blockDim.x) {
-        for (int l = 0; l < K; ++l) {
-          R x = Ub[i * K + l];
-          for (int k = 0; k < l; ++k) x -= Ub[i * K + k] * G[k * K + l];
-          Ub[i * K + l] = x / G[l * K + l];
+        if (K <= 16) {   // the row in registers
+          R u[16];
+#pragma unroll
+          for (int l = 0; l < 16; ++l)
+            if (l < K) {
+              R x = Ub[i * K + l];
+#pragma unroll
+              for (int k = 0; k < l; ++k) x = fma(-u[k], G[k * K + l], x);
+              u[l] = x / G[l * K + l];
+              Ub[i * K + l] = u[l];
+            }
+        } else {
+          for (int l = 0; l < K; ++l) {
+            R x = Ub[i * K + l];
+            for (int k = 0; k < l; ++k) x -= Ub[i * K + k] * G[k * K + l];
+            Ub[i * K + l] = x / G[l * K + l];
+          }
         }
       }
       __syncthreads();
@@ -1389,7 +1569,10 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
         // column of U per half-warp (lane l holds rows l, l + 16, ...), the
         // reflectors applied one at a time, last first.  Each is a dot
         // product over the half-warp (shuffles) and an axpy; columns are
-        // independent, so there is no barrier.
+        // independent, so there is no barrier.  A reflector is zero above its
+        // first row, so the row groups above it are left out (half of the
+        // work): apply_reflectors takes the reflectors whose first row is in
+        // one group of sixteen.
         const int c = warp * 2 + (lane >> 4), l = lane & 15;
         float u[8];
 #pragma unroll
@@ -1397,23 +1580,19 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
           const int i = l + 16 * r;
           u[r] = (c < K && i < rowsU) ? Uk[i * K + c] : 0.f;
         }
-        for (int j = nref - 1; j >= 0; --j) {
-          const int pv = tall ? j : j + 1;
-          const float tj = taus[j], sj = scs[j];
-          float v[8], d = 0.f;
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int i = l + 16 * r;
-            const float wv = (i > pv && i < rowsU) ? (tall ? W[i * ld + j] : W[j * ld + i]) : 0.f;
-            v[r] = i == pv ? 1.f : sj * wv;
-            d = fmaf(v[r], u[r], d);
-          }
-#pragma unroll
-          for (int o = 8; o >= 1; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-          const float cf = -tj * d;
-#pragma unroll
-          for (int r = 0; r < 8; ++r) u[r] = fmaf(cf, v[r], u[r]);
-        }
+        int j = nref - 1;
+        const int off = tall ? 0 : 1;   // first row of reflector j: j + off
+        const float* Wf = reinterpret_cast<const float*>(W);
+        const float* tf = reinterpret_cast<const float*>(taus);
+        const float* sf = reinterpret_cast<const float*>(scs);
+        j = apply_reflectors<7>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<6>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<5>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<4>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<3>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<2>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<1>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        apply_reflectors<0>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
         if (c < K) {
 #pragma unroll
           for (int r = 0; r < 8; ++r) {

@@ -42,8 +42,12 @@ size_t dyn_smem_bytes(const Geometry& g, size_t elem, bool truncates, bool wm_in
   return reals_region_bytes(g, elem, truncates, wm_in_smem) + (size_t)kGemmSmemInts * sizeof(int);
 }
 
+// The truncation matrix goes to shared memory up to 212 KB with its buffers: a
+// block may have 227 KB and the kernels that truncate hold at most 14 KB of
+// static arrays.  D = 10, Dc = 20 in FP32 needs 203 KB; in global memory its
+// Householder columns took 62 kcycles each.
 bool wm_fits_smem(const Geometry& g, size_t elem) {
-  return dyn_smem_bytes(g, elem, true, true) <= 200 * 1024;
+  return dyn_smem_bytes(g, elem, true, true) <= 212 * 1024;
 }
 
 static size_t zip_elems(const Geometry& g, bool wm_in_smem) {

@@ -375,12 +375,12 @@ __device__ void carve_zip(const Geometry& g, R*& p, ZipBufs<R>& zb, R* wm_smem, 
   w.Ubs = sh; sh += P * Dc;
   w.Uks = sh;
   w.Qmax = (int)P;
+  w.Kmax = (int)Dc;
   w.wm_shared = wm_smem != nullptr;
   w.tau = p; p += 4 * P;
   w.t = p; p += 2 * P;
   w.t2 = p; p += 2 * P;
   w.lam = p; p += Dc;
-  w.Z = p; p += Dc * 2 * P;
   w.lu = p; p += Dc * 6 * 2 * P;
   w.Ub = p; p += P * Dc;
   w.Uk = p; p += P * Dc;

@@ -393,17 +393,6 @@ __device__ __noinline__ void bidiag(R* W, int ld, int P, int Q, R* t, R* tau, R*
 // K * 16 points spread over the lanes in NCH chunks so that each lane runs NCH
 // independent Sturm recurrences.  In the first step all values share one
 // interval, so its 16 points are counted once.
-// The quotient t2 / q is t2 times the hardware reciprocal of q, fused with the
-// subtraction; __fdividef's scaling for |q| > 2^126 is not needed, as the clamp
-// keeps |q| >= pivmin >= 2^-116 tmax^2, so |t2 / q| stays below 2^117.
-__device__ __forceinline__ int sturm_count_step(float& q, float x, float t2, float pivmin) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
-  q = __fmaf_rn(-t2, r, -x);
-  if (fabsf(q) < pivmin) q = -pivmin;
-  return (int)(__float_as_uint(q) >> 31);
-}
-
 template <int NCH>
 __device__ __noinline__ void bisect_f32(const float* t2, int n2, int K, float bound, float pivmin, float* lam) {
   constexpr int G = 16, NIT = 7;   // 17^7 >= 2^26
@@ -456,93 +445,6 @@ __device__ __noinline__ void bisect_f32(const float* t2, int n2, int K, float bo
 #pragma unroll
   for (int c = 0; c < NCH; ++c)
     if (gl == 0 && 2 * c + half < K) lam[2 * c + half] = 0.5f * (lo[c] + hi[c]);
-}
-
-// ------------------------------------------------------ inverse iteration
-// inverse_iteration's recurrences (one lane per vector, element i of vector k
-// at i * K + k), with the row interchange taken by selects instead of a
-// branch: lanes that differ no longer run both sides one after the other.
-// FP32 keeps its two approximate divisions per row; FP64 divides once per row
-// (the multiplier is formed from the pivot's reciprocal) and scales the first
-// iterate by a power of two.
-template <typename R>
-__device__ __noinline__ void inverse_iteration_lane(const R* t, int n2, R lam, R pivtiny, R* ws, int K, int k, unsigned seed) {
-  const int st = n2 * K;
-  R* rdd = ws + k;
-  R* du = rdd + st;
-  R* mult = du + st;
-  R* b = mult + st;
-  unsigned long long piv = 0ull;   // n2 <= 64
-  unsigned h = seed * 2654435761u + 12345u;
-  auto start = [&]() {
-    h ^= h << 13; h ^= h >> 17; h ^= h << 5;
-    return R((int)(h & 0xffffu) - 32768) / R(32768) + R(0.001);
-  };
-  R cur_d = -lam, cur_u = t[0];
-  R bi = start();
-#pragma unroll 2
-  for (int i = 0; i < n2 - 1; ++i) {
-    const R sub = t[i];
-    const R nd = -lam, nu = i + 1 < n2 - 1 ? t[i + 1] : R(0);
-    const R bn = start();
-    const bool sw = !(fabs(cur_d) >= fabs(sub));
-    R d = sw ? sub : (cur_d == R(0) ? pivtiny : cur_d);
-    const R num = sw ? cur_d : sub;
-    R lm, rd;
-    if constexpr (sizeof(R) == 4) {
-      lm = __fdividef(num, d);
-      if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
-      rd = __fdividef(1.f, d);
-    } else {
-      if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
-      rd = R(1) / d;
-      lm = num * rd;
-    }
-    const R u = sw ? nd : cur_u, y = sw ? cur_u : nd;
-    const R bs = sw ? bn : bi, bo = sw ? bi : bn;
-    rdd[i * K] = rd;
-    du[i * K] = u;
-    mult[i * K] = lm;
-    b[i * K] = bs;
-    if (sw) piv |= 1ull << i;
-    cur_d = fma(-lm, u, y);
-    cur_u = sw ? -lm * nu : nu;
-    bi = fma(-lm, bs, bo);
-  }
-  if (fabs(cur_d) < pivtiny) cur_d = cur_d < R(0) ? -pivtiny : pivtiny;
-  rdd[(n2 - 1) * K] = sturm_div(R(1), cur_d);
-  du[(n2 - 1) * K] = R(0);
-  b[(n2 - 1) * K] = bi;
-  R sc = R(1);
-#pragma unroll 1
-  for (int it = 0; it < 2; ++it) {
-    if (it == 1) {
-      R bf = b[0] * sc;
-#pragma unroll 4
-      for (int i = 0; i < n2 - 1; ++i) {
-        const R bn = b[(i + 1) * K] * sc;
-        const R lm = mult[i * K];
-        const bool sw = (piv >> i) & 1ull;
-        const R bs = sw ? bn : bf, bo = sw ? bf : bn;
-        b[i * K] = bs;
-        bf = fma(-lm, bs, bo);
-      }
-      b[(n2 - 1) * K] = bf;
-    }
-    R y1 = R(0), y2 = R(0), mx = R(0);
-#pragma unroll 4
-    for (int i = n2 - 1; i >= 0; --i) {
-      const R du2 = (((piv >> i) & 1ull) && i + 1 < n2 - 1) ? t[i + 1] : R(0);
-      const R y = fma(-du2, y2, fma(-du[i * K], y1, b[i * K])) * rdd[i * K];
-      b[i * K] = y;
-      mx = fmax(mx, fabs(y));
-      y2 = y1;
-      y1 = y;
-    }
-    if constexpr (sizeof(R) == 4) sc = mx > R(0) ? R(1) / mx : R(1);
-    else sc = pow2<R>(-pow2_exponent(mx));
-  }
-  for (int i = 0; i < n2; ++i) b[i * K] = b[i * K] * sc;
 }
 
 // ------------------------------------------------------------- truncation
@@ -929,13 +831,13 @@ __device__ __noinline__ void topk_left(R* sm, const Layout& L, int m, int n, int
   const R tmax = values(t, sm + L.t2, Q, K, lam, ws);
   PEPS_PHASE(2);
   const R pivtiny = Eps<R>::eps * fmax(tmax, Eps<R>::tiny * R(1e10));
-  if (l < K) inverse_iteration_lane(t, n2, lam[l], pivtiny, ws, K, l, (unsigned)(l + 1));
+  const R sc = l < K ? inverse_iteration(t, n2, lam[l], pivtiny, ws, K, l, (unsigned)(l + 1)) : R(0);
+  if (l < K) sm[L.va + l] = sc;
   __syncwarp();
   PEPS_PHASE(3);
   R* Ub = sm + L.Ub;
   R* Uk = sm + L.Uk;
-  const R* Z = ws + 3 * n2 * K;
-  for (int e = l; e < Q * K; e += 32) Ub[e] = Z[(2 * (e / K) + (tall ? 1 : 0)) * K + e % K];
+  for (int e = l; e < Q * K; e += 32) Ub[e] = ws[((2 * (e / K) + (tall ? 1 : 0)) * K + e % K) * 4 + 3] * sm[L.va + e % K];
   __syncwarp();
   orthonormalise(Ub, Uk, Q, K);
   PEPS_PHASE(4);
