@@ -575,6 +575,15 @@ peps_status run_graphed(peps_ctx* c, int op, const void* S, int n, const void* c
   c->capturing = true;
   peps_status st = enqueue();
   c->capturing = false;
+  if (small_boundary(c)) {
+    a.slot_elems = (mc_small_slot_elems(c->g) + 31) / 32 * 32;
+    // as many chains side by side as are resident and have a slot (a CTA's slot holds two or three)
+    const int slots = (int)std::min<size_t>(scratch_bytes(c, c->nslots) / c->elem / a.slot_elems, 1u << 20);
+    const int grid = std::max(1, std::min(n, std::min(slots, max_blocks_mc_small<R>(c->g))));
+    Prof pf(c, 7);
+    PEPS_CUDA(launch_mc_small<R>(a, S, nsweeps, seed, chain0, sweep0, (long long*)accepted, grid, c->stream));
+    return PEPS_OK;
+  }
   cudaError_t e = cudaStreamEndCapture(c->stream, &graph);
   if (st != PEPS_OK) {
     if (graph) cudaGraphDestroy(graph);
@@ -776,8 +785,9 @@ peps_status correlations_impl(peps_ctx* c, const uint64_t* S, int n, const int* 
   PEPS_CUDA(c->corr_sites.ensure(tab.size() * sizeof(int)));
   PEPS_CUDA(cudaMemcpyAsync(c->corr_sites.p, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   PEPS_CUDA(c->corr_x.ensure((size_t)c->chunk * sizeof(double)));
-  const int res = max_blocks_corr<R>(g);
-  const size_t slot = (corr_slot_elems(g, c->wm_smem) + 31) / 32 * 32;
+  const bool one_warp = small_boundary(c);
+  const int res = one_warp ? max_blocks_corr_small<R>(g) : max_blocks_corr<R>(g);
+  const size_t slot = ((one_warp ? corr_small_slot_elems(g) : corr_slot_elems(g, c->wm_smem)) + 31) / 32 * 32;
   PEPS_CUDA(c->corr_scratch.ensure(slot * c->elem * res));
   if (corr) PEPS_CUDA(cudaMemsetAsync(corr, 0, (size_t)nc * nc * sizeof(double), c->stream));
   CorrArgs ca;
@@ -799,7 +809,8 @@ peps_status correlations_impl(peps_ctx* c, const uint64_t* S, int n, const int* 
     ca.status = sm.status;
     PEPS_CUDA(cudaMemsetAsync(ca.xsum, 0, (size_t)m * sizeof(double), c->stream));
     const int grid = std::max(1, std::min(m * nc, res));
-    PEPS_CUDA(launch_corr<R>(a, ca, grid, c->stream));
+    if (one_warp) PEPS_CUDA(launch_corr_small<R>(a, ca, grid, c->stream));
+    else PEPS_CUDA(launch_corr<R>(a, ca, grid, c->stream));
     PEPS_CUDA(launch_corr_finalize(g, ca, Sc, m, sm.status, m2 ? m2 + c0 : nullptr, c->stream));
     if (status) PEPS_CUDA(cudaMemcpyAsync(status + c0, sm.status, m * 4, cudaMemcpyDeviceToDevice, c->stream));
   }

@@ -17,7 +17,7 @@
 // difference of the per-row log norms of the two sweeps above row r.
 #include <algorithm>
 
-#include "kernels_common.cuh"
+#include "small_ops.cuh"
 
 namespace peps {
 
@@ -29,34 +29,20 @@ size_t corr_slot_elems(const Geometry& g, bool wm_in_smem) {
          2 * tmp_elems(g) + 64;
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_corr(KArgs<R> a, CorrArgs c) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ R red[64];
-  __shared__ uint64_t sp[kMaxWords];
-  __shared__ int ones[kMaxDcD + 1];
-  __shared__ double dred[kWarps];
-  __shared__ R wv[kMaxDcD];
-  __shared__ int eG[kMaxL + 1];   // G_col is stored scaled by 2^-eG[col]
+template <typename R, class Ops>
+__device__ void corr_items(const KArgs<R>& a, const CorrArgs& c, Ops& ops, R* p, uint64_t* sp, int* ones, int* eG) {
+  // G_col is stored scaled by 2^-eG[col]
   const Geometry& g = a.g;
   const int Lx = g.Lx, Ly = g.Ly, Dc = g.Dc, D = g.D;
   const size_t envT = (size_t)Dc * D * Dc;
   const int D4 = D * D * D * D;
-  R* p = a.scratch + (size_t)blockIdx.x * c.slot_elems;
-  ZipBufs<R> zb;
-  R* gsm;
-  int* gism;
-  smem_split<R>(smem_raw, g, true, a.smem_wm != 0, gsm, gism);
-  carve_zip<R>(g, p, zb, a.smem_wm ? gsm : nullptr, red, dred, wv, gsm, gism);
   R* Mbuf[2];
   Mbuf[0] = p; p += (size_t)Lx * envT;
   Mbuf[1] = p; p += (size_t)Lx * envT;
   R* Gb = p; p += (size_t)(Lx + 1) * envT;
   R* F0 = p; p += envT;
   R* F1 = p; p += envT;
-  R* Bb = p; p += D4;
-  R* t0 = p; p += tmp_elems(g);
-  R* t1 = p;
+  R* Bb = p;
   for (int k = threadIdx.x; k <= Lx; k += blockDim.x) ones[k] = 1;
   for (int item = blockIdx.x; item < a.n * c.nc; item += gridDim.x) {
     const int cfg = item / c.nc, pi = item % c.nc;
@@ -85,10 +71,9 @@ __global__ void __launch_bounds__(kThreads) k_corr(KArgs<R> a, CorrArgs c) {
       int eacc = 0;
       for (int col = Lx - 1; col >= 0; --col) {
         const int site = r * Lx + col;
-        run_op<R>(OP_COL1_RIGHT, D, Dc, Gb + (size_t)(col + 1) * envT, Mu + (size_t)col * envT,
-                  tptr(a, site, spin_of(sp, site)), Md + (size_t)col * envT, nullptr, Gb + (size_t)col * envT, t0,
-                  t1, gsm, gism);
-        eacc += normalize_pow2(Gb + (size_t)col * envT, (int)envT, red);
+        ops.col1(true, Gb + (size_t)(col + 1) * envT, Mu + (size_t)col * envT,
+                  tptr(a, site, spin_of(sp, site)), Md + (size_t)col * envT, Gb + (size_t)col * envT);
+        eacc += ops.normalize(Gb + (size_t)col * envT, (int)envT);
         if (threadIdx.x == 0) eG[col] = eacc;
       }
       __syncthreads();
@@ -100,9 +85,9 @@ __global__ void __launch_bounds__(kThreads) k_corr(KArgs<R> a, CorrArgs c) {
         const int sj = spin_of(sp, j);            // unchanged for j != i
         const int pj = c.pos[j];
         if (pj >= 0 && j > i && sj != si) {
-          run_op<R>(OP_SITE_ENV, D, Dc, F, Mu + (size_t)col * envT, Md + (size_t)col * envT,
-                    Gb + (size_t)(col + 1) * envT, nullptr, Bb, t0, t1, gsm, gism);
-          const R w = block_dot(Bb, tptr(a, j, 1 - sj), D4, red);
+          ops.site_env(F, Mu + (size_t)col * envT, Md + (size_t)col * envT,
+                    Gb + (size_t)(col + 1) * envT, Bb);
+          const R w = ops.dot(Bb, tptr(a, j, 1 - sj), D4);
           const double ratio = (Wr != 0.0 && lsdiff > -INFINITY)
                                    ? ldexp((double)w, eF + eG[col + 1]) / Wr * exp(lsdiff)
                                    : 0.0;
@@ -114,22 +99,79 @@ __global__ void __launch_bounds__(kThreads) k_corr(KArgs<R> a, CorrArgs c) {
           }
         }
         if (col < Lx - 1) {
-          run_op<R>(OP_COL1_LEFT, D, Dc, F, Mu + (size_t)col * envT, tptr(a, j, sj), Md + (size_t)col * envT,
-                    nullptr, Fn, t0, t1, gsm, gism);
-          eF += normalize_pow2(Fn, (int)envT, red);
+          ops.col1(false, F, Mu + (size_t)col * envT, tptr(a, j, sj), Md + (size_t)col * envT, Fn);
+          eF += ops.normalize(Fn, (int)envT);
           F = Fn;
           Fn = (Fn == F0) ? F1 : F0;
         }
       }
       if (r < Ly - 1) {
         const int* bdin = r == 0 ? ones : a.bd + (size_t)(r - 1) * (Lx + 1);
-        const double nrm = absorb_row<R>(a, Mbuf[cur], Mbuf[cur ^ 1], r, 0, (r % 2) == 0, bdin, sp, zb, red);
+        const double nrm = ops.absorb(Mbuf[cur], Mbuf[cur ^ 1], r, 0, (r % 2) == 0, bdin, sp);
         lsdiff += (nrm > 0.0 ? log(nrm) : -INFINITY) - a.lnU[(size_t)cfg * Ly + r];
         cur ^= 1;
       }
     }
     if (threadIdx.x == 0 && xs != 0.0) atomicAdd(&c.xsum[cfg], xs);
   }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kThreads) k_corr(KArgs<R> a, CorrArgs c) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ R red[64];
+  __shared__ uint64_t sp[kMaxWords];
+  __shared__ int ones[kMaxDcD + 1];
+  __shared__ double dred[kWarps];
+  __shared__ R wv[kMaxDcD];
+  __shared__ int eG[kMaxL + 1];
+  const Geometry& g = a.g;
+  CtaOps<R> ops(a, red);
+  R* gsm;
+  int* gism;
+  smem_split<R>(smem_raw, g, true, a.smem_wm != 0, gsm, gism);
+  R* p = a.scratch + (size_t)blockIdx.x * c.slot_elems;
+  carve_zip<R>(g, p, ops.zb, a.smem_wm ? gsm : nullptr, red, dred, wv, gsm, gism);
+  ops.t0 = p; p += tmp_elems(g);
+  ops.t1 = p; p += tmp_elems(g);
+  corr_items<R>(a, c, ops, p, sp, ones, eG);
+}
+
+// One warp per (configuration, first site), for the models small.cuh takes.
+// 6x6 D = 3 Dc = 6 FP64, 128 configurations, 16 sites: 15 ms against 220.
+template <typename R>
+__global__ void __launch_bounds__(32) k_corr_small(KArgs<R> a, CorrArgs c) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t sp[kMaxWords];
+  __shared__ int ones[kMaxL + 1];
+  __shared__ int eG[kMaxL + 1];
+  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw));
+  corr_items<R>(a, c, ops, a.scratch + (size_t)blockIdx.x * c.slot_elems, sp, ones, eG);
+}
+
+size_t corr_small_slot_elems(const Geometry& g) {
+  const size_t envT = (size_t)g.Dc * g.D * g.Dc;
+  return 2 * (size_t)g.Lx * envT + (size_t)(g.Lx + 3) * envT + (size_t)g.D * g.D * g.D * g.D;
+}
+
+template <typename R>
+int max_blocks_corr_small(const Geometry& g) {
+  int dev = 0, nsm = 0, nb = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem = (size_t)small::ops_total(g.D, g.Dc) * sizeof(R);
+  prefer_shared(k_corr_small<R>, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_corr_small<R>, 32, smem);
+  return nsm * (nb < 1 ? 1 : nb);
+}
+
+template <typename R>
+cudaError_t launch_corr_small(const KArgs<R>& a, const CorrArgs& c, int grid, cudaStream_t st) {
+  const size_t smem = (size_t)small::ops_total(a.g.D, a.g.Dc) * sizeof(R);
+  cudaError_t e = prefer_shared(k_corr_small<R>, smem);
+  if (e != cudaSuccess) return e;
+  k_corr_small<R><<<grid, 32, smem, st>>>(a, c);
+  return cudaGetLastError();
 }
 
 // M^2 per configuration: (1/n^2) [n/2 + (sum_p eps_p S^z_p)^2 + xsum] over the
@@ -210,6 +252,8 @@ cudaError_t launch_corr_finalize(const Geometry& g, const CorrArgs& c, const uin
 }
 
 #define PEPS_INST(R)                                                                                    \
+  template int max_blocks_corr_small<R>(const Geometry&);                                               \
+  template cudaError_t launch_corr_small<R>(const KArgs<R>&, const CorrArgs&, int, cudaStream_t);       \
   template int max_blocks_corr<R>(const Geometry&);                                                     \
   template cudaError_t launch_corr<R>(const KArgs<R>&, const CorrArgs&, int, cudaStream_t);
 PEPS_INST(double)

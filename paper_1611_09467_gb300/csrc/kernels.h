@@ -96,6 +96,20 @@ template <typename R> cudaError_t launch_boundary_packed(const KArgs<R>* models_
                                                          int grid, cudaStream_t st);
 size_t dyn_smem_bytes(const Geometry& g, size_t elem, bool truncates, bool wm_in_smem);
 template <typename R> int max_blocks_mc(const Geometry& g);
+// Sandwiches with one warp per item, for the models boundary_small_fits accepts.
+bool row_has_fused(const Geometry& g);
+size_t row_small_slot_elems(const Geometry& g);
+size_t pair_small_slot_elems(const Geometry& g);
+template <typename R> int max_blocks_row_small(const Geometry& g);
+template <typename R> int max_blocks_pair_small(const Geometry& g);
+template <typename R> cudaError_t launch_row_small(const KArgs<R>& a, int grid, cudaStream_t st);
+template <typename R> cudaError_t launch_pair_small(const KArgs<R>& a, int grid, cudaStream_t st);
+// Metropolis chains with one warp each, for the models boundary_small_fits accepts.
+size_t mc_small_slot_elems(const Geometry& g);
+template <typename R> int max_blocks_mc_small(const Geometry& g);
+template <typename R> cudaError_t launch_mc_small(const KArgs<R>& a, uint64_t* S, int nsweeps, uint64_t seed,
+                                                  uint64_t chain0, uint64_t sweep0, long long* accepted, int grid,
+                                                  cudaStream_t st);
 template <typename R> int max_blocks_row(const Geometry& g, int generic = 0);
 template <typename R> int max_blocks_pair(const Geometry& g);
 template <typename R> int max_blocks_pair_fused(const Geometry& g);   // 0: no fused step for (D, Dc)
@@ -114,6 +128,10 @@ struct CorrArgs {
 size_t corr_slot_elems(const Geometry& g, bool wm_in_smem);
 template <typename R> int max_blocks_corr(const Geometry& g);
 template <typename R> cudaError_t launch_corr(const KArgs<R>& a, const CorrArgs& c, int grid, cudaStream_t st);
+// The same with one warp per item, for the models boundary_small_fits accepts.
+size_t corr_small_slot_elems(const Geometry& g);
+template <typename R> int max_blocks_corr_small(const Geometry& g);
+template <typename R> cudaError_t launch_corr_small(const KArgs<R>& a, const CorrArgs& c, int grid, cudaStream_t st);
 // M^2 per configuration and the S^z S^z part of the correlation sums.
 cudaError_t launch_corr_finalize(const Geometry& g, const CorrArgs& c, const uint64_t* S, int n, const int* status,
                                  double* m2, cudaStream_t st);
