@@ -114,7 +114,9 @@ struct peps_ctx {
   peps_ctx* parent = nullptr;                        // set on clones (model buffers borrowed)
   DevBuf env, small, O, scratch, gsum, go;
   int chunk = 0;  // configurations per pass
-  int res_small = 0;   // resident CTAs of the one-warp boundary sweeps (0: the model is too large for them)
+  // resident CTAs of the one-warp kernels (0: the model is too large for them,
+  // or another kernel is the better one for it)
+  int res_small = 0, res_row_small = 0, res_pair_small = 0;
   int res_boundary = 0, res_row = 0, res_pair = 0, res_mc = 0;  // resident CTAs per kernel
   bool pair_tc = false;  // two-row step on the tensor cores (PEPS_MIXED_TF32, D = 8, Dc = 16)
   // kernel variants (peps_autotune): row_generic 1 takes the generic single-row
@@ -338,23 +340,54 @@ KArgs<R> make_args(peps_ctx* c, const uint64_t* S, int n, const Small& sm) {
 template <typename R>
 peps_status sandwich_chunk(peps_ctx* c, const KArgs<R>& a, const uint64_t* S, int n, bool need_env_l,
                            bool need_pairs, Small& sm, cudaStream_t st) {
-  int grid;
+  // One-warp kernels: as many items side by side as are resident and have a slot.
+  // A warp takes two to four times as long as a CTA on one item (8x8 FP32 two-row
+  // D = 5 Dc = 6: 6.8 against 2.4 ms a wave; FP64 D = 4 Dc = 8: 13 against 8.5) but
+  // four times as many run side by side, so they are the better ones from a few
+  // items per SM on (at 152 configurations 7.6 against 9.8 ms and 15 against 29
+  // ms).  Two-row transfers of up to 400 entries are faster on a warp at any
+  // number (FP64 D = 3 Dc = 6, one configuration: 3.5 against 9.7 ms), and so are
+  // single-row ones but for FP64 D = 4 Dc = 8, whose fused kernel is ahead up to
+  // two items per SM (1.8 against 2.3 ms; 3.4 against 2.3 above).
+  const Geometry& g = c->g;
+  const bool warps = small_boundary(c);
+  const bool tiny = g.Dc * g.Dc * g.D * g.D <= 400;
+  const bool row_warps = warps && c->res_row_small && !c->row_generic &&
+                         (tiny || !row_has_fused(g) || n * g.Ly > 2 * c->nsm);
+  const bool pair_warps = warps && c->res_pair_small && c->pair_mode == 0 &&
+                          (tiny || n * (g.Ly - 1) >= (c->elem == 8 ? 3 : 6) * c->nsm);
+  auto warp_grid = [&](KArgs<R>& b, size_t slot, int items, int res) {
+    b.slot_elems = (slot + 31) / 32 * 32;
+    const size_t slots = scratch_bytes(c, c->nslots) / c->elem / b.slot_elems;
+    return (int)std::max<size_t>(1, std::min<size_t>(slots, std::min(items, res)));
+  };
   if (need_env_l) {
-    grid = std::min(n * c->g.Ly, std::min(c->nslots, c->res_row));
+    const int items = n * c->g.Ly;
     Prof pf(c, 1);
-    PEPS_CUDA(launch_row<R>(a, std::max(grid, 1), st, c->row_generic));
+    if (row_warps) {
+      KArgs<R> b = a;
+      const int grid = warp_grid(b, row_small_slot_elems(c->g), items, c->res_row_small);
+      PEPS_CUDA(launch_row_small<R>(b, grid, st));
+    } else {
+      const int grid = std::min(items, std::min(c->nslots, c->res_row));
+      PEPS_CUDA(launch_row<R>(a, std::max(grid, 1), st, c->row_generic));
+    }
   }
   if (need_pairs && c->g.Ly > 1) {
-    grid = std::min(n * (c->g.Ly - 1), std::min(c->nslots, c->res_pair));
+    const int items = n * (c->g.Ly - 1);
+    const int grid = std::max(1, std::min(items, std::min(c->nslots, c->res_pair)));
     Prof pf(c, 2);
+    bool tc = false;
     if constexpr (sizeof(R) == 4) {
-      if (c->pair_tc && c->pair_mode == 0) {
-        PEPS_CUDA(launch_pair_tc(a, std::max(grid, 1), st));
-      } else {
-        PEPS_CUDA(launch_pair<R>(a, std::max(grid, 1), st, c->pair_mode == 2));
-      }
-    } else {
-      PEPS_CUDA(launch_pair<R>(a, std::max(grid, 1), st, c->pair_mode == 2));
+      tc = c->pair_tc && c->pair_mode == 0;
+      if (tc) PEPS_CUDA(launch_pair_tc(a, grid, st));
+    }
+    if (!tc && pair_warps) {
+      KArgs<R> b = a;
+      const int wgrid = warp_grid(b, pair_small_slot_elems(c->g), items, c->res_pair_small);
+      PEPS_CUDA(launch_pair_small<R>(b, wgrid, st));
+    } else if (!tc) {
+      PEPS_CUDA(launch_pair<R>(a, grid, st, c->pair_mode == 2));
     }
   } else {
     PEPS_CUDA(cudaMemsetAsync(sm.eloc_v, 0, (size_t)n * c->g.Ly * sizeof(double), st));
@@ -542,6 +575,15 @@ peps_status mc_impl(peps_ctx* c, uint64_t* S, int n, int nsweeps, uint64_t seed,
   Small sm;
   sm.carve(c->small.p, c->chunk, c->g.Ly);
   KArgs<R> a = make_args<R>(c, S, n, sm);
+  if (small_boundary(c)) {
+    a.slot_elems = (mc_small_slot_elems(c->g) + 31) / 32 * 32;
+    // as many chains side by side as are resident and have a slot (a CTA's slot holds two or three)
+    const int slots = (int)std::min<size_t>(scratch_bytes(c, c->nslots) / c->elem / a.slot_elems, 1u << 20);
+    const int grid = std::max(1, std::min(n, std::min(slots, max_blocks_mc_small<R>(c->g))));
+    Prof pf(c, 7);
+    PEPS_CUDA(launch_mc_small<R>(a, S, nsweeps, seed, chain0, sweep0, (long long*)accepted, grid, c->stream));
+    return PEPS_OK;
+  }
   const int grid = std::min(n, std::min(c->nslots, c->res_mc));
   Prof pf(c, 7);
   PEPS_CUDA(launch_mc<R>(a, S, nsweeps, seed, chain0, sweep0, (long long*)accepted, std::max(grid, 1), c->stream));
@@ -575,15 +617,6 @@ peps_status run_graphed(peps_ctx* c, int op, const void* S, int n, const void* c
   c->capturing = true;
   peps_status st = enqueue();
   c->capturing = false;
-  if (small_boundary(c)) {
-    a.slot_elems = (mc_small_slot_elems(c->g) + 31) / 32 * 32;
-    // as many chains side by side as are resident and have a slot (a CTA's slot holds two or three)
-    const int slots = (int)std::min<size_t>(scratch_bytes(c, c->nslots) / c->elem / a.slot_elems, 1u << 20);
-    const int grid = std::max(1, std::min(n, std::min(slots, max_blocks_mc_small<R>(c->g))));
-    Prof pf(c, 7);
-    PEPS_CUDA(launch_mc_small<R>(a, S, nsweeps, seed, chain0, sweep0, (long long*)accepted, grid, c->stream));
-    return PEPS_OK;
-  }
   cudaError_t e = cudaStreamEndCapture(c->stream, &graph);
   if (st != PEPS_OK) {
     if (graph) cudaGraphDestroy(graph);
@@ -835,7 +868,9 @@ peps_ctx* ctx_clone(peps_ctx* c, cudaStream_t stream, double workspace_gb, int s
   k->wm_smem = c->wm_smem;
   // a worker that shares the GPU with `share` lanes sizes its persistent grids to its part
   auto part = [&](int r) { return std::max(std::min(r, c->nsm), r / std::max(share, 1)); };
-  k->res_small = part(c->res_small);
+  k->res_small = c->res_small ? part(c->res_small) : 0;
+  k->res_row_small = c->res_row_small ? part(c->res_row_small) : 0;
+  k->res_pair_small = c->res_pair_small ? part(c->res_pair_small) : 0;
   k->res_boundary = part(c->res_boundary);
   k->res_row = part(c->res_row);
   k->res_pair = part(c->res_pair);
@@ -945,6 +980,14 @@ peps_status peps_create(const peps_params* p, const double* A_host, void* stream
     const size_t smem = boundary_small_smem(c->g, c->elem);
     c->res_small = c->elem == 8 ? max_blocks_boundary_small<double>(smem)
                                 : max_blocks_boundary_small<float>(smem);
+    // sandwiches: always in FP64; in FP32 where there is no fused kernel
+    if (c->elem == 8) {
+      c->res_row_small = max_blocks_row_small<double>(c->g);
+      c->res_pair_small = max_blocks_pair_small<double>(c->g);
+    } else {
+      if (!row_has_fused(c->g)) c->res_row_small = max_blocks_row_small<float>(c->g);
+      if (!max_blocks_pair_fused<float>(c->g)) c->res_pair_small = max_blocks_pair_small<float>(c->g);
+    }
   }
   if (c->elem == 8) {
     c->res_boundary = max_blocks_boundary<double>(c->g);

@@ -2,32 +2,23 @@
 // of vertical and diagonal exchanges.  One CTA per (configuration, row pair):
 // k_pair (generic), k_pair_fused (shared-memory slices, fixed D and Dc) and
 // k_pair_tc (tcgen05 tensor cores, TF32, D = 8, Dc = 16).
-#include "kernels_common.cuh"
+#include "small_ops.cuh"
 
 namespace peps {
 
 // ---------------------------------------------------------------- k_pair
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
-  extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ R red[64];
-  __shared__ uint64_t sp[kMaxWords];
+template <typename R, class Ops>
+__device__ void pair_items(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int* eH) {
   const Geometry& g = a.g;
   const int Lx = g.Lx, Ly = g.Ly, Dc = g.Dc, D = g.D;
   const int envT = Dc * D * Dc, envT2 = Dc * D * D * Dc;
-  R* gsm;
-  int* gism;
-  smem_split<R>(smem_raw, g, false, false, gsm, gism);
-  R* p = a.scratch + (size_t)blockIdx.x * a.slot_elems;
   R* Hb = p; p += (size_t)(Lx + 1) * envT2;
   R* E0 = p; p += envT2;
   R* E1 = p; p += envT2;
   R* X1 = p; p += envT2;
-  R* X2 = p; p += envT2;
-  R* t0 = p; p += tmp_elems(g);
-  R* t1 = p;
+  R* X2 = p;
   const int npairs = Ly - 1;
-  __shared__ int eH[kMaxL + 1];   // H_c is stored scaled by 2^-eH[c]
+  // H_c is stored scaled by 2^-eH[c]
   for (int item = blockIdx.x; item < a.n * npairs; item += gridDim.x) {
     const int cfg = item / npairs, r = item % npairs;
     __syncthreads();
@@ -40,10 +31,10 @@ __global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
     int eacc = 0;
     for (int c = Lx - 1; c >= 0; --c) {
       const int s1 = r * Lx + c, s2 = (r + 1) * Lx + c;
-      run_op<R>(OP_COL2_RIGHT, D, Dc, Hb + (size_t)(c + 1) * envT2, Mu + (size_t)c * envT,
+      ops.col2(true, Hb + (size_t)(c + 1) * envT2, Mu + (size_t)c * envT,
                 tptr(a, s1, spin_of(sp, s1)), tptr(a, s2, spin_of(sp, s2)), Md + (size_t)c * envT,
-                Hb + (size_t)c * envT2, t0, t1, gsm, gism);
-      eacc += normalize_pow2(Hb + (size_t)c * envT2, envT2, red);
+                Hb + (size_t)c * envT2);
+      eacc += ops.normalize(Hb + (size_t)c * envT2, envT2);
       if (threadIdx.x == 0) eH[c] = eacc;
     }
     const R W = Hb[0];
@@ -58,8 +49,8 @@ __global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
       const R* Muc = Mu + (size_t)c * envT;
       const R* Mdc = Md + (size_t)c * envT;
       if (a1 != a2) {  // vertical pair (r,c)-(r+1,c)
-        run_op<R>(OP_COL2_LEFT, D, Dc, E, Muc, tptr(a, i1, a2), tptr(a, i2, a1), Mdc, X1, t0, t1, gsm, gism);
-        const R wp = block_dot(X1, Hb + (size_t)(c + 1) * envT2, envT2, red);
+        ops.col2(false, E, Muc, tptr(a, i1, a2), tptr(a, i2, a1), Mdc, X1);
+        const R wp = ops.dot(X1, Hb + (size_t)(c + 1) * envT2, envT2);
         if (ok) ev += 0.5 * g.J1 * ldexp((double)wp / (double)W, eE + eH[c + 1] - eH[0]);
       }
       if (c < Lx - 1 && g.J2 != 0.0) {
@@ -68,23 +59,23 @@ __global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
         const R* Mun = Mu + (size_t)(c + 1) * envT;
         const R* Mdn = Md + (size_t)(c + 1) * envT;
         if (a1 != b2) {  // diagonal (r,c)-(r+1,c+1)
-          run_op<R>(OP_COL2_LEFT, D, Dc, E, Muc, tptr(a, i1, b2), tptr(a, i2, a2), Mdc, X1, t0, t1, gsm, gism);
-          const int eX = normalize_pow2(X1, envT2, red);
-          run_op<R>(OP_COL2_LEFT, D, Dc, X1, Mun, tptr(a, j1, b1), tptr(a, j2, a1), Mdn, X2, t0, t1, gsm, gism);
-          const R wp = block_dot(X2, Hb + (size_t)(c + 2) * envT2, envT2, red);
+          ops.col2(false, E, Muc, tptr(a, i1, b2), tptr(a, i2, a2), Mdc, X1);
+          const int eX = ops.normalize(X1, envT2);
+          ops.col2(false, X1, Mun, tptr(a, j1, b1), tptr(a, j2, a1), Mdn, X2);
+          const R wp = ops.dot(X2, Hb + (size_t)(c + 2) * envT2, envT2);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
         if (b1 != a2) {  // anti-diagonal (r,c+1)-(r+1,c)
-          run_op<R>(OP_COL2_LEFT, D, Dc, E, Muc, tptr(a, i1, a1), tptr(a, i2, b1), Mdc, X1, t0, t1, gsm, gism);
-          const int eX = normalize_pow2(X1, envT2, red);
-          run_op<R>(OP_COL2_LEFT, D, Dc, X1, Mun, tptr(a, j1, a2), tptr(a, j2, b2), Mdn, X2, t0, t1, gsm, gism);
-          const R wp = block_dot(X2, Hb + (size_t)(c + 2) * envT2, envT2, red);
+          ops.col2(false, E, Muc, tptr(a, i1, a1), tptr(a, i2, b1), Mdc, X1);
+          const int eX = ops.normalize(X1, envT2);
+          ops.col2(false, X1, Mun, tptr(a, j1, a2), tptr(a, j2, b2), Mdn, X2);
+          const R wp = ops.dot(X2, Hb + (size_t)(c + 2) * envT2, envT2);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
       }
       if (c < Lx - 1) {
-        run_op<R>(OP_COL2_LEFT, D, Dc, E, Muc, tptr(a, i1, a1), tptr(a, i2, a2), Mdc, En, t0, t1, gsm, gism);
-        eE += normalize_pow2(En, envT2, red);
+        ops.col2(false, E, Muc, tptr(a, i1, a1), tptr(a, i2, a2), Mdc, En);
+        eE += ops.normalize(En, envT2);
         E = En;
         En = (En == E0) ? E1 : E0;
       }
@@ -94,6 +85,55 @@ __global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
       if (!ok) atomicOr(&a.flags[cfg], kFlagZeroW);
     }
   }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ R red[64];
+  __shared__ uint64_t sp[kMaxWords];
+  __shared__ int eH[kMaxL + 1];
+  CtaOps<R> ops(a, red);
+  smem_split<R>(smem_raw, a.g, false, false, ops.zb.gsm, ops.zb.gism);
+  R* p = a.scratch + (size_t)blockIdx.x * a.slot_elems;
+  ops.t0 = p; p += tmp_elems(a.g);
+  ops.t1 = p; p += tmp_elems(a.g);
+  pair_items<R>(a, ops, p, sp, eH);
+}
+
+// One warp per (configuration, row pair), for the models small.cuh takes.
+// 4x4 D = 2 Dc = 4 FP64, 64 configurations: 0.33 ms against 0.65 with
+// k_pair_fused (barriers around products of 64 outputs); 8x8 D = 4 Dc = 8 FP64,
+// 304 configurations: 29 against 49 ms.
+template <typename R>
+__global__ void __launch_bounds__(32) k_pair_small(KArgs<R> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t sp[kMaxWords];
+  __shared__ int eH[kMaxL + 1];
+  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw));
+  pair_items<R>(a, ops, a.scratch + (size_t)blockIdx.x * a.slot_elems, sp, eH);
+}
+
+size_t pair_small_slot_elems(const Geometry& g) { return (size_t)(g.Lx + 5) * g.Dc * g.D * g.D * g.Dc; }
+
+template <typename R>
+int max_blocks_pair_small(const Geometry& g) {
+  int dev = 0, nsm = 0, nb = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem = (size_t)small::ops_reals(g.D, g.Dc) * sizeof(R);
+  prefer_shared(k_pair_small<R>, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pair_small<R>, 32, smem);
+  return nsm * (nb < 1 ? 1 : nb);
+}
+
+template <typename R>
+cudaError_t launch_pair_small(const KArgs<R>& a, int grid, cudaStream_t st) {
+  const size_t smem = (size_t)small::ops_reals(a.g.D, a.g.Dc) * sizeof(R);
+  cudaError_t e = prefer_shared(k_pair_small<R>, smem);
+  if (e != cudaSuccess) return e;
+  k_pair_small<R><<<grid, 32, smem, st>>>(a);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ k_pair_fused
@@ -353,7 +393,7 @@ template <typename R>
 static int pair_fused_id(const Geometry& g) {
   if (g.D == 2 && g.Dc == 4) return 1;
   if (g.D == 4 && g.Dc == 8) return 2;
-  if (sizeof(R) == 4 && g.D == 6 && g.Dc == 12) return 3;
+  if (g.D == 6 && g.Dc == 12) return 3;
   if (sizeof(R) == 4 && g.D == 8 && g.Dc == 16) return 4;
   return 0;
 }
@@ -363,7 +403,7 @@ int max_blocks_pair_fused(const Geometry& g) {
   switch (pair_fused_id<R>(g)) {
     case 1: return fused_blocks<R, 2, 4>();
     case 2: return fused_blocks<R, 4, 8>();
-    case 3: return fused_blocks<R, sizeof(R) == 4 ? 6 : 2, sizeof(R) == 4 ? 12 : 4>();
+    case 3: return fused_blocks<R, 6, 12>();
     case 4: return fused_blocks<R, sizeof(R) == 4 ? 8 : 2, sizeof(R) == 4 ? 16 : 4>();
   }
   return 0;
@@ -412,7 +452,7 @@ cudaError_t launch_pair(const KArgs<R>& a, int grid, cudaStream_t st, int generi
   switch (generic ? 0 : pair_fused_id<R>(a.g)) {
     case 1: return launch_pair_fused<R, 2, 4>(a, grid, st);
     case 2: return launch_pair_fused<R, 4, 8>(a, grid, st);
-    case 3: return launch_pair_fused<R, sizeof(R) == 4 ? 6 : 2, sizeof(R) == 4 ? 12 : 4>(a, grid, st);
+    case 3: return launch_pair_fused<R, 6, 12>(a, grid, st);
     case 4: return launch_pair_fused<R, sizeof(R) == 4 ? 8 : 2, sizeof(R) == 4 ? 16 : 4>(a, grid, st);
   }
   const size_t smem = dyn_smem_bytes(a.g, sizeof(R), false, false);
@@ -423,6 +463,8 @@ cudaError_t launch_pair(const KArgs<R>& a, int grid, cudaStream_t st, int generi
 }
 
 #define PEPS_INST(R)                                                                                    \
+  template int max_blocks_pair_small<R>(const Geometry&);                                               \
+  template cudaError_t launch_pair_small<R>(const KArgs<R>&, int, cudaStream_t);                        \
   template int max_blocks_pair<R>(const Geometry&);                                                     \
   template int max_blocks_pair_fused<R>(const Geometry&);                                               \
   template cudaError_t launch_pair<R>(const KArgs<R>&, int, cudaStream_t, int);

@@ -2,32 +2,23 @@
 // amplitude ratios of horizontal spin exchanges and Delta = B/W.  One CTA per
 // (configuration, row); k_row_fused keeps every intermediate in shared memory
 // for (D, Dc) = (2,4), (4,8), (6,12), (8,16).
-#include "kernels_common.cuh"
+#include "small_ops.cuh"
 
 namespace peps {
 
 // ----------------------------------------------------------------- k_row
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ R red[64];
-  __shared__ uint64_t sp[kMaxWords];
+template <typename R, class Ops>
+__device__ void row_items(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int* eG) {
+  // G_c is stored scaled by 2^-eG[c]
   const Geometry& g = a.g;
   const int Lx = g.Lx, Ly = g.Ly, Dc = g.Dc, D = g.D;
   const int envT = Dc * D * Dc, D4 = D * D * D * D;
-  R* gsm;
-  int* gism;
-  smem_split<R>(smem_raw, g, false, false, gsm, gism);
-  R* p = a.scratch + (size_t)blockIdx.x * a.slot_elems;
   R* Gb = p; p += (size_t)(Lx + 1) * envT;
   R* F0 = p; p += envT;
   R* F1 = p; p += envT;
   R* X1 = p; p += envT;
   R* X2 = p; p += envT;
-  R* Bb = p; p += D4;
-  R* t0 = p; p += tmp_elems(g);
-  R* t1 = p;
-  __shared__ int eG[kMaxL + 1];   // G_c is stored scaled by 2^-eG[c]
+  R* Bb = p;
   for (int item = blockIdx.x; item < a.n * Ly; item += gridDim.x) {
     const int cfg = item / Ly, r = item % Ly;
     __syncthreads();
@@ -40,9 +31,9 @@ __global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
     int eacc = 0;
     for (int c = Lx - 1; c >= 0; --c) {
       const int site = r * Lx + c;
-      run_op<R>(OP_COL1_RIGHT, D, Dc, Gb + (size_t)(c + 1) * envT, Mu + (size_t)c * envT,
-                tptr(a, site, spin_of(sp, site)), Md + (size_t)c * envT, nullptr, Gb + (size_t)c * envT, t0, t1, gsm, gism);
-      eacc += normalize_pow2(Gb + (size_t)c * envT, envT, red);
+      ops.col1(true, Gb + (size_t)(c + 1) * envT, Mu + (size_t)c * envT,
+                tptr(a, site, spin_of(sp, site)), Md + (size_t)c * envT, Gb + (size_t)c * envT);
+      eacc += ops.normalize(Gb + (size_t)c * envT, envT);
       if (threadIdx.x == 0) eG[c] = eacc;
     }
     const R W = Gb[0];
@@ -55,8 +46,8 @@ __global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
       const int site = r * Lx + c;
       const int s = spin_of(sp, site);
       if (a.O != nullptr) {
-        run_op<R>(OP_SITE_ENV, D, Dc, F, Mu + (size_t)c * envT, Md + (size_t)c * envT,
-                  Gb + (size_t)(c + 1) * envT, nullptr, Bb, t0, t1, gsm, gism);
+        ops.site_env(F, Mu + (size_t)c * envT, Md + (size_t)c * envT,
+                  Gb + (size_t)(c + 1) * envT, Bb);
         R* Oo = a.O + ((size_t)cfg * g.N + site) * D4;
         const R inv = ok ? (R)ldexp(1.0 / (double)W, eF + eG[c + 1] - eG[0]) : R(0);
         for (int e = threadIdx.x; e < D4; e += blockDim.x) Oo[e] = Bb[e] * inv;
@@ -64,17 +55,15 @@ __global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
       if (c < Lx - 1) {
         const int s2 = spin_of(sp, site + 1);
         if (s != s2) {
-          run_op<R>(OP_COL1_LEFT, D, Dc, F, Mu + (size_t)c * envT, tptr(a, site, s2), Md + (size_t)c * envT,
-                    nullptr, X1, t0, t1, gsm, gism);
-          const int eX = normalize_pow2(X1, envT, red);
-          run_op<R>(OP_COL1_LEFT, D, Dc, X1, Mu + (size_t)(c + 1) * envT, tptr(a, site + 1, s),
-                    Md + (size_t)(c + 1) * envT, nullptr, X2, t0, t1, gsm, gism);
-          const R wp = block_dot(X2, Gb + (size_t)(c + 2) * envT, envT, red);
+          ops.col1(false, F, Mu + (size_t)c * envT, tptr(a, site, s2), Md + (size_t)c * envT, X1);
+          const int eX = ops.normalize(X1, envT);
+          ops.col1(false, X1, Mu + (size_t)(c + 1) * envT, tptr(a, site + 1, s),
+                    Md + (size_t)(c + 1) * envT, X2);
+          const R wp = ops.dot(X2, Gb + (size_t)(c + 2) * envT, envT);
           if (ok) eh += 0.5 * g.J1 * ldexp((double)wp / (double)W, eF + eX + eG[c + 2] - eG[0]);
         }
-        run_op<R>(OP_COL1_LEFT, D, Dc, F, Mu + (size_t)c * envT, tptr(a, site, s), Md + (size_t)c * envT,
-                  nullptr, Fn, t0, t1, gsm, gism);
-        eF += normalize_pow2(Fn, envT, red);
+        ops.col1(false, F, Mu + (size_t)c * envT, tptr(a, site, s), Md + (size_t)c * envT, Fn);
+        eF += ops.normalize(Fn, envT);
         F = Fn;
         Fn = (Fn == F0) ? F1 : F0;
       }
@@ -85,6 +74,57 @@ __global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
       if (!ok) atomicOr(&a.flags[cfg], kFlagZeroW);
     }
   }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ R red[64];
+  __shared__ uint64_t sp[kMaxWords];
+  __shared__ int eG[kMaxL + 1];
+  CtaOps<R> ops(a, red);
+  smem_split<R>(smem_raw, a.g, false, false, ops.zb.gsm, ops.zb.gism);
+  R* p = a.scratch + (size_t)blockIdx.x * a.slot_elems;
+  ops.t0 = p; p += tmp_elems(a.g);
+  ops.t1 = p; p += tmp_elems(a.g);
+  row_items<R>(a, ops, p, sp, eG);
+}
+
+// One warp per (configuration, row), for the models small.cuh takes: k_row's
+// contractions with each product on one warp in shared memory (small_ops.cuh).
+// 6x6 D = 3 Dc = 6 FP64, 128 configurations with Delta: 0.8 ms against 25 with k_row.
+template <typename R>
+__global__ void __launch_bounds__(32) k_row_small(KArgs<R> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t sp[kMaxWords];
+  __shared__ int eG[kMaxL + 1];
+  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw));
+  row_items<R>(a, ops, a.scratch + (size_t)blockIdx.x * a.slot_elems, sp, eG);
+}
+
+size_t row_small_slot_elems(const Geometry& g) {
+  const size_t envT = (size_t)g.Dc * g.D * g.Dc;
+  return (size_t)(g.Lx + 5) * envT + (size_t)g.D * g.D * g.D * g.D;
+}
+
+template <typename R>
+int max_blocks_row_small(const Geometry& g) {
+  int dev = 0, nsm = 0, nb = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem = (size_t)small::ops_reals(g.D, g.Dc) * sizeof(R);
+  prefer_shared(k_row_small<R>, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_row_small<R>, 32, smem);
+  return nsm * (nb < 1 ? 1 : nb);
+}
+
+template <typename R>
+cudaError_t launch_row_small(const KArgs<R>& a, int grid, cudaStream_t st) {
+  const size_t smem = (size_t)small::ops_reals(a.g.D, a.g.Dc) * sizeof(R);
+  cudaError_t e = prefer_shared(k_row_small<R>, smem);
+  if (e != cudaSuccess) return e;
+  k_row_small<R><<<grid, 32, smem, st>>>(a);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------- k_row_fused
@@ -171,6 +211,8 @@ static int row_fused_id(const Geometry& g) {
   return 0;
 }
 
+bool row_has_fused(const Geometry& g) { return row_fused_id<float>(g) != 0; }
+
 template <typename R, int D, int Dc>
 static int row_fused_blocks() {
   int dev = 0, nsm = 0, nb = 0;
@@ -224,6 +266,8 @@ cudaError_t launch_row(const KArgs<R>& a, int grid, cudaStream_t st, int generic
 }
 
 #define PEPS_INST(R)                                                                                    \
+  template int max_blocks_row_small<R>(const Geometry&);                                                \
+  template cudaError_t launch_row_small<R>(const KArgs<R>&, int, cudaStream_t);                         \
   template int max_blocks_row<R>(const Geometry&, int);                                                 \
   template cudaError_t launch_row<R>(const KArgs<R>&, int, cudaStream_t, int);
 PEPS_INST(double)
