@@ -17,7 +17,13 @@
 //      weights divided out again (zero weights and entries past an open edge
 //      give zero); Gamma_j' likewise.
 // The gates of one group act on disjoint bonds, so a group is one launch
-// with one CTA per bond.  Gate: exp(-dtau J S.S) = e^{-dtau J/4} (I - P_s) +
+// with one CTA per bond.  A launch has few CTAs and each is bound by FP64
+// instructions (a warp's costs the SM 16 cycles) and their latencies, so the
+// scalars are formed once, not by every lane of every warp: the SVD has
+// eight lanes a column pair and rotates V beside T, the two QRs run side by side on
+// half of the CTA each, weights, their inverses and the gate are tabulated, and
+// the matrices are in shared memory where they fit (D <= 7).  8x8 D = 5 with
+// next-nearest gates: 21 ms a Trotter step against 82 before.  Gate: exp(-dtau J S.S) = e^{-dtau J/4} (I - P_s) +
 // e^{3 dtau J/4} P_s, P_s the singlet projector (S.S = 1/4 on the triplet,
 // -3/4 on the singlet); a SWAP gate routes next-nearest pairs through their
 // shared neighbour.
@@ -29,8 +35,8 @@
 #include <vector>
 
 #include "../../include/peps.h"
+#include "fast64.cuh"
 #include "kernels.h"
-#include "qr.cuh"
 
 namespace peps {
 namespace su {
@@ -98,66 +104,198 @@ __device__ double gate_entry(int kind, double J1, double J2, double dtau, int p,
 }
 
 // One-sided Jacobi SVD of the row-major m2 x n2 matrix T (shared memory):
-// columns are rotated pairwise (round-robin order, one warp per pair) until
-// every pair is orthogonal to working precision; V (row-major n2 x n2)
-// accumulates the rotations, so T_in = T_out V^T with T_out = U diag(sigma).
-__device__ void jacobi_svd(double* T, int m2, int n2, double* V, int* s_rot) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// columns are rotated pairwise (round-robin order) until every pair is
+// orthogonal to working precision; V (row-major n2 x n2) accumulates the
+// rotations, so T_in = T_out V^T with T_out = U diag(sigma).
+// Each quarter of the SM issues an FP64 warp instruction every 64 cycles,
+// whatever its lanes do, so a round costs the instructions of its longest
+// warp.  A pair has 8 lanes, which split its rows and hold them in registers
+// from the dot products to the rotation; a T warp takes four pairs with one set
+// of scalar instructions.  V is rotated by other warps, in the round after,
+// beside the next dot products of T (cosines and sines through cs, two
+// rounds deep).  One barrier a round, for the warps that take part.
+__device__ __forceinline__ void jacobi_pair(int round, int k, int np, int& p, int& q) {
+  if (k == 0) {
+    p = round;
+    q = np - 1;
+  } else {
+    p = (round + k) % (np - 1);
+    q = (round - k + np - 1) % (np - 1);
+  }
+  if (p > q) {
+    const int t = p;
+    p = q;
+    q = t;
+  }
+}
+
+template <int RP>
+__device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int round, int np, int npair, double tol2,
+                                               double2* cs) {
+  const int gl = threadIdx.x & 7, k = threadIdx.x >> 3;
+  int p = 0, q = 0;
+  if (k < npair) jacobi_pair(round, k, np, p, q);
+  const bool on = k < npair && q < n2;
+  if (!on) p = q = 0;
+  double a[RP], b[RP];
+#pragma unroll
+  for (int x = 0; x < RP; ++x) {
+    const int r = gl + x * 8;
+    a[x] = r < m2 ? T[r * n2 + p] : 0.0;
+    b[x] = r < m2 ? T[r * n2 + q] : 0.0;
+  }
+  double al = 0.0, be = 0.0, ga = 0.0;
+#pragma unroll
+  for (int x = 0; x < RP; ++x) {
+    al = fma(a[x], a[x], al);
+    be = fma(b[x], b[x], be);
+    ga = fma(a[x], b[x], ga);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    al += __shfl_xor_sync(0xffffffffu, al, o);
+    be += __shfl_xor_sync(0xffffffffu, be, o);
+    ga += __shfl_xor_sync(0xffffffffu, ga, o);
+  }
+  const bool rot = on && ga * ga > tol2 * al * be;
+  double2 cn = make_double2(1.0, 0.0);
+  if (__any_sync(0xffffffffu, rot)) {
+    // the rotation with t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
+    // zeta = (be - al) / (2 ga): cos^2 = (1 + |be - al| / h) / 2 and
+    // sin = 2 ga / (2 h cos), h^2 = (be - al)^2 + (2 ga)^2
+    const double d = be - al, g2 = 2.0 * ga;
+    const double rh = quick_rsqrt(fma(d, d, g2 * g2));
+    const double c2 = fma(0.5 * fabs(d), rh, 0.5);
+    const double rc = quick_rsqrt(c2);
+    const double c = c2 * rc;
+    const double sn = (d == 0.0 ? fabs(g2) : (d > 0.0 ? g2 : -g2)) * (0.5 * rh) * rc;
+    if (rot) {
+      cn = make_double2(c, sn);
+#pragma unroll
+      for (int x = 0; x < RP; ++x) {
+        const int r = gl + x * 8;
+        if (r < m2) {
+          T[r * n2 + p] = c * a[x] - sn * b[x];
+          T[r * n2 + q] = sn * a[x] + c * b[x];
+        }
+      }
+    }
+  }
+  if (gl == 0 && k < npair) cs[k] = cn;
+  return rot;
+}
+
+__device__ void jacobi_svd(double* T, int m2, int n2, double* V, double2* cs, int* s_rot) {
   for (int e = threadIdx.x; e < n2 * n2; e += blockDim.x) V[e] = (e / n2 == e % n2) ? 1.0 : 0.0;
-  const int np = n2 + (n2 & 1);            // players, one dummy when n2 is odd
-  const double tol = 1e-15 * (double)m2;
+  const int np = n2 + (n2 & 1), npair = np / 2;   // players, one dummy when n2 is odd
+  const int nt = (npair + 3) / 4;                 // T warps, four pairs each; up to 32 pairs
+  // V warps: one on the quarter of the SM that has no T warp, else four beside the T warps
+  // (all of them where T takes all eight: T warps then also rotate V)
+  const int v0 = nt <= 3 ? 3 : (nt <= 4 ? 4 : 0), v1 = nt <= 3 ? 4 : kW;
+  const int warp = threadIdx.x >> 5, rp = (m2 + 7) / 8;
+  const bool is_t = warp < nt, is_v = warp >= v0 && warp < v1;
+  const int busy = v1 > nt ? v1 : nt;             // the warps that meet at the barrier: 0 .. busy - 1
+  const double tol = 1e-15 * (double)m2, tol2 = tol * tol;
+  __syncthreads();
   for (int sweep = 0; sweep < 40; ++sweep) {
     if (threadIdx.x == 0) *s_rot = 0;
     __syncthreads();
-    for (int round = 0; round < np - 1; ++round) {
-      for (int k = warp; k < np / 2; k += kW) {
-        int p, q;
-        if (k == 0) {
-          p = round;
-          q = np - 1;
-        } else {
-          p = (round + k) % (np - 1);
-          q = (round - k + np - 1) % (np - 1);
+    if (warp < busy) {
+      bool rotated = false;
+      for (int round = 0; round < np; ++round) {   // one more for V's last round
+        if (is_t && round < np - 1) {
+          double2* c = cs + (round & 1) * 32;
+          bool r;
+          if (rp <= 1) r = jacobi_round_t<1>(T, m2, n2, round, np, npair, tol2, c);
+          else if (rp <= 2) r = jacobi_round_t<2>(T, m2, n2, round, np, npair, tol2, c);
+          else if (rp <= 3) r = jacobi_round_t<3>(T, m2, n2, round, np, npair, tol2, c);
+          else if (rp <= 4) r = jacobi_round_t<4>(T, m2, n2, round, np, npair, tol2, c);
+          else r = jacobi_round_t<8>(T, m2, n2, round, np, npair, tol2, c);
+          rotated = rotated || r;
         }
-        if (p >= n2 || q >= n2) continue;
-        if (p > q) {
-          const int t = p;
-          p = q;
-          q = t;
-        }
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int r = lane; r < m2; r += 32) {
-          const double a = T[r * n2 + p], b = T[r * n2 + q];
-          al += a * a;
-          be += b * b;
-          ga += a * b;
-        }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        if (ga != 0.0 && fabs(ga) > tol * sqrt(al * be)) {
-          const double zeta = (be - al) / (2.0 * ga);
-          const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-          for (int r = lane; r < m2; r += 32) {
-            const double a = T[r * n2 + p], b = T[r * n2 + q];
-            T[r * n2 + p] = c * a - s * b;
-            T[r * n2 + q] = s * a + c * b;
+        if (is_v && round > 0) {
+          const double2* c = cs + ((round - 1) & 1) * 32;
+          const int step = (v1 - v0) * 32;
+          for (int e = threadIdx.x - v0 * 32; e < npair * n2; e += step) {
+            const int k = e / n2, r = e - k * n2;
+            const double2 x = c[k];
+            if (x.y != 0.0) {
+              int p, q;
+              jacobi_pair(round - 1, k, np, p, q);
+              const double a = V[r * n2 + p], b = V[r * n2 + q];
+              V[r * n2 + p] = x.x * a - x.y * b;
+              V[r * n2 + q] = x.y * a + x.x * b;
+            }
           }
-          for (int r = lane; r < n2; r += 32) {
-            const double a = V[r * n2 + p], b = V[r * n2 + q];
-            V[r * n2 + p] = c * a - s * b;
-            V[r * n2 + q] = s * a + c * b;
-          }
-          if (lane == 0) *s_rot = 1;
         }
+        asm volatile("bar.sync 1, %0;" ::"r"(32 * busy) : "memory");
       }
-      __syncthreads();
+      if (rotated) *s_rot = 1;
     }
+    __syncthreads();
     if (*s_rot == 0) break;
     __syncthreads();
   }
   __syncthreads();
+}
+
+// Householder QR (qr.cuh's convention) of the column-major m x n matrix M by
+// half of the CTA (threads 128 h ..): its first warp forms the reflector, its
+// four warps update the columns.
+__device__ void house_qr_half(double* M, int m, int n, double* tau, int h) {
+  const int t = threadIdx.x & 127, warp = t >> 5, lane = t & 31;
+  const int k_end = min(m, n);
+  for (int k = 0; k < k_end; ++k) {
+    double* x = M + (size_t)k * m;
+    if (warp == 0) {
+      double s2 = 0.0;
+      for (int r = k + 1 + lane; r < m; r += 32) s2 = fma(x[r], x[r], s2);
+      s2 = warp_sum(s2);
+      double ta = 0.0;
+      if (s2 != 0.0) {
+        const double alpha = x[k];
+        const double nrm2 = fma(alpha, alpha, s2), rn = quick_rsqrt(nrm2);
+        const double beta = alpha <= 0.0 ? nrm2 * rn : -(nrm2 * rn);
+        ta = (beta - alpha) * (alpha <= 0.0 ? rn : -rn);
+        const double sc = quick_rcp(alpha - beta);
+        __syncwarp();
+        for (int r = k + 1 + lane; r < m; r += 32) x[r] *= sc;
+        if (lane == 0) x[k] = beta;
+      }
+      if (lane == 0) tau[k] = ta;
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + h) : "memory");
+    const double ta = tau[k];
+    if (ta != 0.0) {
+      for (int c = k + 1 + warp; c < n; c += 4) {
+        double* y = M + (size_t)c * m;
+        double w = 0.0;
+        for (int r = k + 1 + lane; r < m; r += 32) w = fma(x[r], y[r], w);
+        w = (warp_sum(w) + y[k]) * ta;
+        __syncwarp();
+        if (lane == 0) y[k] -= w;
+        for (int r = k + 1 + lane; r < m; r += 32) y[r] = fma(-w, x[r], y[r]);
+      }
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + h) : "memory");
+  }
+}
+
+// One column y of Q y, Q the product of house_qr_half's reflectors, by one warp.
+__device__ __forceinline__ void apply_q_column(const double* M, const double* tau, double* y, int m, int nref) {
+  const int lane = threadIdx.x & 31;
+  for (int k = nref - 1; k >= 0; --k) {
+    const double t = tau[k];
+    if (t == 0.0) continue;
+    const double* v = M + (size_t)k * m;
+    double w = 0.0;
+    for (int r = k + 1 + lane; r < m; r += 32) w = fma(v[r], y[r], w);
+    w = (warp_sum(w) + y[k]) * t;
+    __syncwarp();
+    if (lane == 0) y[k] -= w;
+    for (int r = k + 1 + lane; r < m; r += 32) y[r] = fma(-w, v[r], y[r]);
+    __syncwarp();
+  }
 }
 
 struct Args {
@@ -170,17 +308,26 @@ struct Args {
   size_t slot;
 };
 
-// Shared memory: Theta and V (n2max^2 each, n2max = 4D), sigma, order, tau.
-__host__ __device__ inline size_t smem_doubles(int D) {
+// Shared memory: Theta and V (n2max^2 each, n2max = 4D), sigma and its inverse,
+// tau, the leg weights and their inverses ([2 sites][4 legs][D] each), the gate;
+// then M_i, M_j, N_i, N_j (D^3 x 2D each) where they fit.
+__host__ __device__ inline size_t smem_small_doubles(int D) {
   const size_t n2 = 4 * (size_t)D;
-  return 2 * n2 * n2 + n2 + 2 * 2 * (size_t)D + 16;
+  return 2 * n2 * n2 + 2 * n2 + 2 * 2 * (size_t)D + 2 * 8 * (size_t)D + 16;
+}
+__host__ __device__ inline size_t mats_doubles(int D) { return 4 * (size_t)D * D * D * 2 * D; }
+__host__ __device__ inline bool mats_in_smem(int D) {
+  return (smem_small_doubles(D) + mats_doubles(D)) * sizeof(double) <= 200 * 1024;
+}
+__host__ __device__ inline size_t smem_doubles(int D) {
+  return smem_small_doubles(D) + (mats_in_smem(D) ? mats_doubles(D) : 0);
 }
 
 __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ double red[kW];
   __shared__ int s_rot, s_order[64];
   __shared__ double s_nrm;
+  __shared__ double2 cs[64];
   const Geom& g = a.g;
   const int D = g.D, n = 2 * D, m = D * D * D, D4 = D * D * D * D;
   const Upd up = a.ups[blockIdx.x];
@@ -193,16 +340,32 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
     if (x != li) oi[t++] = x;
   for (int x = 0, t = 0; x < 4; ++x)
     if (x != lj) oj[t++] = x;
-  double* Mi = a.scratch + (size_t)blockIdx.x * a.slot;
-  double* Mj = Mi + (size_t)m * n;
-  double* Ni = Mj + (size_t)m * n;
-  double* Nj = Ni + (size_t)m * n;
   const int n2max = 4 * D;
   double* Th = sm;
   double* V = Th + (size_t)n2max * n2max;
   double* sig = V + (size_t)n2max * n2max;
-  double* tau_i = sig + n2max;
+  double* rsig = sig + n2max;
+  double* tau_i = rsig + n2max;
   double* tau_j = tau_i + n;
+  double* wt = tau_j + n;        // [2][4][D] weight of an index of a leg, 1 on the updated bond
+  double* wi = wt + 8 * D;       // their inverses, zero for zero
+  double* gate = wi + 8 * D;     // [4][4]
+  double* Mi = mats_in_smem(D) ? gate + 16 : a.scratch + (size_t)blockIdx.x * a.slot;
+  double* Mj = Mi + (size_t)m * n;
+  double* Ni = Mj + (size_t)m * n;
+  double* Nj = Ni + (size_t)m * n;
+  // ---- tables
+  for (int e = threadIdx.x; e < 8 * D; e += blockDim.x) {
+    const int site = e / (4 * D), leg = e / D % 4, x = e % D;
+    const double w = leg == (site ? lj : li) ? 1.0 : leg_w(g, a.lam, site ? j : i, leg, x);
+    wt[e] = w;
+    wi[e] = inv_or_zero(w);
+  }
+  if (threadIdx.x >= 240) {
+    const int e = threadIdx.x - 240;
+    gate[e] = gate_entry(up.kind, a.J1, a.J2, a.dtau, e >> 2, e & 3);
+  }
+  __syncthreads();
   // ---- 1. M_i, M_j with the weights absorbed
   for (int e = threadIdx.x; e < m * n; e += blockDim.x) {
     const int col = e / m, row = e % m;
@@ -214,7 +377,7 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
     legs[oi[2]] = o[2];
     legs[li] = x;
     double v = a.Gam[((size_t)i * 2 + s) * D4 + ((legs[0] * D + legs[1]) * D + legs[2]) * D + legs[3]];
-    v *= leg_w(g, a.lam, i, oi[0], o[0]) * leg_w(g, a.lam, i, oi[1], o[1]) * leg_w(g, a.lam, i, oi[2], o[2]);
+    v *= wt[oi[0] * D + o[0]] * wt[oi[1] * D + o[1]] * wt[oi[2] * D + o[2]];
     v *= a.lam[(size_t)bond * D + x];
     Mi[e] = v;
     legs[oj[0]] = o[0];
@@ -222,57 +385,53 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
     legs[oj[2]] = o[2];
     legs[lj] = x;
     double w = a.Gam[((size_t)j * 2 + s) * D4 + ((legs[0] * D + legs[1]) * D + legs[2]) * D + legs[3]];
-    w *= leg_w(g, a.lam, j, oj[0], o[0]) * leg_w(g, a.lam, j, oj[1], o[1]) * leg_w(g, a.lam, j, oj[2], o[2]);
+    w *= wt[(4 + oj[0]) * D + o[0]] * wt[(4 + oj[1]) * D + o[1]] * wt[(4 + oj[2]) * D + o[2]];
     Mj[e] = w;
   }
   __syncthreads();
-  // ---- 2. QR of both
-  qr::house_qr<double>(Mi, m, n, tau_i, red);
-  qr::house_qr<double>(Mj, m, n, tau_j, red);
+  // ---- 2. QR of both, side by side
+  if (threadIdx.x < kT / 2) house_qr_half(Mi, m, n, tau_i, 0);
+  else house_qr_half(Mj, m, n, tau_j, 1);
+  __syncthreads();
   const int ki = min(m, n), kj = min(m, n);
   const int m2 = 2 * ki, n2 = 2 * kj;
   // ---- 3. Theta[(a, s_i'), (s_j', b)]
   for (int e = threadIdx.x; e < m2 * n2; e += blockDim.x) {
     const int r = e / n2, c = e % n2;
     const int ai = r >> 1, sp = r & 1, sq = c / kj, bj = c % kj;
-    double P[2][2];
-    for (int si = 0; si < 2; ++si)
-      for (int sj = 0; sj < 2; ++sj) {
-        double t = 0.0;
-        for (int x = 0; x < D; ++x) {
-          const int ci = si * D + x, cj = sj * D + x;
-          const double ri = ai <= ci ? Mi[(size_t)ci * m + ai] : 0.0;
-          const double rj = bj <= cj ? Mj[(size_t)cj * m + bj] : 0.0;
-          t += ri * rj;
-        }
-        P[si][sj] = t;
-      }
     double v = 0.0;
-    for (int q = 0; q < 4; ++q) v += gate_entry(up.kind, a.J1, a.J2, a.dtau, sp * 2 + sq, q) * P[q >> 1][q & 1];
+    for (int q = 0; q < 4; ++q) {
+      const int si = q >> 1, sj = q & 1;
+      double t = 0.0;
+      for (int x = 0; x < D; ++x) {
+        const int ci = si * D + x, cj = sj * D + x;
+        if (ai <= ci && bj <= cj) t = fma(Mi[(size_t)ci * m + ai], Mj[(size_t)cj * m + bj], t);
+      }
+      v = fma(gate[(sp * 2 + sq) * 4 + q], t, v);
+    }
     Th[e] = v;
   }
   __syncthreads();
-  // ---- 4. SVD; the K largest singular values, in decreasing order
-  jacobi_svd(Th, m2, n2, V, &s_rot);
+  // ---- 4. SVD; the K largest singular values, in decreasing order (equal ones by column)
+  jacobi_svd(Th, m2, n2, V, cs, &s_rot);
   for (int c = threadIdx.x; c < n2; c += blockDim.x) {
     double t = 0.0;
-    for (int r = 0; r < m2; ++r) t += Th[r * n2 + c] * Th[r * n2 + c];
-    sig[c] = sqrt(t);
+    for (int r = 0; r < m2; ++r) t = fma(Th[r * n2 + c], Th[r * n2 + c], t);
+    const double sg = sqrt(t);
+    sig[c] = sg;
+    rsig[c] = sg > 0.0 ? 1.0 / sg : 0.0;
   }
   __syncthreads();
   const int K = min(D, min(m2, n2));
+  for (int c = threadIdx.x; c < n2; c += blockDim.x) {
+    int rank = 0;
+    for (int q = 0; q < n2; ++q) rank += sig[q] > sig[c] || (sig[q] == sig[c] && q < c) ? 1 : 0;
+    if (rank < K) s_order[rank] = c;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    bool used[64];
-    for (int c = 0; c < n2; ++c) used[c] = false;
     double nrm2 = 0.0;
-    for (int t = 0; t < K; ++t) {
-      int best = -1;
-      for (int c = 0; c < n2; ++c)
-        if (!used[c] && (best < 0 || sig[c] > sig[best])) best = c;
-      used[best] = true;
-      s_order[t] = best;
-      nrm2 += sig[best] * sig[best];
-    }
+    for (int t = 0; t < K; ++t) nrm2 = fma(sig[s_order[t]], sig[s_order[t]], nrm2);
     s_nrm = sqrt(nrm2);
   }
   __syncthreads();
@@ -280,43 +439,41 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
   // ---- new weight
   for (int x = threadIdx.x; x < D; x += blockDim.x)
     a.lam[(size_t)bond * D + x] = x < K ? (nrm > 0.0 ? sig[s_order[x]] / nrm : sig[s_order[x]]) : 0.0;
-  // ---- 5. N_i = [R_i'; 0], N_j = [R_j'; 0], then the reflectors
+  // ---- 5. N_i = [R_i'; 0], N_j = [R_j'; 0], then the reflectors, a column a warp
   for (int e = threadIdx.x; e < m * n; e += blockDim.x) {
     const int col = e / m, row = e % m;
     const int s = col / D, x = col % D;
     double vi = 0.0, vj = 0.0;
     if (x < K) {
       const int c = s_order[x];
-      const double sg = sig[c];
-      if (row < ki && sg > 0.0) vi = Th[(row * 2 + s) * n2 + c] / sg;
+      if (row < ki) vi = Th[(row * 2 + s) * n2 + c] * rsig[c];
       if (row < kj) vj = V[(s * kj + row) * n2 + c];
     }
     Ni[e] = vi;
     Nj[e] = vj;
   }
   __syncthreads();
-  qr::apply_q<double>(Mi, tau_i, Ni, m, n, n);
-  qr::apply_q<double>(Mj, tau_j, Nj, m, n, n);
-  // ---- back to Gamma with the outer weights divided out (the bond weight
-  // was just written; no thread reads it below)
+  for (int c = threadIdx.x >> 5; c < 2 * n; c += kW) {
+    if (c < n) apply_q_column(Mi, tau_i, Ni + (size_t)c * m, m, ki);
+    else apply_q_column(Mj, tau_j, Nj + (size_t)(c - n) * m, m, kj);
+  }
+  __syncthreads();
+  // ---- back to Gamma with the outer weights divided out
   for (int e = threadIdx.x; e < 2 * D4; e += blockDim.x) {
     const int s = e / D4, w = e % D4;
     const int legs[4] = {w / (D * D * D), w / (D * D) % D, w / D % D, w % D};
     {
       const int row = (legs[oi[0]] * D + legs[oi[1]]) * D + legs[oi[2]];
       const int col = s * D + legs[li];
-      double v = Ni[(size_t)col * m + row];
-      v *= inv_or_zero(leg_w(g, a.lam, i, oi[0], legs[oi[0]])) * inv_or_zero(leg_w(g, a.lam, i, oi[1], legs[oi[1]])) *
-           inv_or_zero(leg_w(g, a.lam, i, oi[2], legs[oi[2]]));
-      a.Gam[((size_t)i * 2) * D4 + e] = v;
+      const double f = wi[oi[0] * D + legs[oi[0]]] * wi[oi[1] * D + legs[oi[1]]] * wi[oi[2] * D + legs[oi[2]]];
+      a.Gam[((size_t)i * 2) * D4 + e] = Ni[(size_t)col * m + row] * f;
     }
     {
       const int row = (legs[oj[0]] * D + legs[oj[1]]) * D + legs[oj[2]];
       const int col = s * D + legs[lj];
-      double v = Nj[(size_t)col * m + row];
-      v *= inv_or_zero(leg_w(g, a.lam, j, oj[0], legs[oj[0]])) * inv_or_zero(leg_w(g, a.lam, j, oj[1], legs[oj[1]])) *
-           inv_or_zero(leg_w(g, a.lam, j, oj[2], legs[oj[2]]));
-      a.Gam[((size_t)j * 2) * D4 + e] = v;
+      const double f = wi[(4 + oj[0]) * D + legs[oj[0]]] * wi[(4 + oj[1]) * D + legs[oj[1]]] *
+                       wi[(4 + oj[2]) * D + legs[oj[2]]];
+      a.Gam[((size_t)j * 2) * D4 + e] = Nj[(size_t)col * m + row] * f;
     }
   }
 }
