@@ -21,7 +21,7 @@ OUT = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT, "libpeps.so")
 PHASE_OUT = os.path.join(OUT, "phase")
 PHASE_LIB = os.path.join(PHASE_OUT, "libpeps.so")
-SOURCES = ["kernels.cu", "small.cu", "row.cu", "pair.cu", "mc.cu", "corr.cu", "su.cu", "peaks.cu", "api.cu", "serve.cu"]
+SOURCES = ["boundary_f32.cu", "boundary_f64.cu", "static.cu", "kernels.cu", "small.cu", "row.cu", "pair.cu", "mc.cu", "corr.cu", "su.cu", "peaks.cu", "api.cu", "serve.cu"]
 INCLUDE = os.path.join(ROOT, "include")
 
 

@@ -354,8 +354,10 @@ peps_status sandwich_chunk(peps_ctx* c, const KArgs<R>& a, const uint64_t* S, in
   const bool tiny = g.Dc * g.Dc * g.D * g.D <= 400;
   const bool row_warps = warps && c->res_row_small && !c->row_generic &&
                          (tiny || !row_has_fused(g) || n * g.Ly > 2 * c->nsm);
+  // two-row items per SM from which warps are ahead: against the fused kernel in FP64, the generic one in FP64, in FP32
+  const int pair_few = c->elem == 8 ? (row_has_fused(g) ? 3 : 1) : 6;
   const bool pair_warps = warps && c->res_pair_small && c->pair_mode == 0 &&
-                          (tiny || n * (g.Ly - 1) >= (c->elem == 8 ? 3 : 6) * c->nsm);
+                          (tiny || n * (g.Ly - 1) >= pair_few * c->nsm);
   auto warp_grid = [&](KArgs<R>& b, size_t slot, int items, int res) {
     b.slot_elems = (slot + 31) / 32 * 32;
     const size_t slots = scratch_bytes(c, c->nslots) / c->elem / b.slot_elems;
@@ -447,7 +449,8 @@ peps_status evaluate_chunk(peps_ctx* c, const uint64_t* S, int n, bool need_env_
     const int res = c->boundary_ctas > 0 ? std::min(c->boundary_ctas, c->res_boundary) : c->res_boundary;
     const int grid = std::min(n * dirs, std::min(c->nslots, res));
     Prof pf(c, 0);
-    PEPS_CUDA(launch_boundary<R>(a, dirs, std::max(grid, 1), c->stream));
+    PEPS_CUDA(launch_boundary<R>(a, nullptr, nullptr, 0, dirs, a.scratch, a.slot_elems,
+                                 dyn_smem_bytes(c->g, c->elem, true, c->wm_smem), std::max(grid, 1), c->stream));
   }
   return sandwich_chunk<R>(c, a, S, n, need_env_l, need_pairs, sm, c->stream);
 }
@@ -773,7 +776,7 @@ peps_status packed_impl(peps_packer* pk, int nreq, peps_ctx* const* ctxs, const 
     slot[cls] = (slot[cls] + 31) / 32 * 32;
     if (nm[cls])
       grid[cls] = std::max(1, std::min(total[cls], cls == 0 ? max_blocks_boundary_small<R>(smem[cls])
-                                                            : max_blocks_boundary_packed<R>(smem[cls])));
+                                                            : max_blocks_boundary<R>(smem[cls])));
   }
   PEPS_CUDA(pk->scratch.ensure(sizeof(R) * std::max(slot[0] * grid[0], slot[1] * grid[1])));
   PEPS_CUDA(pk->models.ensure(sizeof(KArgs<R>) * nreq));
@@ -785,8 +788,8 @@ peps_status packed_impl(peps_packer* pk, int nreq, peps_ctx* const* ctxs, const 
     PEPS_CUDA(launch_boundary_small<R>(models[0], (const KArgs<R>*)pk->models.p, (const int*)pk->start.p, nm[0], dirs,
                                        (R*)pk->scratch.p, slot[0], smem[0], grid[0], pk->stream));
   if (nm[1])
-    PEPS_CUDA(launch_boundary_packed<R>((const KArgs<R>*)pk->models.p + first1, (const int*)pk->start.p + nm[0] + 1,
-                                        nm[1], dirs, (R*)pk->scratch.p, slot[1], smem[1], grid[1], pk->stream));
+    PEPS_CUDA(launch_boundary<R>(models[first1], (const KArgs<R>*)pk->models.p + first1,
+                                 (const int*)pk->start.p + nm[0] + 1, nm[1], dirs, (R*)pk->scratch.p, slot[1], smem[1], grid[1], pk->stream));
   for (int i = 0; i < nreq; ++i) {
     peps_ctx* c = ctxs[i];
     const bool want_e = eloc && eloc[i], want_O = O && O[i];
@@ -990,13 +993,13 @@ peps_status peps_create(const peps_params* p, const double* A_host, void* stream
     }
   }
   if (c->elem == 8) {
-    c->res_boundary = max_blocks_boundary<double>(c->g);
+    c->res_boundary = max_blocks_boundary<double>(dyn_smem_bytes(c->g, c->elem, true, c->wm_smem));
     c->res_row = max_blocks_row<double>(c->g);
     c->res_pair = max_blocks_pair_fused<double>(c->g);
     if (!c->res_pair) c->res_pair = max_blocks_pair<double>(c->g);
     c->res_mc = max_blocks_mc<double>(c->g);
   } else {
-    c->res_boundary = max_blocks_boundary<float>(c->g);
+    c->res_boundary = max_blocks_boundary<float>(dyn_smem_bytes(c->g, c->elem, true, c->wm_smem));
     c->res_row = max_blocks_row<float>(c->g);
     c->pair_tc = p->prec == PEPS_MIXED_TF32 && c->g.D == 8 && c->g.Dc == 16;
     c->res_pair = c->pair_tc ? max_blocks_pair_tc() : max_blocks_pair_fused<float>(c->g);

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "contract.cuh"
+#include "fast64.cuh"
 #include "sturm64.cuh"
 
 // Phase markers inside the truncation.  Empty in the library; the
@@ -420,12 +421,89 @@ PEPS_HD int zip_gemm_reals(const GemmDesc& g) {
   return 0;
 }
 
-// C = A B for the zip-up contractions: gemm_wk when the descriptor fits it
-// and `sm_reals` reals of shared scratch, else cta_gemm.  Same results either
-// way.
+// C = A B in FP64 with both operands whole in shared memory (k-major) and the
+// 4 x 4 output tiles dealt to the threads one after the other: what bounds it
+// is the number of FP64 instructions a warp issues, and fixed CTA tiles of
+// 128 x 64 issued three times the needed ones at 144 x 36 or 72 x 72 outputs
+// (10x10 D = 6).  Each output is the same chain over k.
+static __device__ __noinline__ void gemm_dealt(const GemmDesc& g, const double* A, const double* B,
+                                               double* __restrict__ C, double* sm, int* ism) {
+  const int M = g.M, N = g.N, K = g.K, tid = threadIdx.x;
+  double* As = sm;           // [K][M]
+  double* Bs = sm + K * M;   // [K][N]
+  int* rA = ism;
+  int* rC = rA + M;
+  int* cB = rC + M;
+  int* cC = cB + N;
+  int* ktA = cC + N;
+  int* ktB = ktA + K;
+  __syncthreads();
+  for (int e = tid; e < M; e += kThreads) {
+    rA[e] = ixoff(g.am, e);
+    rC[e] = ixoff(g.cm, e);
+  }
+  for (int e = tid; e < N; e += kThreads) {
+    cB[e] = ixoff(g.bn, e);
+    cC[e] = ixoff(g.cn, e);
+  }
+  for (int k = tid; k < K; k += kThreads) {
+    ktA[k] = ixoff(g.ak, k);
+    ktB[k] = ixoff(g.bk, k);
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int e = tid; e < K * M; e += kThreads) As[e] = A[rA[e % M] + ktA[e / M]];
+#pragma unroll 4
+  for (int e = tid; e < K * N; e += kThreads) Bs[e] = B[ktB[e / N] + cB[e % N]];
+  __syncthreads();
+  const int tn = (N + 3) / 4, nt = ((M + 3) / 4) * tn;
+  for (int t = tid; t < nt; t += kThreads) {
+    const int i0 = (t / tn) * 4, j0 = (t % tn) * 4;
+    double acc[4][4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) acc[x][y] = 0.0;
+    int ia[4], jb[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      ia[q] = min(i0 + q, M - 1);
+      jb[q] = min(j0 + q, N - 1);
+    }
+#pragma unroll 2
+    for (int k = 0; k < K; ++k) {
+      double a[4], b[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        a[q] = As[k * M + ia[q]];
+        b[q] = Bs[k * N + jb[q]];
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y)
+        if (i0 + x < M && j0 + y < N) C[rC[i0 + x] + cC[j0 + y]] = acc[x][y];
+  }
+  __syncthreads();
+}
+
+// C = A B for the zip-up contractions: gemm_dealt in FP64 and gemm_wk in FP32
+// when the descriptor fits them and `sm_reals` reals of shared scratch, else
+// cta_gemm.  Same results either way.
 template <typename R>
 __device__ __noinline__ void zip_gemm(const GemmDesc& g, const R* A, const R* B, R* __restrict__ C, R* sm, int* ism,
                          int sm_reals) {
+  if constexpr (sizeof(R) == 8) {
+    if (g.nb == 1 && g.K * (g.M + g.N) <= sm_reals && 2 * (g.M + g.N + g.K) <= kGemmSmemInts) {
+      gemm_dealt(g, A, B, C, sm, ism);
+      return;
+    }
+  }
   const int need = zip_gemm_reals(g);
   if (need > 0 && need <= sm_reals) {
     if (g.N > 64) gemm_wk<R, 64, 128, 4, 8, 16>(g, A, B, C, sm, ism);
@@ -543,17 +621,33 @@ PEPS_HD size_t trunc_ws_elems(int pq, int kmax, bool with_wm) {
 }
 
 // Householder vector for x = (alpha, rest): returns tau, scale for rest, beta.
-template <typename R>
-__device__ __forceinline__ void householder(R alpha, R ss, R& tau, R& scale, R& beta) {
-  if (ss <= R(0)) {
-    tau = R(0);
-    scale = R(0);
+__device__ __forceinline__ void householder(float alpha, float ss, float& tau, float& scale, float& beta) {
+  if (ss <= 0.f) {
+    tau = 0.f;
+    scale = 0.f;
     beta = alpha;
   } else {
-    const R nrm = dsqrt(alpha * alpha + ss);
-    beta = alpha >= R(0) ? -nrm : nrm;
+    const float nrm = dsqrt(alpha * alpha + ss);
+    beta = alpha >= 0.f ? -nrm : nrm;
     tau = (beta - alpha) / beta;
-    scale = R(1) / (alpha - beta);
+    scale = 1.f / (alpha - beta);
+  }
+}
+// FP64: one reciprocal square root gives the norm and 1 / beta, so the chain
+// holds eleven FP64 instructions instead of about forty.
+__device__ __forceinline__ void householder(double alpha, double ss, double& tau, double& scale, double& beta) {
+  if (ss <= 0.0) {
+    tau = 0.0;
+    scale = 0.0;
+    beta = alpha;
+  } else {
+    const double n2 = fma(alpha, alpha, ss);
+    const double r = quick_rsqrt(n2);
+    const bool neg = __double2hiint(alpha) < 0;   // beta takes the other sign
+    const double nrm = n2 * r;
+    beta = neg ? nrm : -nrm;
+    tau = (beta - alpha) * (neg ? r : -r);
+    scale = quick_rcp(alpha - beta);
   }
 }
 
@@ -690,6 +784,42 @@ __device__ __forceinline__ float quick_div(float num, float d) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return __fmul_rn(num, r);
 }
+// Comparisons of magnitudes, start values and scales of the inverse iteration.
+// FP64 does them on the bits: an FP64 instruction, a comparison too, keeps its
+// unit busy for 64 cycles.
+__device__ __forceinline__ bool abs_ge(float a, float b) { return fabsf(a) >= fabsf(b); }
+__device__ __forceinline__ bool abs_ge(double a, double b) {
+  return (__double_as_longlong(a) & 0x7fffffffffffffffll) >= (__double_as_longlong(b) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ bool is_zero(float a) { return a == 0.f; }
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) & 0x7fffffffffffffffll) == 0; }
+__device__ __forceinline__ float with_sign(float m, float s) { return s < 0.f ? -m : m; }
+__device__ __forceinline__ double with_sign(double m, double s) {
+  return __hiloint2double(__double2hiint(m) | (__double2hiint(s) & 0x80000000), __double2loint(m));
+}
+__device__ __forceinline__ float inv_start(unsigned h, float) {
+  return float((int)(h & 0xffffu) - 32768) / 32768.f + 0.001f;
+}
+__device__ __forceinline__ double inv_start(unsigned h, double) {   // magnitude in [1/2, 1), random sign
+  return __hiloint2double((int)((h & 0x800fffffu) | 0x3fe00000u), (int)(h * 2654435761u));
+}
+// Largest magnitude so far, and the scale that brings it to about one.
+struct MaxOf32 {
+  float m = 0.f;
+  __device__ void add(float y) { m = fmaxf(m, fabsf(y)); }
+  __device__ float scale() const { return m > 0.f ? 1.f / m : 1.f; }
+};
+struct MaxOf64 {
+  int m = 0;
+  __device__ void add(double y) { m = max(m, __double2hiint(y) & 0x7fffffff); }
+  __device__ double scale() const {
+    const int e = m >> 20;
+    return e > 0 && e < 2046 ? __hiloint2double((2046 - e) << 20, 0) : 1.0;
+  }
+};
+template <typename R> struct MaxOf;
+template <> struct MaxOf<float> { typedef MaxOf32 type; };
+template <> struct MaxOf<double> { typedef MaxOf64 type; };
 // The workspace start for `p`: the next multiple of 32 bytes.
 template <typename R>
 __device__ __forceinline__ R* inv_align(R* p) {
@@ -704,7 +834,7 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
   unsigned h = seed * 2654435761u + 12345u;
   auto start = [&]() {
     h ^= h << 13; h ^= h >> 17; h ^= h << 5;
-    return R((int)(h & 0xffffu) - 32768) / R(32768) + R(0.001);
+    return inv_start(h, R(0));
   };
   // ---- factorisation, carrying dd[i], du[i] (current row) and dd[i+1],
   // du[i+1], with the forward elimination of the start vector (carrying b[i])
@@ -717,8 +847,8 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
     const R tn = i + 1 < n2 - 1 ? t[i + 1] : R(0);
     const R nd = -lam;
     const R bn = start();
-    const bool sw = !(fabs(cur_d) >= fabs(sub));
-    R d = sw ? sub : (cur_d == R(0) ? pivtiny : cur_d);
+    const bool sw = !abs_ge(cur_d, sub);
+    R d = sw ? sub : (is_zero(cur_d) ? pivtiny : cur_d);
     const R num = sw ? cur_d : sub;
     R lm, rd;
     if constexpr (sizeof(R) == 4) {
@@ -726,8 +856,8 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
       if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
       rd = quick_div(1.f, d);
     } else {
-      if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
-      rd = R(1) / d;
+      if (!abs_ge(d, pivtiny)) d = with_sign(pivtiny, d);
+      rd = quick_rcp(d);
       lm = num * rd;
     }
     const R u = sw ? nd : cur_u, y = sw ? cur_u : nd;
@@ -782,12 +912,13 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
       wl[3] = bf;
     }
     // ---- backward: U^-1, carrying y[i+1], y[i+2]; track max |y|
-    R y1 = R(0), y2 = R(0), mx = R(0);
+    R y1 = R(0), y2 = R(0);
+    typename MaxOf<R>::type mx;
     auto step = [&](R* p, const InvRow<R>& v, R tn) {
       const R d2 = flag_get(v.mult) ? tn : R(0);
       const R y = fma(-d2, y2, fma(-v.du, y1, v.b)) * v.rdd;
       p[3] = y;
-      mx = fmax(mx, fabs(y));
+      mx.add(y);
       y2 = y1;
       y1 = y;
     };
@@ -816,7 +947,7 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
 #pragma unroll
       for (int q = 0; q < B; ++q) step(w - q * st, cv[q], ct[q]);
     }
-    sc = mx > R(0) ? R(1) / mx : R(1);
+    sc = mx.scale();
   }
   return sc;
 }
@@ -1138,6 +1269,272 @@ __device__ __forceinline__ int apply_reflectors(const float* W, int ld, bool tal
   return jlo - 1;
 }
 
+// W[i][c] -= cf(c) rf(i) for i0 <= i < P, col0 <= c < col0 + ncol <= 256: a warp
+// takes every eighth row, two at a time, with its column factors and the rows'
+// chunks of 32 columns in registers, so that a row's loads do not wait for the
+// stores of the one before.  The number of chunks is a template argument: a
+// predicated-off FP64 instruction still takes its issue time.  note(i, chunk,
+// entry, acc) sees the updated entries in order; done(acc) ends a warp's part.
+template <typename R, int NCH, class CF, class RF, class Note>
+__device__ __forceinline__ R rank1_chunks(R* W, int ld, int i0, int P, int col0, int ncol, CF cf, RF rf, Note note) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool last = 32 * (NCH - 1) + lane < ncol;
+  R w[NCH], acc = R(0);
+#pragma unroll
+  for (int t = 0; t < NCH; ++t) w[t] = (t < NCH - 1 || last) ? cf(col0 + lane + 32 * t) : R(0);
+  int i = i0 + warp;
+  for (; i + kWarps < P; i += 2 * kWarps) {
+    R* r0 = W + i * ld + col0 + lane;
+    R* r1 = r0 + kWarps * ld;
+    const R v0 = rf(i), v1 = rf(i + kWarps);
+    R x0[NCH], x1[NCH];
+#pragma unroll
+    for (int t = 0; t < NCH; ++t)
+      if (t < NCH - 1 || last) {
+        x0[t] = r0[32 * t] - w[t] * v0;
+        x1[t] = r1[32 * t] - w[t] * v1;
+      }
+#pragma unroll
+    for (int t = 0; t < NCH; ++t)
+      if (t < NCH - 1 || last) {
+        r0[32 * t] = x0[t];
+        r1[32 * t] = x1[t];
+      }
+#pragma unroll
+    for (int t = 0; t < NCH; ++t)
+      if (t < NCH - 1 || last) note(i, t, x0[t], acc);
+#pragma unroll
+    for (int t = 0; t < NCH; ++t)
+      if (t < NCH - 1 || last) note(i + kWarps, t, x1[t], acc);
+  }
+  if (i < P) {
+    R* r0 = W + i * ld + col0 + lane;
+    const R v0 = rf(i);
+#pragma unroll
+    for (int t = 0; t < NCH; ++t)
+      if (t < NCH - 1 || last) {
+        const R x = r0[32 * t] - w[t] * v0;
+        r0[32 * t] = x;
+        note(i, t, x, acc);
+      }
+  }
+  return acc;
+}
+template <typename R, class CF, class RF, class Note, class Done>
+__device__ __forceinline__ void rank1_rows(R* W, int ld, int i0, int P, int col0, int ncol, CF cf, RF rf, Note note,
+                                           Done done) {
+  R acc;
+  switch ((ncol + 31) >> 5) {
+    case 1: acc = rank1_chunks<R, 1>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    case 2: acc = rank1_chunks<R, 2>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    case 3: acc = rank1_chunks<R, 3>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    case 4: acc = rank1_chunks<R, 4>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    case 5: acc = rank1_chunks<R, 5>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    case 6: acc = rank1_chunks<R, 6>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    case 7: acc = rank1_chunks<R, 7>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+    default: acc = rank1_chunks<R, 8>(W, ld, i0, P, col0, ncol, cf, rf, note); break;
+  }
+  done(acc);
+}
+
+// Householder bidiagonalisation (W = Q_L B Q_R^T, B upper bidiagonal) of X or its
+// transpose in W (shared or global memory), for the blocks bidiag_tiles_f32 does
+// not take.  One function for both sweep directions: it is most of the
+// truncation's code.
+template <typename R>
+static __device__ __noinline__ void bidiag_shared(const R* X, int m, int n, bool tall, int P, int Q, R* W, int ld, R* tt,
+                                                  R* tau4, int qm, R* wv_, R* red) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    R* tauL = tau4;
+    R* tauR = tau4 + qm;
+    for (int e = tid; e < m * n; e += blockDim.x) {
+      const int i = e / n, j = e % n;
+      if (tall) W[i * ld + j] = X[e];
+      else W[j * ld + i] = X[e];
+    }
+    __syncthreads();
+    // ---------------- bidiagonalisation: W = Q_L B Q_R^T, B upper bidiagonal
+    // Reflectors are kept unscaled in W with their scale factors in sL / sR
+    // (v = scale * stored, implicit 1 on the diagonal / super-diagonal).  The
+    // norm each Householder vector needs is accumulated while the previous
+    // rank-1 update writes those entries, and every thread forms the scalars
+    // itself, so one column costs four barriers.
+    R* wv = wv_;
+    R* sL = tau4 + 2 * qm;        // left scale factors (t2 is filled later)
+    R* sR = sL + qm;
+    R* part = red + 40;                // per-warp partial norms (8)
+    {
+      R ss = R(0);
+      for (int i = 1 + tid; i < P; i += blockDim.x) ss += W[i * ld] * W[i * ld];
+      ss = block_sum(ss, red + 16);
+      if (tid < kWarps) part[tid] = tid == 0 ? ss : R(0);
+      __syncthreads();
+    }
+    for (int j = 0; j < Q; ++j) {
+      // -- left reflector on column j (rows j..P-1); its norm is in part[]
+      R colnorm = R(0);
+      for (int q = 0; q < kWarps; ++q) colnorm += part[q];
+      R tau, scale, beta;
+      householder(W[j * ld + j], colnorm, tau, scale, beta);
+      if (tid == 0) {
+        tt[2 * j] = beta;
+        tauL[j] = tau;
+        sL[j] = scale;
+      }
+      const int ncol = Q - j - 1;
+      R rownorm = R(0);                // squared norm of row j beyond j+1 after the left update
+      if (tau != R(0) && ncol > 0) {
+        // wv[c] = tau * (W[j][c] + scale * sum_{i>j} W[i][j] W[i][c])
+        int tpc = kThreads / ncol;
+        tpc = tpc >= 32 ? 32 : tpc >= 16 ? 16 : tpc >= 8 ? 8 : tpc >= 4 ? 4 : tpc >= 2 ? 2 : 1;
+        const int cpr = kThreads / tpc;
+        for (int cb = 0; cb < ncol; cb += cpr) {
+          const int cl = cb + tid / tpc, gl = tid % tpc;
+          const bool act = cl < ncol;
+          const int c = j + 1 + (act ? cl : 0);
+          R s0 = R(0), s1 = R(0), s2 = R(0), s3 = R(0);
+          int i = j + 1 + gl;
+#pragma unroll 2
+          for (; i + 3 * tpc < P; i += 4 * tpc) {
+            s0 += W[i * ld + j] * W[i * ld + c];
+            s1 += W[(i + tpc) * ld + j] * W[(i + tpc) * ld + c];
+            s2 += W[(i + 2 * tpc) * ld + j] * W[(i + 2 * tpc) * ld + c];
+            s3 += W[(i + 3 * tpc) * ld + j] * W[(i + 3 * tpc) * ld + c];
+          }
+          for (; i < P; i += tpc) s0 += W[i * ld + j] * W[i * ld + c];
+          const R sacc = warp_sum((s0 + s1) + (s2 + s3), tpc);
+          if (act && gl == 0) wv[c] = tau * (W[j * ld + c] + scale * sacc);
+        }
+        __syncthreads();
+        // W[i][c] -= wv[c] v_i for i >= j, c > j; warp 0 takes row j and its norm
+        rank1_rows<R>(
+            W, ld, j, P, j + 1, ncol, [&](int c) { return wv[c]; },
+            [&](int i) { return i == j ? R(1) : scale * W[i * ld + j]; },
+            [&](int i, int t, R x, R& acc) {
+              if (i == j && 32 * t + lane >= 1) acc += x * x;
+            },
+            [&](R acc) {
+              if (warp == 0) {
+                acc = warp_sum(acc);
+                if (lane == 0) red[5] = acc;
+              }
+            });
+        __syncthreads();
+        rownorm = red[5];
+      } else if (ncol > 0) {
+        if (warp == 0) {
+          R rn = R(0);
+          for (int c = j + 2 + lane; c < Q; c += 32) rn += W[j * ld + c] * W[j * ld + c];
+          rn = warp_sum(rn);
+          if (lane == 0) red[5] = rn;
+        }
+        __syncthreads();
+        rownorm = red[5];
+      }
+      if (j < Q - 1) {
+        // -- right reflector on row j (columns j+1..Q-1)
+        R tr, sr, br;
+        householder(W[j * ld + j + 1], rownorm, tr, sr, br);
+        if (tid == 0) {
+          tt[2 * j + 1] = br;
+          tauR[j] = tr;
+          sR[j] = sr;
+        }
+        const int nrow = P - j - 1;
+        if (tr != R(0)) {
+          // wv[i] = tr * (W[i][j+1] + sr * sum_{c>j+1} W[i][c] W[j][c])
+          int tpc = kThreads / nrow;
+          tpc = tpc >= 32 ? 32 : tpc >= 16 ? 16 : tpc >= 8 ? 8 : tpc >= 4 ? 4 : tpc >= 2 ? 2 : 1;
+          const int rpr = kThreads / tpc;
+          for (int rb = 0; rb < nrow; rb += rpr) {
+            const int rl = rb + tid / tpc, gl = tid % tpc;
+            const bool act = rl < nrow;
+            const int i = j + 1 + (act ? rl : 0);
+            R s0 = R(0), s1 = R(0), s2 = R(0), s3 = R(0);
+            int c = j + 2 + gl;
+#pragma unroll 2
+            for (; c + 3 * tpc < Q; c += 4 * tpc) {
+              s0 += W[i * ld + c] * W[j * ld + c];
+              s1 += W[i * ld + c + tpc] * W[j * ld + c + tpc];
+              s2 += W[i * ld + c + 2 * tpc] * W[j * ld + c + 2 * tpc];
+              s3 += W[i * ld + c + 3 * tpc] * W[j * ld + c + 3 * tpc];
+            }
+            for (; c < Q; c += tpc) s0 += W[i * ld + c] * W[j * ld + c];
+            const R sacc = warp_sum((s0 + s1) + (s2 + s3), tpc);
+            if (act && gl == 0) wv[i] = tr * (W[i * ld + j + 1] + sr * sacc);
+          }
+          __syncthreads();
+          // W[i][c] -= wv[i] v'_c for i > j, c > j; lane 0 of each warp sums column j+1 below row j+1
+          rank1_rows<R>(
+              W, ld, j + 1, P, j + 1, ncol, [&](int c) { return c == j + 1 ? R(1) : sr * W[j * ld + c]; },
+              [&](int i) { return wv[i]; },
+              [&](int i, int t, R x, R& acc) {
+                if (t == 0 && lane == 0 && i > j + 1) acc += x * x;
+              },
+              [&](R acc) {
+                if (lane == 0) part[warp] = acc;
+              });
+          __syncthreads();
+        } else {
+          // no right update: column j+1's norm below row j+1 as it stands
+          R cn = R(0);
+          for (int i = j + 2 + tid; i < P; i += blockDim.x) cn += W[i * ld + j + 1] * W[i * ld + j + 1];
+          cn = block_sum(cn, red + 16);
+          if (tid < kWarps) part[tid] = tid == 0 ? cn : R(0);
+          __syncthreads();
+        }
+      }
+    }
+    // the last column's diagonal entry (tt[2Q-2], written by thread 0) is
+    // read by another warp in the bisection set-up below
+    __syncthreads();
+}
+
+// Gram-Schmidt with re-orthogonalisation of the columns of Ub (Q x K); a
+// degenerate direction is replaced by a unit vector.
+template <typename R>
+static __device__ __noinline__ void gram_schmidt(R* Ub, int Q, int K, R* red) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int j = 0; j < K; ++j) {
+    for (int attempt = 0; attempt <= Q; ++attempt) {
+      R s = R(0);
+      for (int i = tid; i < Q; i += blockDim.x) s += Ub[i * K + j] * Ub[i * K + j];
+      R nrm0 = dsqrt(block_sum(s, red + 16));
+      if (nrm0 > R(0)) {
+        for (int i = tid; i < Q; i += blockDim.x) Ub[i * K + j] /= nrm0;
+        __syncthreads();
+      }
+      for (int pass = 0; pass < 2; ++pass) {
+        for (int p = warp; p < j; p += kWarps) {
+          R d = R(0);
+          for (int i = lane; i < Q; i += 32) d += Ub[i * K + p] * Ub[i * K + j];
+          d = warp_sum(d);
+          if (lane == 0) red[32 + p] = d;
+        }
+        __syncthreads();
+        for (int i = tid; i < Q; i += blockDim.x) {
+          R v = Ub[i * K + j];
+          for (int p = 0; p < j; ++p) v -= red[32 + p] * Ub[i * K + p];
+          Ub[i * K + j] = v;
+        }
+        __syncthreads();
+      }
+      s = R(0);
+      for (int i = tid; i < Q; i += blockDim.x) s += Ub[i * K + j] * Ub[i * K + j];
+      const R nrm = dsqrt(block_sum(s, red + 16));
+      if (nrm0 > R(0) && nrm > R(1e-3)) {
+        for (int i = tid; i < Q; i += blockDim.x) Ub[i * K + j] /= nrm;
+        __syncthreads();
+        break;
+      }
+      // degenerate direction (zero singular value or lost vector): try a unit vector
+      const int q = (j + attempt) % Q;
+      for (int i = tid; i < Q; i += blockDim.x) Ub[i * K + j] = i == q ? R(1) : R(0);
+      __syncthreads();
+    }
+  }
+}
+
 // Writes U_K (m x K) through (uo_r, uo_c) and C' = U_K^T X (K x n) through
 // (co_r, co_c).  X is not modified.  K <= min(m, n), K <= 32.
 template <typename R>
@@ -1175,159 +1572,7 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
       tiled = true;
     }
   }
-  if (!tiled) {
-    for (int e = tid; e < m * n; e += blockDim.x) {
-      const int i = e / n, j = e % n;
-      if (tall) W[i * ld + j] = X[e];
-      else W[j * ld + i] = X[e];
-    }
-    __syncthreads();
-    // ---------------- bidiagonalisation: W = Q_L B Q_R^T, B upper bidiagonal
-    // Reflectors are kept unscaled in W with their scale factors in sL / sR
-    // (v = scale * stored, implicit 1 on the diagonal / super-diagonal).  The
-    // norm each Householder vector needs is accumulated while the previous
-    // rank-1 update writes those entries, and every thread forms the scalars
-    // itself, so one column costs four barriers.
-    R* wv = w.wv;
-    R* sL = w.tau + 2 * w.Qmax;        // left scale factors (t2 is filled later)
-    R* sR = sL + w.Qmax;
-    R* part = red + 40;                // per-warp partial norms (8)
-    {
-      R ss = R(0);
-      for (int i = 1 + tid; i < P; i += blockDim.x) ss += W[i * ld] * W[i * ld];
-      ss = block_sum(ss, red + 16);
-      if (tid < kWarps) part[tid] = tid == 0 ? ss : R(0);
-      __syncthreads();
-    }
-    for (int j = 0; j < Q; ++j) {
-      // -- left reflector on column j (rows j..P-1); its norm is in part[]
-      R colnorm = R(0);
-      for (int q = 0; q < kWarps; ++q) colnorm += part[q];
-      R tau, scale, beta;
-      householder(W[j * ld + j], colnorm, tau, scale, beta);
-      if (tid == 0) {
-        w.t[2 * j] = beta;
-        tauL[j] = tau;
-        sL[j] = scale;
-      }
-      const int ncol = Q - j - 1;
-      R rownorm = R(0);                // squared norm of row j beyond j+1 after the left update
-      if (tau != R(0) && ncol > 0) {
-        // wv[c] = tau * (W[j][c] + scale * sum_{i>j} W[i][j] W[i][c])
-        int tpc = kThreads / ncol;
-        tpc = tpc >= 32 ? 32 : tpc >= 16 ? 16 : tpc >= 8 ? 8 : tpc >= 4 ? 4 : tpc >= 2 ? 2 : 1;
-        const int cpr = kThreads / tpc;
-        for (int cb = 0; cb < ncol; cb += cpr) {
-          const int cl = cb + tid / tpc, gl = tid % tpc;
-          const bool act = cl < ncol;
-          const int c = j + 1 + (act ? cl : 0);
-          R s0 = R(0), s1 = R(0), s2 = R(0), s3 = R(0);
-          int i = j + 1 + gl;
-          for (; i + 3 * tpc < P; i += 4 * tpc) {
-            s0 += W[i * ld + j] * W[i * ld + c];
-            s1 += W[(i + tpc) * ld + j] * W[(i + tpc) * ld + c];
-            s2 += W[(i + 2 * tpc) * ld + j] * W[(i + 2 * tpc) * ld + c];
-            s3 += W[(i + 3 * tpc) * ld + j] * W[(i + 3 * tpc) * ld + c];
-          }
-          for (; i < P; i += tpc) s0 += W[i * ld + j] * W[i * ld + c];
-          const R sacc = warp_sum((s0 + s1) + (s2 + s3), tpc);
-          if (act && gl == 0) wv[c] = tau * (W[j * ld + c] + scale * sacc);
-        }
-        __syncthreads();
-        // W[i][c] -= wv[c] v_i for i >= j, c > j; warp 0 takes row j and its norm
-        for (int i = j + warp; i < P; i += kWarps) {
-          const R v = i == j ? R(1) : scale * W[i * ld + j];
-          R rn = R(0);
-          for (int c = j + 1 + lane; c < Q; c += 32) {
-            const R x = W[i * ld + c] - wv[c] * v;
-            W[i * ld + c] = x;
-            if (c >= j + 2) rn += x * x;
-          }
-          if (i == j) {
-            rn = warp_sum(rn);
-            if (lane == 0) red[5] = rn;
-          }
-        }
-        __syncthreads();
-        rownorm = red[5];
-      } else if (ncol > 0) {
-        if (warp == 0) {
-          R rn = R(0);
-          for (int c = j + 2 + lane; c < Q; c += 32) rn += W[j * ld + c] * W[j * ld + c];
-          rn = warp_sum(rn);
-          if (lane == 0) red[5] = rn;
-        }
-        __syncthreads();
-        rownorm = red[5];
-      }
-      if (j < Q - 1) {
-        // -- right reflector on row j (columns j+1..Q-1)
-        R tr, sr, br;
-        householder(W[j * ld + j + 1], rownorm, tr, sr, br);
-        if (tid == 0) {
-          w.t[2 * j + 1] = br;
-          tauR[j] = tr;
-          sR[j] = sr;
-        }
-        const int nrow = P - j - 1;
-        if (tr != R(0)) {
-          // wv[i] = tr * (W[i][j+1] + sr * sum_{c>j+1} W[i][c] W[j][c])
-          int tpc = kThreads / nrow;
-          tpc = tpc >= 32 ? 32 : tpc >= 16 ? 16 : tpc >= 8 ? 8 : tpc >= 4 ? 4 : tpc >= 2 ? 2 : 1;
-          const int rpr = kThreads / tpc;
-          for (int rb = 0; rb < nrow; rb += rpr) {
-            const int rl = rb + tid / tpc, gl = tid % tpc;
-            const bool act = rl < nrow;
-            const int i = j + 1 + (act ? rl : 0);
-            R s0 = R(0), s1 = R(0), s2 = R(0), s3 = R(0);
-            int c = j + 2 + gl;
-            for (; c + 3 * tpc < Q; c += 4 * tpc) {
-              s0 += W[i * ld + c] * W[j * ld + c];
-              s1 += W[i * ld + c + tpc] * W[j * ld + c + tpc];
-              s2 += W[i * ld + c + 2 * tpc] * W[j * ld + c + 2 * tpc];
-              s3 += W[i * ld + c + 3 * tpc] * W[j * ld + c + 3 * tpc];
-            }
-            for (; c < Q; c += tpc) s0 += W[i * ld + c] * W[j * ld + c];
-            const R sacc = warp_sum((s0 + s1) + (s2 + s3), tpc);
-            if (act && gl == 0) wv[i] = tr * (W[i * ld + j + 1] + sr * sacc);
-          }
-          __syncthreads();
-          // W[i][c] -= wv[i] v'_c for i > j, c > j; lane 0 of each warp sums column j+1 below row j+1
-          R vl[8];
-  #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const int c = j + 1 + lane + 32 * t;
-            vl[t] = c == j + 1 ? R(1) : (c < Q ? sr * W[j * ld + c] : R(0));
-          }
-          R cn = R(0);
-          for (int i = j + 1 + warp; i < P; i += kWarps) {
-            const R wi = wv[i];
-  #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-              const int c = j + 1 + lane + 32 * t;
-              if (c < Q) {
-                const R x = W[i * ld + c] - wi * vl[t];
-                W[i * ld + c] = x;
-                if (t == 0 && lane == 0 && i > j + 1) cn += x * x;
-              }
-            }
-          }
-          if (lane == 0) part[warp] = cn;
-          __syncthreads();
-        } else {
-          // no right update: column j+1's norm below row j+1 as it stands
-          R cn = R(0);
-          for (int i = j + 2 + tid; i < P; i += blockDim.x) cn += W[i * ld + j + 1] * W[i * ld + j + 1];
-          cn = block_sum(cn, red + 16);
-          if (tid < kWarps) part[tid] = tid == 0 ? cn : R(0);
-          __syncthreads();
-        }
-      }
-    }
-    // the last column's diagonal entry (w.t[2Q-2], written by thread 0) is
-    // read by another warp in the bisection set-up below
-    __syncthreads();
-  }   // !tiled
+  if (!tiled) bidiag_shared<R>(X, m, n, tall, P, Q, W, ld, w.t, w.tau, w.Qmax, w.wv, red);
   PEPS_PHASE(1);
   // ---------------- Sturm sections for the K largest singular values
   const int n2 = 2 * Q;
@@ -1359,7 +1604,7 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
     __syncthreads();
     section_f32(t2f, n2, K, 4.001f, Eps<float>::tiny * 4096.f, lamf);
     __syncthreads();
-    if (warp == 0) refine_values_f64(w.t2, n2, K, lamf, pow2<R>(e2), w.lam);
+    if (warp < 4) refine_values_f64(tid, K <= 8 ? 16 : K <= 16 ? 8 : 4, w.t2, n2, K, lamf, pow2<R>(e2), w.lam);
   }
   __syncthreads();
   PEPS_PHASE(2);
@@ -1417,9 +1662,16 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
             bad = 1;
             break;
           }
-          const R r = dsqrt(d);
-          __syncwarp();
-          if (lane > j && lane < K) G[j * K + lane] /= r;
+          R r;
+          if constexpr (sizeof(R) == 4) {
+            r = dsqrt(d);
+            __syncwarp();
+            if (lane > j && lane < K) G[j * K + lane] /= r;
+          } else {   // the diagonal holds 1 / r
+            r = quick_rsqrt(d);
+            __syncwarp();
+            if (lane > j && lane < K) G[j * K + lane] *= r;
+          }
           __syncwarp();
           if (lane == j) G[j * K + j] = r;
           if (lane > j && lane < K) {
@@ -1454,14 +1706,14 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
               R x = Ub[i * K + l];
 #pragma unroll
               for (int k = 0; k < l; ++k) x = fma(-u[k], G[k * K + l], x);
-              u[l] = x / G[l * K + l];
+              u[l] = sizeof(R) == 4 ? x / G[l * K + l] : x * G[l * K + l];
               Ub[i * K + l] = u[l];
             }
         } else {
           for (int l = 0; l < K; ++l) {
             R x = Ub[i * K + l];
             for (int k = 0; k < l; ++k) x -= Ub[i * K + k] * G[k * K + l];
-            Ub[i * K + l] = x / G[l * K + l];
+            Ub[i * K + l] = sizeof(R) == 4 ? x / G[l * K + l] : x * G[l * K + l];
           }
         }
       }
@@ -1469,44 +1721,7 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
     }
   }
   // ---------------- Gram-Schmidt with re-orthogonalisation (CGS2), fallback
-  for (int j = 0; j < K && need_cgs; ++j) {
-    for (int attempt = 0; attempt <= Q; ++attempt) {
-      R s = R(0);
-      for (int i = tid; i < Q; i += blockDim.x) s += Ub[i * K + j] * Ub[i * K + j];
-      R nrm0 = dsqrt(block_sum(s, red + 16));
-      if (nrm0 > R(0)) {
-        for (int i = tid; i < Q; i += blockDim.x) Ub[i * K + j] /= nrm0;
-        __syncthreads();
-      }
-      for (int pass = 0; pass < 2; ++pass) {
-        for (int p = warp; p < j; p += kWarps) {
-          R d = R(0);
-          for (int i = lane; i < Q; i += 32) d += Ub[i * K + p] * Ub[i * K + j];
-          d = warp_sum(d);
-          if (lane == 0) red[32 + p] = d;
-        }
-        __syncthreads();
-        for (int i = tid; i < Q; i += blockDim.x) {
-          R v = Ub[i * K + j];
-          for (int p = 0; p < j; ++p) v -= red[32 + p] * Ub[i * K + p];
-          Ub[i * K + j] = v;
-        }
-        __syncthreads();
-      }
-      s = R(0);
-      for (int i = tid; i < Q; i += blockDim.x) s += Ub[i * K + j] * Ub[i * K + j];
-      const R nrm = dsqrt(block_sum(s, red + 16));
-      if (nrm0 > R(0) && nrm > R(1e-3)) {
-        for (int i = tid; i < Q; i += blockDim.x) Ub[i * K + j] /= nrm;
-        __syncthreads();
-        break;
-      }
-      // degenerate direction (zero singular value or lost vector): try a unit vector
-      const int q = (j + attempt) % Q;
-      for (int i = tid; i < Q; i += blockDim.x) Ub[i * K + j] = i == q ? R(1) : R(0);
-      __syncthreads();
-    }
-  }
+  if (need_cgs) gram_schmidt<R>(Ub, Q, K, red);
   PEPS_PHASE(4);
   // ---------------- back-transformation by the stored reflectors, in blocks
   // U = H_0 H_1 ... H_{nref-1} [Ub; 0].  A block of nb consecutive reflectors
@@ -1775,9 +1990,34 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
       w.Uk[e] = v;
     }
     __syncthreads();
-    // C' = U_K^T X
-    GemmDesc g = gemm(K, n, m, ix1(1), kx(m, 0, K), kx(m, 0, n), ix1(1), co_r, co_c);
-    cta_gemm<R>(g, w.Uk, X, Cout, false, w.gsm, w.gism);
+    for (int e = tid; e < m * K; e += blockDim.x) Uk[e] = w.Uk[e];
+    __syncthreads();
+    // C' = U_K^T X: an item is a column and four rows (a full tile of the GEMM
+    // engine would spend most of its FP64 instructions on padding: K is 6 to 32)
+    constexpr int CH = 4, XB = 8;
+    const int nchunk = (K + CH - 1) / CH;
+    for (int item = tid; item < n * nchunk; item += blockDim.x) {
+      const int j = item % n, a0 = (item / n) * CH;
+      R sacc[CH];
+#pragma unroll
+      for (int q = 0; q < CH; ++q) sacc[q] = R(0);
+      for (int ib = 0; ib < m; ib += XB) {
+        R xb[XB];
+#pragma unroll
+        for (int u = 0; u < XB; ++u) xb[u] = ib + u < m ? X[(ib + u) * n + j] : R(0);
+#pragma unroll
+        for (int u = 0; u < XB; ++u)
+          if (ib + u < m) {
+#pragma unroll
+            for (int q = 0; q < CH; ++q)
+              if (a0 + q < K) sacc[q] = fma(Uk[(ib + u) * K + a0 + q], xb[u], sacc[q]);
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < CH; ++q)
+        if (a0 + q < K) Cout[ixoff(co_r, a0 + q) + ixoff(co_c, j)] = sacc[q];
+    }
+    __syncthreads();
   }
   PEPS_PHASE(6);
 }

@@ -69,14 +69,12 @@ size_t mc_slot_elems(const Geometry& g, bool wm_in_smem);
 size_t wm_smem_bytes(const Geometry& g, size_t elem);
 bool wm_fits_smem(const Geometry& g, size_t elem);
 
-template <typename R> cudaError_t launch_boundary(const KArgs<R>& a, int dirs, int grid, cudaStream_t st);
 // generic != 0 takes the generic kernel even where a fused one exists for (D, Dc).
 template <typename R> cudaError_t launch_row(const KArgs<R>& a, int grid, cudaStream_t st, int generic = 0);
 template <typename R> cudaError_t launch_pair(const KArgs<R>& a, int grid, cudaStream_t st, int generic = 0);
 template <typename R> cudaError_t launch_mc(const KArgs<R>& a, uint64_t* S, int nsweeps, uint64_t seed,
                                             uint64_t chain0, uint64_t sweep0, long long* accepted,
                                             int grid, cudaStream_t st);
-template <typename R> int max_blocks_boundary(const Geometry& g);
 // Boundary sweeps with one warp per sweep (small.cuh), for the models
 // boundary_small_fits accepts: of one model (nm = 0) or packed as below; a slot
 // is one boundary MPS, the resident count is for smem bytes of shared memory.
@@ -86,14 +84,15 @@ template <typename R> int max_blocks_boundary_small(size_t smem);
 template <typename R> cudaError_t launch_boundary_small(const KArgs<R>& one, const KArgs<R>* models_dev,
                                                         const int* start_dev, int nm, int dirs, R* scratch,
                                                         size_t slot_elems, size_t smem, int grid, cudaStream_t st);
-// Boundary sweeps of several models in one launch (k_boundary_packed): models_dev
-// [nm] kernel arguments in device memory, start_dev [nm + 1] first work item of
-// each model (n * dirs items per model), one scratch slot of slot_elems reals
-// per CTA, smem bytes of dynamic shared memory (the largest model's).
-template <typename R> int max_blocks_boundary_packed(size_t smem);
-template <typename R> cudaError_t launch_boundary_packed(const KArgs<R>* models_dev, const int* start_dev, int nm,
-                                                         int dirs, R* scratch, size_t slot_elems, size_t smem,
-                                                         int grid, cudaStream_t st);
+// Boundary sweeps with one CTA each, of one model (nm = 0) or of several in one
+// launch: models_dev [nm] kernel arguments in device memory, start_dev [nm + 1]
+// first work item of each model (n * dirs items per model), one scratch slot of
+// slot_elems reals per CTA, smem bytes of dynamic shared memory (the largest
+// model's).
+template <typename R> int max_blocks_boundary(size_t smem);
+template <typename R> cudaError_t launch_boundary(const KArgs<R>& one, const KArgs<R>* models_dev,
+                                                  const int* start_dev, int nm, int dirs, R* scratch,
+                                                  size_t slot_elems, size_t smem, int grid, cudaStream_t st);
 size_t dyn_smem_bytes(const Geometry& g, size_t elem, bool truncates, bool wm_in_smem);
 template <typename R> int max_blocks_mc(const Geometry& g);
 // Sandwiches with one warp per item, for the models boundary_small_fits accepts.

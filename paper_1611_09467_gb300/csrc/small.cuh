@@ -487,7 +487,7 @@ __device__ R values(const R* t, R* t2, int Q, int K, R* lam, R* scratch) {
   else bisect_f32<8>(t2f, n2, K, boundf, pivf, lamf);
   __syncwarp();
   if constexpr (sizeof(R) == 8) {
-    refine_values_f64(t2, n2, K, lamf, pow2<R>(e), lam);
+    refine_values_f64(l, K <= 2 ? 16 : K <= 4 ? 8 : K <= 8 ? 4 : 2, t2, n2, K, lamf, pow2<R>(e), lam);
     __syncwarp();
   }
   return tmax;
@@ -517,9 +517,16 @@ __device__ __noinline__ void orthonormalise(R* Ub, R* G, int Q, int K) {
         need_cgs = true;
         break;
       }
-      const R r = dsqrt(d);
-      __syncwarp();
-      if (l > j && l < K) G[j * K + l] /= r;
+      R r;
+      if constexpr (sizeof(R) == 4) {
+        r = dsqrt(d);
+        __syncwarp();
+        if (l > j && l < K) G[j * K + l] /= r;
+      } else {   // the diagonal holds 1 / r
+        r = quick_rsqrt(d);
+        __syncwarp();
+        if (l > j && l < K) G[j * K + l] *= r;
+      }
       __syncwarp();
       if (l == j) G[j * K + j] = r;
       if (l > j && l < K) {
@@ -546,7 +553,7 @@ __device__ __noinline__ void orthonormalise(R* Ub, R* G, int Q, int K) {
         R x = Ub[l * K + c];
 #pragma unroll
         for (int k = 0; k < c; ++k) x = fma(-u[k], G[k * K + c], x);
-        u[c] = x / G[c * K + c];
+        u[c] = sizeof(R) == 4 ? x / G[c * K + c] : x * G[c * K + c];
         Ub[l * K + c] = u[c];
       }
     }

@@ -11,9 +11,10 @@
 //     the method of bisection", Numer. Math. 9 (1967)).  p is scaled by a
 //     power of two every eight rows; signs and scales are integer work.
 //   * The first 24 bits come from the FP32 sixteen-section; only the rest is
-//     counted in FP64, with as many points per value and step as one warp has
-//     lanes (every FP64 instruction of a warp costs the SM 16 cycles, so
-//     points beyond 32 would be paid for in full).
+//     counted in FP64, with as many points per value and step as the lanes of
+//     one warp, or of four warps, give (an FP64 instruction of a warp keeps one
+//     of the SM's four FP64 units busy for 64 cycles, so further points would
+//     be paid for in full).
 #pragma once
 
 #include <cstdint>
@@ -57,16 +58,20 @@ __device__ __forceinline__ int sturm_count_minors(const double* t2, int n2, doub
 // divisions), so its values are within about 1e-6; this allows eight times that.
 constexpr double kSturmWiden = 0x1p-17;
 
-// The K <= 32 largest singular values by one warp: lam32 the FP32 values
-// (scaled units), t2 the scaled squares; lam[k] receives 2^e times the k-th.
-__device__ __forceinline__ void refine_values_f64(const double* t2, int n2, int K, const float* lam32, double scale,
-                                                  double* lam) {
-  const int l = threadIdx.x & 31;
-  const int G = K <= 2 ? 16 : K <= 4 ? 8 : K <= 8 ? 4 : K <= 16 ? 2 : 1;
+// The K <= 32 largest singular values by whole warps of threads t = 0 .. 31 or
+// 0 .. 127 (G points a value and step, G K <= the number of threads): lam32 the
+// FP32 values (scaled units), t2 the scaled squares; lam[k] receives scale
+// times the k-th.  An FP64 instruction keeps a quarter of the SM busy for 64
+// cycles whatever its lanes do, so a CTA counts with four warps, one a quarter
+// (10x10 D = 6: 240 kcycles a cut against 410 with one warp).
+__device__ __forceinline__ void refine_values_f64(int t, int G, const double* t2, int n2, int K, const float* lam32,
+                                                  double scale, double* lam) {
+  const int l = t & 31;
   // (G + 1)^nit >= 2^38: from the start interval below 2^-15 to under an ulp
-  const int nit = K <= 2 ? 10 : K <= 4 ? 12 : K <= 8 ? 17 : K <= 16 ? 24 : 38;
-  const double inv = K <= 2 ? 1.0 / 17 : K <= 4 ? 1.0 / 9 : K <= 8 ? 1.0 / 5 : K <= 16 ? 1.0 / 3 : 0.5;
-  const int gid = l / G, gl = l - gid * G;
+  const int nit = G >= 16 ? 10 : G >= 8 ? 12 : G >= 4 ? 17 : G >= 2 ? 24 : 38;
+  const double inv = G >= 16 ? 1.0 / 17 : G >= 8 ? 1.0 / 9 : G >= 4 ? 1.0 / 5 : G >= 2 ? 1.0 / 3 : 0.5;
+  const int gid = t / G, gl = t - gid * G, gbase = l / G * G;
+  if (__all_sync(0xffffffffu, gid >= K)) return;
   const int idx = n2 - 1 - gid;   // ascending index of the (gid + 1)-th largest
   const double c = gid < K ? (double)lam32[gid] : 1.0;
   double lo = fmax(c - kSturmWiden, 0.0), hi = c + kSturmWiden;
@@ -74,7 +79,7 @@ __device__ __forceinline__ void refine_values_f64(const double* t2, int n2, int 
     const double step = (hi - lo) * inv;
     const double x = fma(step, (double)(gl + 1), lo);
     const bool pred = sturm_count_minors(t2, n2, x) <= idx;
-    const unsigned bits = (__ballot_sync(0xffffffffu, pred) >> (gid * G)) & ((1u << G) - 1u);
+    const unsigned bits = (__ballot_sync(0xffffffffu, pred) >> gbase) & ((1u << G) - 1u);
     const int gs = __popc(bits);
     if (gs < G) hi = fma(step, (double)(gs + 1), lo);
     lo = fma(step, (double)gs, lo);
