@@ -49,6 +49,8 @@ __device__ void mc_chains(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int* 
           const R* Md;
           if (pass == 0) Md = r == Ly - 1 ? a.triv_mps : envL + (size_t)(r + 1) * Lx * envT;
           else Md = r + 2 > Ly - 1 ? a.triv_mps : envL + (size_t)(r + 2) * Lx * envT;
+          // true bonds of U_{r-1}, by column boundary
+          const int* bu = r == 0 ? ones : a.bd + (size_t)(r - 1) * (Lx + 1);
           const size_t tsz = pass == 0 ? envT : envT2;
           const R* triv = pass == 0 ? a.triv_t1 : a.triv_t2;
           for (size_t e = threadIdx.x; e < tsz; e += blockDim.x) Hb[(size_t)Lx * tsz + e] = triv[e];
@@ -61,7 +63,7 @@ __device__ void mc_chains(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int* 
               ops.col1(true, Hb + (size_t)(c + 1) * tsz, Mu + (size_t)c * envT,
                         tptr(a, i1, spin_of(sp, i1)), Md + (size_t)c * envT, Hb + (size_t)c * tsz);
             else
-              ops.col2(true, Hb + (size_t)(c + 1) * tsz, Mu + (size_t)c * envT,
+              ops.col2(true, bu[c], Hb + (size_t)(c + 1) * tsz, Mu + (size_t)c * envT,
                         tptr(a, i1, spin_of(sp, i1)), tptr(a, i1 + Lx, spin_of(sp, i1 + Lx)),
                         Md + (size_t)c * envT, Hb + (size_t)c * tsz);
             eacc += ops.normalize(Hb + (size_t)c * tsz, (int)tsz);
@@ -90,8 +92,8 @@ __device__ void mc_chains(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int* 
                 w = ops.dot(X1, Hb + (size_t)(c + 1) * tsz, (int)tsz);
                 wp = ops.dot(X2, Hb + (size_t)(c + 2) * tsz, (int)tsz);
               } else {
-                ops.col2(false, E, Muc, tptr(a, i1, s1), tptr(a, i2, s2), Mdc, X1);
-                ops.col2(false, E, Muc, tptr(a, i1, s2), tptr(a, i2, s1), Mdc, Xf);
+                ops.col2(false, bu[c + 1], E, Muc, tptr(a, i1, s1), tptr(a, i2, s2), Mdc, X1);
+                ops.col2(false, bu[c + 1], E, Muc, tptr(a, i1, s2), tptr(a, i2, s1), Mdc, Xf);
                 w = ops.dot(X1, Hb + (size_t)(c + 1) * tsz, (int)tsz);
                 wp = ops.dot(Xf, Hb + (size_t)(c + 1) * tsz, (int)tsz);
               }
@@ -121,7 +123,7 @@ __device__ void mc_chains(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int* 
               if (pass == 0)
                 ops.col1(false, E, Muc, tptr(a, i1, s1), Mdc, X1);
               else
-                ops.col2(false, E, Muc, tptr(a, i1, s1), tptr(a, i2, s2), Mdc, X1);
+                ops.col2(false, bu[c + 1], E, Muc, tptr(a, i1, s1), tptr(a, i2, s2), Mdc, X1);
               chosen = (e + 1) & 3;
             }
             e = chosen;

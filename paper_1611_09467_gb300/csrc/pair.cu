@@ -27,11 +27,14 @@ __device__ void pair_items(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int*
     if (threadIdx.x == 0) eH[Lx] = 0;
     __syncthreads();
     const R* Mu = r == 0 ? a.triv_mps : a.envU + ((size_t)cfg * Ly + (r - 1)) * Lx * envT;
+    // true bonds of U_{r-1}, by column boundary
+    const int* bu = r == 0 ? nullptr : a.bd + (size_t)(r - 1) * (Lx + 1);
+    auto nu = [&](int c) { return bu ? bu[c] : 1; };
     const R* Md = r + 2 > Ly - 1 ? a.triv_mps : a.envL + ((size_t)cfg * Ly + (r + 2)) * Lx * envT;
     int eacc = 0;
     for (int c = Lx - 1; c >= 0; --c) {
       const int s1 = r * Lx + c, s2 = (r + 1) * Lx + c;
-      ops.col2(true, Hb + (size_t)(c + 1) * envT2, Mu + (size_t)c * envT,
+      ops.col2(true, nu(c), Hb + (size_t)(c + 1) * envT2, Mu + (size_t)c * envT,
                 tptr(a, s1, spin_of(sp, s1)), tptr(a, s2, spin_of(sp, s2)), Md + (size_t)c * envT,
                 Hb + (size_t)c * envT2);
       eacc += ops.normalize(Hb + (size_t)c * envT2, envT2);
@@ -49,7 +52,7 @@ __device__ void pair_items(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int*
       const R* Muc = Mu + (size_t)c * envT;
       const R* Mdc = Md + (size_t)c * envT;
       if (a1 != a2) {  // vertical pair (r,c)-(r+1,c)
-        ops.col2(false, E, Muc, tptr(a, i1, a2), tptr(a, i2, a1), Mdc, X1);
+        ops.col2(false, nu(c + 1), E, Muc, tptr(a, i1, a2), tptr(a, i2, a1), Mdc, X1);
         const R wp = ops.dot(X1, Hb + (size_t)(c + 1) * envT2, envT2);
         if (ok) ev += 0.5 * g.J1 * ldexp((double)wp / (double)W, eE + eH[c + 1] - eH[0]);
       }
@@ -59,22 +62,22 @@ __device__ void pair_items(const KArgs<R>& a, Ops& ops, R* p, uint64_t* sp, int*
         const R* Mun = Mu + (size_t)(c + 1) * envT;
         const R* Mdn = Md + (size_t)(c + 1) * envT;
         if (a1 != b2) {  // diagonal (r,c)-(r+1,c+1)
-          ops.col2(false, E, Muc, tptr(a, i1, b2), tptr(a, i2, a2), Mdc, X1);
+          ops.col2(false, nu(c + 1), E, Muc, tptr(a, i1, b2), tptr(a, i2, a2), Mdc, X1);
           const int eX = ops.normalize(X1, envT2);
-          ops.col2(false, X1, Mun, tptr(a, j1, b1), tptr(a, j2, a1), Mdn, X2);
+          ops.col2(false, nu(c + 2), X1, Mun, tptr(a, j1, b1), tptr(a, j2, a1), Mdn, X2);
           const R wp = ops.dot(X2, Hb + (size_t)(c + 2) * envT2, envT2);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
         if (b1 != a2) {  // anti-diagonal (r,c+1)-(r+1,c)
-          ops.col2(false, E, Muc, tptr(a, i1, a1), tptr(a, i2, b1), Mdc, X1);
+          ops.col2(false, nu(c + 1), E, Muc, tptr(a, i1, a1), tptr(a, i2, b1), Mdc, X1);
           const int eX = ops.normalize(X1, envT2);
-          ops.col2(false, X1, Mun, tptr(a, j1, a2), tptr(a, j2, b2), Mdn, X2);
+          ops.col2(false, nu(c + 2), X1, Mun, tptr(a, j1, a2), tptr(a, j2, b2), Mdn, X2);
           const R wp = ops.dot(X2, Hb + (size_t)(c + 2) * envT2, envT2);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
       }
       if (c < Lx - 1) {
-        ops.col2(false, E, Muc, tptr(a, i1, a1), tptr(a, i2, a2), Mdc, En);
+        ops.col2(false, nu(c + 1), E, Muc, tptr(a, i1, a1), tptr(a, i2, a2), Mdc, En);
         eE += ops.normalize(En, envT2);
         E = En;
         En = (En == E0) ? E1 : E0;
@@ -164,11 +167,14 @@ __global__ void __launch_bounds__(kThreads) k_pair_fused(KArgs<R> a) {
     __syncthreads();
     const R* Mu = r == 0 ? a.triv_mps : a.envU + ((size_t)cfg * Ly + (r - 1)) * Lx * envT;
     const R* Md = r + 2 > Ly - 1 ? a.triv_mps : a.envL + ((size_t)cfg * Ly + (r + 2)) * Lx * envT;
+    // true bonds of L_{r+2}, by column boundary
+    const int* bl = r + 2 > Ly - 1 ? nullptr : a.bd + (size_t)(Ly + Ly - 3 - r) * (Lx + 1);
+    auto nb = [&](int c) { return bl ? bl[c] : 1; };
     int eacc = 0;
     for (int c = Lx - 1; c >= 0; --c) {
       const int s1 = r * Lx + c, s2 = (r + 1) * Lx + c;
       int e = 0;
-      pair_step_fused<R, D, Dc>(true, Hb + (size_t)(c + 1) * envT2, Hb + (size_t)c * envT2, Mu + (size_t)c * envT,
+      pair_step_fused<R, D, Dc>(true, nb(c + 1), Hb + (size_t)(c + 1) * envT2, Hb + (size_t)c * envT2, Mu + (size_t)c * envT,
                                 tptr(a, s1, spin_of(sp, s1)), tptr(a, s2, spin_of(sp, s2)), Md + (size_t)c * envT,
                                 nullptr, sm, red, &e);
       eacc += e;
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_fused(KArgs<R> a) {
       const R* Muc = Mu + (size_t)c * envT;
       const R* Mdc = Md + (size_t)c * envT;
       if (a1 != a2) {  // vertical pair (r,c)-(r+1,c)
-        const R wp = pair_step_fused<R, D, Dc>(false, E, nullptr, Muc, tptr(a, i1, a2), tptr(a, i2, a1), Mdc,
+        const R wp = pair_step_fused<R, D, Dc>(false, nb(c), E, nullptr, Muc, tptr(a, i1, a2), tptr(a, i2, a1), Mdc,
                                                Hb + (size_t)(c + 1) * envT2, sm, red);
         if (ok) ev += 0.5 * g.J1 * ldexp((double)wp / (double)W, eE + eH[c + 1] - eH[0]);
       }
@@ -197,22 +203,22 @@ __global__ void __launch_bounds__(kThreads) k_pair_fused(KArgs<R> a) {
         const R* Mdn = Md + (size_t)(c + 1) * envT;
         if (a1 != b2) {  // diagonal (r,c)-(r+1,c+1)
           int eX = 0;
-          pair_step_fused<R, D, Dc>(false, E, X1, Muc, tptr(a, i1, b2), tptr(a, i2, a2), Mdc, nullptr, sm, red, &eX);
-          const R wp = pair_step_fused<R, D, Dc>(false, X1, nullptr, Mun, tptr(a, j1, b1), tptr(a, j2, a1), Mdn,
+          pair_step_fused<R, D, Dc>(false, nb(c), E, X1, Muc, tptr(a, i1, b2), tptr(a, i2, a2), Mdc, nullptr, sm, red, &eX);
+          const R wp = pair_step_fused<R, D, Dc>(false, nb(c + 1), X1, nullptr, Mun, tptr(a, j1, b1), tptr(a, j2, a1), Mdn,
                                                  Hb + (size_t)(c + 2) * envT2, sm, red);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
         if (b1 != a2) {  // anti-diagonal (r,c+1)-(r+1,c)
           int eX = 0;
-          pair_step_fused<R, D, Dc>(false, E, X1, Muc, tptr(a, i1, a1), tptr(a, i2, b1), Mdc, nullptr, sm, red, &eX);
-          const R wp = pair_step_fused<R, D, Dc>(false, X1, nullptr, Mun, tptr(a, j1, a2), tptr(a, j2, b2), Mdn,
+          pair_step_fused<R, D, Dc>(false, nb(c), E, X1, Muc, tptr(a, i1, a1), tptr(a, i2, b1), Mdc, nullptr, sm, red, &eX);
+          const R wp = pair_step_fused<R, D, Dc>(false, nb(c + 1), X1, nullptr, Mun, tptr(a, j1, a2), tptr(a, j2, b2), Mdn,
                                                  Hb + (size_t)(c + 2) * envT2, sm, red);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
       }
       if (c < Lx - 1) {
         int e1 = 0;
-        pair_step_fused<R, D, Dc>(false, E, En, Muc, tptr(a, i1, a1), tptr(a, i2, a2), Mdc, nullptr, sm, red, &e1);
+        pair_step_fused<R, D, Dc>(false, nb(c), E, En, Muc, tptr(a, i1, a1), tptr(a, i2, a2), Mdc, nullptr, sm, red, &e1);
         eE += e1;
         E = En;
         En = (En == E0) ? E1 : E0;
@@ -280,11 +286,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_pair_tc(KArgs<float> a) {
     __syncthreads();
     const float* Mu = r == 0 ? a.triv_mps : a.envU + ((size_t)cfg * Ly + (r - 1)) * Lx * envT;
     const float* Md = r + 2 > Ly - 1 ? a.triv_mps : a.envL + ((size_t)cfg * Ly + (r + 2)) * Lx * envT;
+    // true bonds of L_{r+2}, by column boundary
+    const int* bl = r + 2 > Ly - 1 ? nullptr : a.bd + (size_t)(Ly + Ly - 3 - r) * (Lx + 1);
+    auto nb = [&](int c) { return bl ? bl[c] : 1; };
     int eacc = 0;
     for (int c = Lx - 1; c >= 0; --c) {
       const int s1 = r * Lx + c, s2 = (r + 1) * Lx + c;
       int e = 0;
-      pair_step_tc(st, true, Hb + (size_t)(c + 1) * envT2, Hb + (size_t)c * envT2, Mu + (size_t)c * envT,
+      pair_step_tc(st, true, nb(c + 1), Hb + (size_t)(c + 1) * envT2, Hb + (size_t)c * envT2, Mu + (size_t)c * envT,
                    tile(1, s1, spin_of(sp, s1)), tile(1, s2, spin_of(sp, s2)) + kTcTile, Md + (size_t)c * envT,
                    nullptr, sm, red, &e);
       eacc += e;
@@ -303,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_pair_tc(KArgs<float> a) {
       const float* Muc = Mu + (size_t)c * envT;
       const float* Mdc = Md + (size_t)c * envT;
       if (a1 != a2) {
-        const float wp = pair_step_tc(st, false, E, nullptr, Muc, tile(0, i1, a2), tile(0, i2, a1) + kTcTile, Mdc,
+        const float wp = pair_step_tc(st, false, nb(c), E, nullptr, Muc, tile(0, i1, a2), tile(0, i2, a1) + kTcTile, Mdc,
                                       Hb + (size_t)(c + 1) * envT2, sm, red);
         if (ok) ev += 0.5 * g.J1 * ldexp((double)wp / (double)W, eE + eH[c + 1] - eH[0]);
       }
@@ -314,26 +323,26 @@ __global__ void __launch_bounds__(kThreads, 2) k_pair_tc(KArgs<float> a) {
         const float* Mdn = Md + (size_t)(c + 1) * envT;
         if (a1 != b2) {
           int eX = 0;
-          pair_step_tc(st, false, E, X1, Muc, tile(0, i1, b2), tile(0, i2, a2) + kTcTile, Mdc, nullptr, sm, red,
+          pair_step_tc(st, false, nb(c), E, X1, Muc, tile(0, i1, b2), tile(0, i2, a2) + kTcTile, Mdc, nullptr, sm, red,
                        &eX);
           __syncthreads();
-          const float wp = pair_step_tc(st, false, X1, nullptr, Mun, tile(0, j1, b1), tile(0, j2, a1) + kTcTile, Mdn,
+          const float wp = pair_step_tc(st, false, nb(c + 1), X1, nullptr, Mun, tile(0, j1, b1), tile(0, j2, a1) + kTcTile, Mdn,
                                         Hb + (size_t)(c + 2) * envT2, sm, red);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
         if (b1 != a2) {
           int eX = 0;
-          pair_step_tc(st, false, E, X1, Muc, tile(0, i1, a1), tile(0, i2, b1) + kTcTile, Mdc, nullptr, sm, red,
+          pair_step_tc(st, false, nb(c), E, X1, Muc, tile(0, i1, a1), tile(0, i2, b1) + kTcTile, Mdc, nullptr, sm, red,
                        &eX);
           __syncthreads();
-          const float wp = pair_step_tc(st, false, X1, nullptr, Mun, tile(0, j1, a2), tile(0, j2, b2) + kTcTile, Mdn,
+          const float wp = pair_step_tc(st, false, nb(c + 1), X1, nullptr, Mun, tile(0, j1, a2), tile(0, j2, b2) + kTcTile, Mdn,
                                         Hb + (size_t)(c + 2) * envT2, sm, red);
           if (ok) ev += 0.5 * g.J2 * ldexp((double)wp / (double)W, eE + eX + eH[c + 2] - eH[0]);
         }
       }
       if (c < Lx - 1) {
         int e1 = 0;
-        pair_step_tc(st, false, E, En, Muc, tile(0, i1, a1), tile(0, i2, a2) + kTcTile, Mdc, nullptr, sm, red, &e1);
+        pair_step_tc(st, false, nb(c), E, En, Muc, tile(0, i1, a1), tile(0, i2, a2) + kTcTile, Mdc, nullptr, sm, red, &e1);
         __syncthreads();
         eE += e1;
         E = En;

@@ -142,9 +142,10 @@ __device__ __forceinline__ void smem_gemm_km_x2(const R* __restrict__ A0, const 
 // tensors of rows r, r+1 at the chosen spins.  If Hdot is null the result is
 // written to Eout scaled by 2^-e (pow2_exponent of its largest entry) and e
 // is stored in *e_out; otherwise <result, Hdot> is returned (all threads) and
-// nothing is written.  Ends with a barrier.
+// nothing is written.  ns: the true dimension of L's in-bond (slices past it
+// are zero).  Ends with a barrier.
 template <typename R, int D, int Dc>
-__device__ R pair_step_fused(bool right, const R* Ein, R* __restrict__ Eout, const R* __restrict__ Mu,
+__device__ R pair_step_fused(bool right, int ns, const R* Ein, R* __restrict__ Eout, const R* __restrict__ Mu,
                              const R* __restrict__ T1, const R* __restrict__ T2, const R* __restrict__ Md,
                              const R* Hdot, R* sm, R* red, int* e_out = nullptr) {
   using S = PairSmem<D, Dc>;
@@ -177,7 +178,7 @@ __device__ R pair_step_fused(bool right, const R* Ein, R* __restrict__ Eout, con
   for (int q = 0; q < S::RPT; ++q)
 #pragma unroll
     for (int x = 0; x < Dc; ++x) acc[q][x] = R(0);
-  for (int s = 0; s < Dc; ++s) {
+  for (int s = 0; s < ns; ++s) {
     // slice s of the input transfer ([x'][x][y1][y2] is slice-contiguous) and of Md
     for (int e = tid; e < S::ES; e += kThreads) Es[e] = Ein[s * S::ES + e];
     for (int e = tid; e < S::MD; e += kThreads) {

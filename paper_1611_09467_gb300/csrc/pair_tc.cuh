@@ -173,8 +173,10 @@ __device__ __forceinline__ void st4(float* p, float a, float b, float c, float d
 // One two-row transfer step, D = 8, Dc = 16, TF32 tensor cores.  Arguments
 // as pair_step_fused, plus the pre-arranged B tiles of T1 (TA) and T2 (TB).
 // Returns <result, Hdot> when Hdot is given; otherwise writes the result
-// scaled by 2^-e to Eout and stores e in *e_out, as pair_step_fused.
-static __device__ float pair_step_tc(PairTc& st, bool right, const float* Ein, float* __restrict__ Eout,
+// scaled by 2^-e to Eout and stores e in *e_out, as pair_step_fused.  ns: the
+// true dimension of L's in-bond; the slices past it are zero and left out (a
+// sixth of all slices at 16x16 D = 8).
+static __device__ float pair_step_tc(PairTc& st, bool right, int ns, const float* Ein, float* __restrict__ Eout,
                               const float* __restrict__ Mu, const float* __restrict__ TA1,
                               const float* __restrict__ TB2, const float* __restrict__ Md,
                               const float* Hdot, float* sm, float* red, int* e_out = nullptr) {
@@ -247,14 +249,14 @@ static __device__ float pair_step_tc(PairTc& st, bool right, const float* Ein, f
   };
   float pe[4], pm[4] = {0.f, 0.f, 0.f, 0.f};
   load_slice(0, pe, pm);
-  for (int s = 0; s < Dc; ++s) {
+  for (int s = 0; s < ns; ++s) {
     // ---- B1 = Ein slice as [n = (y1i, y2i)][k = xi]; B4 = Md slice as [x'o][d2]
     st4(B1 + tc::kmaj(bn, bxq, 16), tc::to_tf32(pe[0]), tc::to_tf32(pe[1]), tc::to_tf32(pe[2]),
         tc::to_tf32(pe[3]));
     if (tid < 32)
       st4(B4 + tc::kmaj(mxo, mdq, 8), tc::to_tf32(pm[0]), tc::to_tf32(pm[1]), tc::to_tf32(pm[2]),
           tc::to_tf32(pm[3]));
-    if (s + 1 < Dc) load_slice(s + 1, pe, pm);
+    if (s + 1 < ns) load_slice(s + 1, pe, pm);
     tc::fence_async_smem();
     tc::tc_fence_before();
     __syncthreads();

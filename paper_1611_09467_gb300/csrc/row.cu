@@ -154,11 +154,14 @@ __global__ void __launch_bounds__(kThreads) k_row_fused(KArgs<R> a) {
     __syncthreads();
     const R* Mu = r == 0 ? a.triv_mps : a.envU + ((size_t)cfg * Ly + (r - 1)) * Lx * envT;
     const R* Md = r == Ly - 1 ? a.triv_mps : a.envL + ((size_t)cfg * Ly + (r + 1)) * Lx * envT;
+    // true bonds of L_{r+1}, by column boundary
+    const int* bl = r == Ly - 1 ? nullptr : a.bd + (size_t)(Ly + Ly - 2 - r) * (Lx + 1);
+    auto nb = [&](int c) { return bl ? bl[c] : 1; };
     int eacc = 0;
     for (int c = Lx - 1; c >= 0; --c) {
       const int site = r * Lx + c;
       int e = 0;
-      row_step_fused<R, D, Dc>(true, Gb + (size_t)(c + 1) * envT, Gb + (size_t)c * envT, Mu + (size_t)c * envT,
+      row_step_fused<R, D, Dc>(true, nb(c + 1), Gb + (size_t)(c + 1) * envT, Gb + (size_t)c * envT, Mu + (size_t)c * envT,
                                tptr(a, site, spin_of(sp, site)), Md + (size_t)c * envT, nullptr, sm, red, &e);
       eacc += e;
       if (threadIdx.x == 0) eG[c] = eacc;
@@ -175,20 +178,20 @@ __global__ void __launch_bounds__(kThreads) k_row_fused(KArgs<R> a) {
       const R* Muc = Mu + (size_t)c * envT;
       const R* Mdc = Md + (size_t)c * envT;
       if (a.O != nullptr)
-        site_env_fused<R, D, Dc>(F, Muc, Mdc, Gb + (size_t)(c + 1) * envT,
+        site_env_fused<R, D, Dc>(nb(c), F, Muc, Mdc, Gb + (size_t)(c + 1) * envT,
                                  ok ? (R)ldexp(1.0 / (double)W, eF + eG[c + 1] - eG[0]) : R(0),
                                  a.O + ((size_t)cfg * g.N + site) * D4, sm);
       if (c < Lx - 1) {
         const int s2 = spin_of(sp, site + 1);
         if (s != s2) {
           int eX = 0;
-          row_step_fused<R, D, Dc>(false, F, X1, Muc, tptr(a, site, s2), Mdc, nullptr, sm, red, &eX);
-          const R wp = row_step_fused<R, D, Dc>(false, X1, nullptr, Mu + (size_t)(c + 1) * envT, tptr(a, site + 1, s),
+          row_step_fused<R, D, Dc>(false, nb(c), F, X1, Muc, tptr(a, site, s2), Mdc, nullptr, sm, red, &eX);
+          const R wp = row_step_fused<R, D, Dc>(false, nb(c + 1), X1, nullptr, Mu + (size_t)(c + 1) * envT, tptr(a, site + 1, s),
                                                 Md + (size_t)(c + 1) * envT, Gb + (size_t)(c + 2) * envT, sm, red);
           if (ok) eh += 0.5 * g.J1 * ldexp((double)wp / (double)W, eF + eX + eG[c + 2] - eG[0]);
         }
         int e1 = 0;
-        row_step_fused<R, D, Dc>(false, F, Fn, Muc, tptr(a, site, s), Mdc, nullptr, sm, red, &e1);
+        row_step_fused<R, D, Dc>(false, nb(c), F, Fn, Muc, tptr(a, site, s), Mdc, nullptr, sm, red, &e1);
         eF += e1;
         F = Fn;
         Fn = (Fn == F0) ? F1 : F0;

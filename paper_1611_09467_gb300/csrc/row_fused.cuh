@@ -54,9 +54,11 @@ struct RowSmem {
 // If Gdot is null the result is written to Fout scaled by 2^-e
 // (pow2_exponent of its largest entry) and e is stored in *e_out; otherwise
 // <result, Gdot> is returned (all threads) and nothing is written.  Ends with
-// a barrier.
+// a barrier.  ns: the true dimension of L's in-bond; slices past it are zero
+// and left out (at 10x10 the edge columns and the rows next to the border have
+// bonds of 1 and D, a fifth of all slices), which changes no sum.
 template <typename R, int D, int Dc>
-__device__ R row_step_fused(bool right, const R* Fin, R* __restrict__ Fout, const R* __restrict__ Mu,
+__device__ R row_step_fused(bool right, int ns, const R* Fin, R* __restrict__ Fout, const R* __restrict__ Mu,
                             const R* __restrict__ T, const R* __restrict__ Md, const R* Gdot, R* sm,
                             R* red, int* e_out = nullptr) {
   using S = RowSmem<D, Dc>;
@@ -92,7 +94,7 @@ __device__ R row_step_fused(bool right, const R* Fin, R* __restrict__ Fout, cons
   for (int q = 0; q < S::OPT; ++q) acc[q] = R(0);
   // three barriers per pair of slices: the slice buffers of consecutive pairs
   // alternate, so loading pair p+1 cannot overwrite what s3 of pair p reads
-  for (int s0 = 0; s0 < Dc; s0 += 2) {
+  for (int s0 = 0; s0 < ns; s0 += 2) {
     const int par = (s0 >> 1) & 1;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -187,9 +189,9 @@ __device__ R row_step_fused(bool right, const R* Fin, R* __restrict__ Fout, cons
 
 // Site environment of column c, scaled: Bout[l][r][u][d] = scale * B, from
 // F_{c-1} ([a'][a][l]), Mu, Md (padded [Dc][D][Dc]) and G_{c+1} ([b'][b][r]).
-// Ends with a barrier.
+// ns: the true dimension of the bond a'.  Ends with a barrier.
 template <typename R, int D, int Dc>
-__device__ void site_env_fused(const R* F, const R* __restrict__ Mu, const R* __restrict__ Md,
+__device__ void site_env_fused(int ns, const R* F, const R* __restrict__ Mu, const R* __restrict__ Md,
                                const R* G, R scale, R* __restrict__ Bout, R* sm) {
   using S = RowSmem<D, Dc>;
   constexpr int DD = S::DD, D3 = S::D3, XY = Dc * D, TM = S::TM;
@@ -211,7 +213,7 @@ __device__ void site_env_fused(const R* F, const R* __restrict__ Mu, const R* __
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[t][i][j] = R(0);
   // three barriers per pair of slices of a'
-  for (int s0 = 0; s0 < Dc; s0 += 2) {
+  for (int s0 = 0; s0 < ns; s0 += 2) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int s = s0 + h;

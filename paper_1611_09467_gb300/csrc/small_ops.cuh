@@ -33,7 +33,7 @@ struct CtaOps {
   __device__ void col1(bool right, const R* F, const R* Mu, const R* T, const R* Md, R* out) {
     run_op<R>(right ? OP_COL1_RIGHT : OP_COL1_LEFT, a.g.D, a.g.Dc, F, Mu, T, Md, nullptr, out, t0, t1, zb.gsm, zb.gism);
   }
-  __device__ void col2(bool right, const R* E, const R* Mu, const R* T1, const R* T2, const R* Md, R* out) {
+  __device__ void col2(bool right, int, const R* E, const R* Mu, const R* T1, const R* T2, const R* Md, R* out) {
     run_op<R>(right ? OP_COL2_RIGHT : OP_COL2_LEFT, a.g.D, a.g.Dc, E, Mu, T1, T2, Md, out, t0, t1, zb.gsm, zb.gism);
   }
   __device__ void site_env(const R* F, const R* Mu, const R* Md, const R* G, R* out) {
@@ -201,7 +201,9 @@ struct WarpOps {
       small::desc_gemm<R>(g, s == 1 ? t0 : t1, s == 1 ? t : d, s == 1 ? t1 : out);
     }
   }
-  __device__ __noinline__ void col2(bool right, const R* E, const R* Mu, const R* T1, const R* T2, const R* Md, R* out) {
+  // nx: the true dimension of U's out-bond; slices past it are zero
+  __device__ __noinline__ void col2(bool right, int nx, const R* E, const R* Mu, const R* T1, const R* T2, const R* Md,
+                                    R* out) {
     const int D = a.g.D, Dc = a.g.Dc, DD = D * D, envT = Dc * D * Dc;
     __syncwarp();
     R* p = sm;
@@ -214,7 +216,8 @@ struct WarpOps {
     R* x1 = x0 + small::up4(Dc * D * (DD + 1));
     R* x2 = x1 + small::up4(Dc * D * (DD + 1));
     __syncwarp();
-    for (int x = 0; x < Dc; ++x)
+    for (int k = nx * DD * Dc + small::lane_id(); k < Dc * DD * Dc; k += 32) out[k] = R(0);
+    for (int x = 0; x < nx; ++x)
       for (int s = 0; s < 4; ++s) {
         const GemmDesc g = right ? small::right2_slice(s, D, Dc) : small::left2_slice(s, D, Dc);
         const R* A = s == 0 ? e : (s == 1 ? x0 : (s == 2 ? x1 : x2));
