@@ -229,32 +229,37 @@ struct ZipDims {
   int k, a, b, i, l, r, o;
 };
 
+// Y is stored with the second step's reduction index first, so that the rows
+// that step stages are contiguous (row-major rows of D^2 reals cost a memory
+// line per lane).
 // Left-to-right, column c:
-//   s0: Y[k][b][l][i] = sum_a C[k][a][l] M[a][i][b]
-//   s1: X[(k,o)][(b,r)] = sum_{l,i} Y[k][b][l][i] T[l][r][i][o]
+//   s0: Y[l][i][k][b] = sum_a C[k][a][l] M[a][i][b]
+//   s1: X[(k,o)][(b,r)] = sum_{l,i} Y[l][i][k][b] T[l][r][i][o]
 PEPS_HD GemmDesc zip_lr_step(int s, const ZipDims& z, int D, int Dc, int sl, int sr, int si, int so) {
+  const int kb = z.k * z.b;
   if (s == 0)
     return gemm(z.k * z.l, z.i * z.b, z.a,
                 ix2(z.l, z.a * z.l, 1), kx(z.a, 0, z.l),         // A = C[k][a][l]: rows (k,l)
                 kx(z.a, 0, D * Dc), ix2(z.b, Dc, 1),             // B = M[a][i][b]: cols (i,b)
-                ix2(z.l, z.b * z.l * z.i, z.i), ix2(z.b, 1, z.l * z.i));  // C = Y[k][b][l][i]
-  return gemm(z.k * z.b, z.r * z.o, z.l * z.i,
-              ix1(z.l * z.i), kx(z.i, z.i, 1),                   // A = Y: rows (k,b), k = (l,i)
+                ix2(z.l, z.b, z.i * kb), ix2(z.b, kb, 1));       // C = Y[l][i][k][b]
+  return gemm(kb, z.r * z.o, z.l * z.i,
+              ix1(1), kx(z.i, z.i * kb, kb),                     // A = Y: rows (k,b), k = (l,i)
               kx(z.i, sl, si), ix2(z.o, sr, so),                 // B = T: k = (l,i), cols (r,o)
               ix2(z.b, z.o * z.b * z.r, z.r), ix2(z.o, 1, z.b * z.r));  // C = X[(k,o)][(b,r)]
 }
 
 // Right-to-left, column c (carry C[b][r][k] comes from the right):
-//   s0: Y[a][k][i][r] = sum_b M[a][i][b] C[b][r][k]
-//   s1: X[(o,k)][(a,l)] = sum_{i,r} Y[a][k][i][r] T[l][r][i][o]
+//   s0: Y[i][r][a][k] = sum_b M[a][i][b] C[b][r][k]
+//   s1: X[(o,k)][(a,l)] = sum_{i,r} Y[i][r][a][k] T[l][r][i][o]
 PEPS_HD GemmDesc zip_rl_step(int s, const ZipDims& z, int D, int Dc, int sl, int sr, int si, int so) {
+  const int ak = z.a * z.k;
   if (s == 0)
     return gemm(z.a * z.i, z.r * z.k, z.b,
                 ix2(z.i, D * Dc, Dc), kx(z.b, 0, 1),             // A = M[a][i][b]: rows (a,i), k = b
                 kx(z.b, 0, z.r * z.k), ix1(1),                   // B = C[b][r][k]: cols (r,k)
-                ix2(z.i, z.k * z.i * z.r, z.r), ix2(z.k, 1, z.i * z.r));  // C = Y[a][k][i][r]
-  return gemm(z.a * z.k, z.l * z.o, z.i * z.r,
-              ix1(z.i * z.r), kx(z.r, z.r, 1),                   // A = Y: rows (a,k), k = (i,r)
+                ix2(z.i, z.k, z.r * ak), ix2(z.k, ak, 1));       // C = Y[i][r][a][k]
+  return gemm(ak, z.l * z.o, z.i * z.r,
+              ix1(1), kx(z.r, z.r * ak, ak),                     // A = Y: rows (a,k), k = (i,r)
               kx(z.r, si, sr), ix2(z.o, sl, so),                 // B = T: k = (i,r), cols (l,o)
               ix2(z.k, z.l, z.a * z.l), ix2(z.o, 1, z.k * z.a * z.l));  // C = X[(o,k)][(a,l)]
 }

@@ -70,6 +70,19 @@ __device__ __forceinline__ void dot2_step(float a, float b, float& s, float& c) 
   c = __fadd_rn(c, __fadd_rn(pe, se));
 }
 
+// Two of them at once in packed FP32x2 instructions: nine for two terms.  A
+// difference is the product with -1 fused into the sum, which rounds once.
+__device__ __forceinline__ void dot2_step2(float2 a, float2 b, float2& s, float2& c) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 p = __fmul2_rn(a, b);
+  const float2 pe = __ffma2_rn(a, b, __fmul2_rn(p, m1));
+  const float2 t = __fadd2_rn(s, p);
+  const float2 z = __ffma2_rn(s, m1, t);
+  const float2 se = __fadd2_rn(__ffma2_rn(__ffma2_rn(z, m1, t), m1, s), __ffma2_rn(z, m1, p));
+  s = t;
+  c = __fadd2_rn(c, __fadd2_rn(pe, se));
+}
+
 template <typename R>
 __device__ __forceinline__ R warp_sum(R v, int width = 32) {
   for (int o = width / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, width);
@@ -605,6 +618,7 @@ struct TruncWork {
   int* gism;
   int Qmax;
   int Kmax;        // Ubs and Uks hold Qmax x Kmax
+  int gsm_reals;   // size of the shared region
   int wm_shared;   // Wm is in shared memory
 };
 
@@ -741,8 +755,8 @@ static __device__ __noinline__ void section_f32(const float* t2, int n2, int K, 
 // row i of vector k at group i * K + k, and the interchange flag is the top
 // exponent bit of the multiplier (|l| <= 1 leaves it free).  The passes over
 // stored rows read them a block of four ahead, since the stores in between keep
-// the compiler from doing so.  FP32 has two approximate divisions per row; FP64
-// one (the multiplier is formed from the pivot's reciprocal).  The second
+// the compiler from doing so.  A row takes one reciprocal: of the pivot, for the
+// multiplier as well.  The second
 // super-diagonal of U is t[i+1] where rows i, i+1 were interchanged and zero
 // otherwise, so it is not stored.  The iterate is left in the fourth entries.
 template <typename R>
@@ -775,14 +789,6 @@ __device__ __forceinline__ bool flag_get(double x) { return __double2hiint(x) & 
 __device__ __forceinline__ float flag_clear(float x) { return __uint_as_float(__float_as_uint(x) & ~0x40000000u); }
 __device__ __forceinline__ double flag_clear(double x) {
   return __hiloint2double(__double2hiint(x) & ~0x40000000, __double2loint(x));
-}
-// num / d as __fdividef computes it for normal d below 2^126: the product with
-// the hardware reciprocal, without its scaling steps.
-__device__ __forceinline__ float quick_div(float num, float d) {
-  if (fabsf(d) < 1.17549435e-38f) return __fdividef(num, d);
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-  return __fmul_rn(num, r);
 }
 // Comparisons of magnitudes, start values and scales of the inverse iteration.
 // FP64 does them on the bits: an FP64 instruction, a comparison too, keeps its
@@ -841,6 +847,7 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
   R cur_d = -lam, cur_u = n2 > 1 ? t[0] : R(0);
   R bi = start();
   R sub = cur_u;
+  const R few = fmax(pivtiny, R(1.17549435e-38));
   R* w = w0;
 #pragma unroll 2
   for (int i = 0; i < n2 - 1; ++i, w += st) {
@@ -852,9 +859,14 @@ static __device__ __noinline__ R inverse_iteration(const R* t, int n2, R lam, R 
     const R num = sw ? cur_d : sub;
     R lm, rd;
     if constexpr (sizeof(R) == 4) {
-      lm = quick_div(num, d);
-      if (fabs(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
-      rd = quick_div(1.f, d);
+      if (fabsf(d) < few) {   // tiny pivots: the divisions as __fdividef takes them
+        lm = __fdividef(num, d);
+        if (fabsf(d) < pivtiny) d = d < R(0) ? -pivtiny : pivtiny;
+        rd = __fdividef(1.f, d);
+      } else {                // one hardware reciprocal gives both
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"(d));
+        lm = __fmul_rn(num, rd);
+      }
     } else {
       if (!abs_ge(d, pivtiny)) d = with_sign(pivtiny, d);
       rd = quick_rcp(d);
@@ -1020,18 +1032,32 @@ static __device__ __noinline__ void bidiag_tiles_f32(const float* X, int n, bool
   const int r0 = ti * 8, c0 = tj * 8;
   const unsigned hmask = (lane & 16) ? 0xffff0000u : 0x0000ffffu;
   float2 a[8][4];   // a[r][q] = columns (2q, 2q+1) of row r of the tile
+  if (tall && (n & 3) == 0 && (reinterpret_cast<size_t>(X) & 15) == 0) {
+    // whole groups of four columns: a quarter of the memory lines per load
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = r0 + r, c = c0 + 2 * q;
-      float x0 = 0.f, x1 = 0.f;
-      if (i < P) {
-        if (c < Q) x0 = tall ? X[i * n + c] : X[c * n + i];
-        if (c + 1 < Q) x1 = tall ? X[i * n + c + 1] : X[(c + 1) * n + i];
+      for (int q = 0; q < 4; q += 2) {
+        const int i = r0 + r, c = c0 + 2 * q;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < P && c < Q) v = *reinterpret_cast<const float4*>(X + i * n + c);
+        a[r][q] = make_float2(v.x, v.y);
+        a[r][q + 1] = make_float2(v.z, v.w);
       }
-      a[r][q] = make_float2(x0, x1);
-    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = r0 + r, c = c0 + 2 * q;
+        float x0 = 0.f, x1 = 0.f;
+        if (i < P) {
+          if (c < Q) x0 = tall ? X[i * n + c] : X[c * n + i];
+          if (c + 1 < Q) x1 = tall ? X[i * n + c + 1] : X[(c + 1) * n + i];
+        }
+        a[r][q] = make_float2(x0, x1);
+      }
+  }
   for (int jb = 0; jb < Q; jb += 8) {
     const int tb = jb >> 3;   // tile row / column of j
 #pragma unroll 1
@@ -1535,112 +1561,14 @@ static __device__ __noinline__ void gram_schmidt(R* Ub, int Q, int K, R* red) {
   }
 }
 
-// Writes U_K (m x K) through (uo_r, uo_c) and C' = U_K^T X (K x n) through
-// (co_r, co_c).  X is not modified.  K <= min(m, n), K <= 32.
+// CholeskyQR2 of the columns of Ub (Q x K) in place; G: K x K.  Returns true where
+// a direction is too small (the caller then takes Gram-Schmidt).
 template <typename R>
-__device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, R* Uout, Ix uo_r,
-                              Ix uo_c, R* Cout, Ix co_r, Ix co_c) {
+static __device__ __noinline__ bool cholesky_qr2(R* Ub, R* G, int Q, int K) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (K == m) {
-    // Nothing is cut: any orthonormal basis of R^m works; take the identity.
-    for (int e = tid; e < m * m; e += blockDim.x) {
-      const int i = e / m, k = e % m;
-      Uout[ixoff(uo_r, i) + ixoff(uo_c, k)] = i == k ? R(1) : R(0);
-    }
-    for (int e = tid; e < m * n; e += blockDim.x) {
-      const int k = e / n, j = e % n;
-      Cout[ixoff(co_r, k) + ixoff(co_c, j)] = X[e];
-    }
-    __syncthreads();
-    return;
-  }
-  PEPS_PHASE(0);
-  const bool tall = m >= n;
-  const int P = tall ? m : n, Q = tall ? n : m;
-  const int ld = w.ldw;
-  R* W = w.Wm;
-  R* tauL = w.tau;
-  R* tauR = w.tau + w.Qmax;
-  R* red = w.red;
-  bool tiled = false;
-  if constexpr (sizeof(R) == 4) {
-    if (P > 32 && P <= 128) {   // below 33 rows the shared-memory version is as fast
-      // the reflectors go to global memory: shared memory then holds the
-      // inverse-iteration workspace
-      W = w.Wg;
-      bidiag_tiles_f32(X, n, tall, P, Q, W, ld, w.t, w.tau, w.Qmax);
-      tiled = true;
-    }
-  }
-  if (!tiled) bidiag_shared<R>(X, m, n, tall, P, Q, W, ld, w.t, w.tau, w.Qmax, w.wv, red);
-  PEPS_PHASE(1);
-  // ---------------- Sturm sections for the K largest singular values
-  const int n2 = 2 * Q;
-  R tmax = R(0);
-  for (int i = tid; i < n2 - 1; i += blockDim.x) tmax = fmax(tmax, fabs(w.t[i]));
-  tmax = warp_max(tmax);
-  if (lane == 0) red[8 + warp] = tmax;
-  __syncthreads();
-  tmax = R(0);
-  for (int i = 0; i < kWarps; ++i) tmax = fmax(tmax, red[8 + i]);
-  if constexpr (sizeof(R) == 4) {
-    // the squares in shared memory (wv is free here) where they fit
-    R* t2 = n2 <= kMaxT2Shared ? w.wv : w.t2;
-    for (int i = tid; i < n2 - 1; i += blockDim.x) t2[i] = w.t[i] * w.t[i];
-    __syncthreads();
-    const R bound = R(2) * tmax * (R(1) + R(4) * Eps<R>::eps) + Eps<R>::tiny;
-    const R pivmin = Eps<R>::tiny * R(1024) * fmax(R(1), tmax * tmax);
-    section_f32(t2, n2, K, bound, pivmin, w.lam);
-  } else {
-    const int e2 = pow2_exponent(tmax);
-    const R down = pow2<R>(-e2);
-    float* t2f = reinterpret_cast<float*>(w.wv);       // >= 512 floats
-    float* lamf = reinterpret_cast<float*>(red + 24);
-    for (int i = tid; i < n2 - 1; i += blockDim.x) {
-      const R v = w.t[i] * down;
-      w.t2[i] = v * v;
-      t2f[i] = (float)(v * v);
-    }
-    __syncthreads();
-    section_f32(t2f, n2, K, 4.001f, Eps<float>::tiny * 4096.f, lamf);
-    __syncthreads();
-    if (warp < 4) refine_values_f64(tid, K <= 8 ? 16 : K <= 16 ? 8 : 4, w.t2, n2, K, lamf, pow2<R>(e2), w.lam);
-  }
-  __syncthreads();
-  PEPS_PHASE(2);
-  // ---------------- inverse iteration, one thread per vector
-  const R pivtiny = Eps<R>::eps * fmax(tmax, Eps<R>::tiny * R(1e10));
-  R* Ub = w.Ubs;
-  {
-    // in shared memory (the matrix buffer, free on the register-tiled path)
-    // when it fits; t in the Ub buffer
-    const bool in_smem = tiled && (size_t)4 * n2 * K <= (size_t)w.Qmax * w.ldw;
-    R* wsR = in_smem ? w.Wm : inv_align(w.lu);
-    const R* tv = w.t;
-    if (n2 <= w.Qmax * w.Kmax) {
-      for (int i = tid; i < n2 - 1; i += blockDim.x) Ub[i] = w.t[i];
-      tv = Ub;
-    }
-    __syncthreads();
-    if (tid < K) red[tid] = inverse_iteration(tv, n2, w.lam[tid], pivtiny, wsR, K, tid, (unsigned)(tid + 1));
-    __syncthreads();
-    PEPS_PHASE(3);
-    // u-parts (odd positions) for a tall matrix, v-parts (even) for a wide one, scaled
-    for (int e = tid; e < Q * K; e += blockDim.x) {
-      const int i = e / K, k = e % K;
-      Ub[e] = wsR[((2 * i + (tall ? 1 : 0)) * K + k) * 4 + 3] * red[k];
-    }
-  }
-  __syncthreads();
-  // ---------------- orthonormal basis of the kept vectors: CholeskyQR2
-  // (G = Ub^T Ub = R^T R, Ub <- Ub R^-1, twice; Fukaya et al. 2014).  Each
-  // pass costs three barriers.  If a direction of Ub is below 1e-3 of its
-  // norm (a cluster or a zero singular value), Gram-Schmidt with replacement
-  // of degenerate directions (below) takes over from the current Ub.
   bool need_cgs = false;
   {
     __shared__ int cq_bad;
-    R* G = w.Uks;   // K x K, free until the back-transformation
     for (int pass = 0; pass < 2 && !need_cgs; ++pass) {
       for (int e = tid; e < K * K; e += blockDim.x) {
         const int a = e / K, b = e % K;
@@ -1720,6 +1648,239 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
       __syncthreads();
     }
   }
+  return need_cgs;
+}
+
+static __device__ __forceinline__ void apply_all_reflectors(const float* Wf, int ld, bool tall, int rowsU, int nref, int K,
+                                                         const float* tf, const float* sf, float* Uk) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int c = warp * 2 + (lane >> 4), l = lane & 15;
+        float u[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int i = l + 16 * r;
+          u[r] = (c < K && i < rowsU) ? Uk[i * K + c] : 0.f;
+        }
+        int j = nref - 1;
+        const int off = tall ? 0 : 1;   // first row of reflector j: j + off
+        j = apply_reflectors<7>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<6>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<5>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<4>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<3>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<2>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        j = apply_reflectors<1>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        apply_reflectors<0>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
+        if (c < K) {
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const int i = l + 16 * r;
+            if (i < rowsU) Uk[i * K + c] = u[r];
+          }
+        }
+}
+
+// The FP32 end of a cut: one Newton-Schulz step on U (m x K in shared memory,
+// Uk), U to Uout, the carry U^T X to Cout (see the caller).  Mns: K x K; Ug: a global copy of U.
+static __device__ __forceinline__ void finish_f32(const float* X, int m, int n, int K, float* Mns, float* Uk, float* Ug,
+                                               float* Uout, Ix uo_r, Ix uo_c, float* Cout, Ix co_r, Ix co_c) {
+    const int tid = threadIdx.x;
+    const float* Uf = Uk;
+    for (int e = tid; e < K * K; e += blockDim.x) {
+      const int a = e / K, b = e % K;
+      float s = 0.f, c = 0.f;
+      for (int i = 0; i < m; ++i) dot2_step(Uf[i * K + a], Uf[i * K + b], s, c);
+      // s is within a factor 2 of 1 on the diagonal, so s - 1 is exact
+      Mns[e] = -0.5f * (a == b ? __fadd_rn(__fsub_rn(s, 1.f), c) : __fadd_rn(s, c));
+    }
+    __syncthreads();
+    // Up to kNsPer entries per thread, the new U replaces the old one in
+    // shared memory once every thread has read the old one; larger U go to
+    // the global copy.
+    constexpr int kNsPer = 8;
+    const bool u_shared = m * K <= kNsPer * kThreads;
+    float* Us = Uk;
+    if (u_shared) {
+      float nv[kNsPer];
+#pragma unroll
+      for (int q = 0; q < kNsPer; ++q) {
+        const int e = tid + q * kThreads;
+        if (e < m * K) {
+          const int i = e / K, k = e % K;
+          float corr = 0.f;
+          for (int a = 0; a < K; ++a) corr = fmaf(Uf[i * K + a], Mns[a * K + k], corr);
+          nv[q] = Uf[i * K + k] + corr;
+          Uout[ixoff(uo_r, i) + ixoff(uo_c, k)] = nv[q];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < kNsPer; ++q) {
+        const int e = tid + q * kThreads;
+        if (e < m * K) Us[e] = nv[q];
+      }
+    } else {
+      for (int e = tid; e < m * K; e += blockDim.x) {
+        const int i = e / K, k = e % K;
+        float corr = 0.f;
+        for (int a = 0; a < K; ++a) corr = fmaf(Uf[i * K + a], Mns[a * K + k], corr);
+        const float v = Uf[i * K + k] + corr;
+        Uout[ixoff(uo_r, i) + ixoff(uo_c, k)] = v;
+        Ug[e] = v;
+      }
+    }
+    __syncthreads();
+    // C' = U_K^T X, X row-major m x n.  One work item is a column j and a
+    // chunk of 8 rows of C'; its X column is read once (coalesced over j),
+    // eight rows at a time so that eight loads are in flight together.
+    constexpr int CH = 8, XB = 8;
+    const float* Uo = u_shared ? Us : Ug;
+    const float* Xf = X;
+    const int nchunk = (K + CH - 1) / CH;
+    for (int item = tid; item < n * nchunk; item += blockDim.x) {
+      const int j = item % n, a0 = (item / n) * CH;
+      float s[CH], c[CH];
+#pragma unroll
+      for (int q = 0; q < CH; ++q) s[q] = c[q] = 0.f;
+      for (int ib = 0; ib < m; ib += XB) {
+        float xb[XB];
+#pragma unroll
+        for (int u = 0; u < XB; ++u) xb[u] = ib + u < m ? Xf[(ib + u) * n + j] : 0.f;
+#pragma unroll
+        for (int u = 0; u < XB; ++u) {
+          const int i = ib + u;
+          if (i < m) {
+#pragma unroll
+            for (int q = 0; q < CH; ++q)
+              if (a0 + q < K) dot2_step(Uo[i * K + a0 + q], xb[u], s[q], c[q]);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < CH; ++q)
+        if (a0 + q < K) Cout[ixoff(co_r, a0 + q) + ixoff(co_c, j)] = __fadd_rn(s[q], c[q]);
+    }
+    __syncthreads();
+}
+
+// Writes U_K (m x K) through (uo_r, uo_c) and C' = U_K^T X (K x n) through
+// (co_r, co_c).  X is not modified.  K <= min(m, n), K <= 32.
+template <typename R>
+__device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, R* Uout, Ix uo_r,
+                              Ix uo_c, R* Cout, Ix co_r, Ix co_c) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (K == m) {
+    // Nothing is cut: any orthonormal basis of R^m works; take the identity.
+    for (int e = tid; e < m * m; e += blockDim.x) {
+      const int i = e / m, k = e % m;
+      Uout[ixoff(uo_r, i) + ixoff(uo_c, k)] = i == k ? R(1) : R(0);
+    }
+    for (int e = tid; e < m * n; e += blockDim.x) {
+      const int k = e / n, j = e % n;
+      Cout[ixoff(co_r, k) + ixoff(co_c, j)] = X[e];
+    }
+    __syncthreads();
+    return;
+  }
+  PEPS_PHASE(0);
+  const bool tall = m >= n;
+  const int P = tall ? m : n, Q = tall ? n : m;
+  const int ld = w.ldw;
+  R* W = w.Wm;
+  R* tauL = w.tau;
+  R* tauR = w.tau + w.Qmax;
+  R* red = w.red;
+  bool tiled = false;
+  if constexpr (sizeof(R) == 4) {
+    if (P > 32 && P <= 128) {   // below 33 rows the shared-memory version is as fast
+      // the reflectors go to global memory: shared memory then holds the
+      // inverse-iteration workspace
+      W = w.Wg;
+      bidiag_tiles_f32(X, n, tall, P, Q, W, ld, w.t, w.tau, w.Qmax);
+      tiled = true;
+    }
+  }
+  if (!tiled) bidiag_shared<R>(X, m, n, tall, P, Q, W, ld, w.t, w.tau, w.Qmax, w.wv, red);
+  PEPS_PHASE(1);
+  // ---------------- Sturm sections for the K largest singular values
+  const int n2 = 2 * Q;
+  R tmax = R(0);
+  for (int i = tid; i < n2 - 1; i += blockDim.x) tmax = fmax(tmax, fabs(w.t[i]));
+  tmax = warp_max(tmax);
+  if (lane == 0) red[8 + warp] = tmax;
+  __syncthreads();
+  tmax = R(0);
+  for (int i = 0; i < kWarps; ++i) tmax = fmax(tmax, red[8 + i]);
+  if constexpr (sizeof(R) == 4) {
+    // the squares in shared memory (wv is free here) where they fit
+    R* t2 = n2 <= kMaxT2Shared ? w.wv : w.t2;
+    for (int i = tid; i < n2 - 1; i += blockDim.x) t2[i] = w.t[i] * w.t[i];
+    __syncthreads();
+    const R bound = R(2) * tmax * (R(1) + R(4) * Eps<R>::eps) + Eps<R>::tiny;
+    const R pivmin = Eps<R>::tiny * R(1024) * fmax(R(1), tmax * tmax);
+    section_f32(t2, n2, K, bound, pivmin, w.lam);
+  } else {
+    const int e2 = pow2_exponent(tmax);
+    const R down = pow2<R>(-e2);
+    float* t2f = reinterpret_cast<float*>(w.wv);       // >= 512 floats
+    float* lamf = reinterpret_cast<float*>(red + 24);
+    for (int i = tid; i < n2 - 1; i += blockDim.x) {
+      const R v = w.t[i] * down;
+      w.t2[i] = v * v;
+      t2f[i] = (float)(v * v);
+    }
+    __syncthreads();
+    section_f32(t2f, n2, K, 4.001f, Eps<float>::tiny * 4096.f, lamf);
+    __syncthreads();
+    if (warp < 4) refine_values_f64(tid, K <= 8 ? 16 : K <= 16 ? 8 : 4, w.t2, n2, K, lamf, pow2<R>(e2), w.lam);
+  }
+  __syncthreads();
+  PEPS_PHASE(2);
+  // ---------------- inverse iteration, one thread per vector
+  const R pivtiny = Eps<R>::eps * fmax(tmax, Eps<R>::tiny * R(1e10));
+  R* Ub = w.Ubs;
+  {
+    // On the register-tiled path the shared region (matrix, Ub, Uk) is free: the
+    // workspace goes there when it fits, t to wv.  The vectors are then read
+    // into registers before Ub, which it may overlap, is written.
+    const bool in_smem = tiled && 4 * n2 * K <= w.gsm_reals && n2 <= kMaxT2Shared;
+    R* wsR = in_smem ? w.gsm : inv_align(w.lu);
+    const R* tv = w.t;
+    if (in_smem || n2 <= w.Qmax * w.Kmax) {
+      R* ts = in_smem ? w.wv : Ub;
+      for (int i = tid; i < n2 - 1; i += blockDim.x) ts[i] = w.t[i];
+      tv = ts;
+    }
+    __syncthreads();
+    if (tid < K) red[tid] = inverse_iteration(tv, n2, w.lam[tid], pivtiny, wsR, K, tid, (unsigned)(tid + 1));
+    __syncthreads();
+    PEPS_PHASE(3);
+    // u-parts (odd positions) for a tall matrix, v-parts (even) for a wide one, scaled
+    constexpr int kPer = 16;   // 128 x 32 entries at most on the tiled path
+    auto entry = [&](int e) {
+      const int i = e / K, k = e % K;
+      return wsR[((2 * i + (tall ? 1 : 0)) * K + k) * 4 + 3] * red[k];
+    };
+    if (in_smem) {
+      R v[kPer];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q)
+        if (tid + q * kThreads < Q * K) v[q] = entry(tid + q * kThreads);
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < kPer; ++q)
+        if (tid + q * kThreads < Q * K) Ub[tid + q * kThreads] = v[q];
+    } else {
+      for (int e = tid; e < Q * K; e += blockDim.x) Ub[e] = entry(e);
+    }
+  }
+  __syncthreads();
+  // ---------------- orthonormal basis of the kept vectors: CholeskyQR2
+  // (G = Ub^T Ub = R^T R, Ub <- Ub R^-1, twice; Fukaya et al. 2014).  Each
+  // pass costs three barriers.  If a direction of Ub is below 1e-3 of its
+  // norm (a cluster or a zero singular value), Gram-Schmidt with replacement
+  // of degenerate directions (below) takes over from the current Ub.
+  const bool need_cgs = cholesky_qr2<R>(Ub, w.Uks, Q, K);
   // ---------------- Gram-Schmidt with re-orthogonalisation (CGS2), fallback
   if (need_cgs) gram_schmidt<R>(Ub, Q, K, red);
   PEPS_PHASE(4);
@@ -1788,33 +1949,9 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
         // first row, so the row groups above it are left out (half of the
         // work): apply_reflectors takes the reflectors whose first row is in
         // one group of sixteen.
-        const int c = warp * 2 + (lane >> 4), l = lane & 15;
-        float u[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int i = l + 16 * r;
-          u[r] = (c < K && i < rowsU) ? Uk[i * K + c] : 0.f;
-        }
-        int j = nref - 1;
-        const int off = tall ? 0 : 1;   // first row of reflector j: j + off
-        const float* Wf = reinterpret_cast<const float*>(W);
-        const float* tf = reinterpret_cast<const float*>(taus);
-        const float* sf = reinterpret_cast<const float*>(scs);
-        j = apply_reflectors<7>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        j = apply_reflectors<6>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        j = apply_reflectors<5>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        j = apply_reflectors<4>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        j = apply_reflectors<3>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        j = apply_reflectors<2>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        j = apply_reflectors<1>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        apply_reflectors<0>(Wf, ld, tall, rowsU, l, off, j, tf, sf, u);
-        if (c < K) {
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int i = l + 16 * r;
-            if (i < rowsU) Uk[i * K + c] = u[r];
-          }
-        }
+        apply_all_reflectors(reinterpret_cast<const float*>(W), ld, tall, rowsU, nref, K,
+                             reinterpret_cast<const float*>(taus), reinterpret_cast<const float*>(scs),
+                             reinterpret_cast<float*>(Uk));
         __syncthreads();
         applied = true;
       }
@@ -1896,83 +2033,7 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
   // U + U (-1/2 (U^T U - I)), so its small correction is not rounded
   // against 1.
   if constexpr (sizeof(R) == 4) {
-    float* Mns = reinterpret_cast<float*>(Ub);
-    const float* Uf = reinterpret_cast<const float*>(Uk);
-    for (int e = tid; e < K * K; e += blockDim.x) {
-      const int a = e / K, b = e % K;
-      float s = 0.f, c = 0.f;
-      for (int i = 0; i < m; ++i) dot2_step(Uf[i * K + a], Uf[i * K + b], s, c);
-      // s is within a factor 2 of 1 on the diagonal, so s - 1 is exact
-      Mns[e] = -0.5f * (a == b ? __fadd_rn(__fsub_rn(s, 1.f), c) : __fadd_rn(s, c));
-    }
-    __syncthreads();
-    // Up to kNsPer entries per thread, the new U replaces the old one in
-    // shared memory once every thread has read the old one; larger U go to
-    // the global copy.
-    constexpr int kNsPer = 8;
-    const bool u_shared = m * K <= kNsPer * kThreads;
-    float* Us = reinterpret_cast<float*>(Uk);
-    if (u_shared) {
-      float nv[kNsPer];
-#pragma unroll
-      for (int q = 0; q < kNsPer; ++q) {
-        const int e = tid + q * kThreads;
-        if (e < m * K) {
-          const int i = e / K, k = e % K;
-          float corr = 0.f;
-          for (int a = 0; a < K; ++a) corr = fmaf(Uf[i * K + a], Mns[a * K + k], corr);
-          nv[q] = Uf[i * K + k] + corr;
-          Uout[ixoff(uo_r, i) + ixoff(uo_c, k)] = nv[q];
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < kNsPer; ++q) {
-        const int e = tid + q * kThreads;
-        if (e < m * K) Us[e] = nv[q];
-      }
-    } else {
-      for (int e = tid; e < m * K; e += blockDim.x) {
-        const int i = e / K, k = e % K;
-        float corr = 0.f;
-        for (int a = 0; a < K; ++a) corr = fmaf(Uf[i * K + a], Mns[a * K + k], corr);
-        const float v = Uf[i * K + k] + corr;
-        Uout[ixoff(uo_r, i) + ixoff(uo_c, k)] = v;
-        w.Uk[e] = v;
-      }
-    }
-    __syncthreads();
-    // C' = U_K^T X, X row-major m x n.  One work item is a column j and a
-    // chunk of 8 rows of C'; its X column is read once (coalesced over j),
-    // eight rows at a time so that eight loads are in flight together.
-    constexpr int CH = 8, XB = 8;
-    const float* Uo = u_shared ? Us : reinterpret_cast<const float*>(w.Uk);
-    const float* Xf = reinterpret_cast<const float*>(X);
-    const int nchunk = (K + CH - 1) / CH;
-    for (int item = tid; item < n * nchunk; item += blockDim.x) {
-      const int j = item % n, a0 = (item / n) * CH;
-      float s[CH], c[CH];
-#pragma unroll
-      for (int q = 0; q < CH; ++q) s[q] = c[q] = 0.f;
-      for (int ib = 0; ib < m; ib += XB) {
-        float xb[XB];
-#pragma unroll
-        for (int u = 0; u < XB; ++u) xb[u] = ib + u < m ? Xf[(ib + u) * n + j] : 0.f;
-#pragma unroll
-        for (int u = 0; u < XB; ++u) {
-          const int i = ib + u;
-          if (i < m) {
-#pragma unroll
-            for (int q = 0; q < CH; ++q)
-              if (a0 + q < K) dot2_step(Uo[i * K + a0 + q], xb[u], s[q], c[q]);
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < CH; ++q)
-        if (a0 + q < K) Cout[ixoff(co_r, a0 + q) + ixoff(co_c, j)] = __fadd_rn(s[q], c[q]);
-    }
-    __syncthreads();
+    finish_f32(X, m, n, K, Ub, Uk, w.Uk, Uout, uo_r, uo_c, Cout, co_r, co_c);
   } else {
     R* Mns = Ub;
     for (int e = tid; e < K * K; e += blockDim.x) {

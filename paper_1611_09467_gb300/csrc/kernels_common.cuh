@@ -355,6 +355,7 @@ __device__ void carve_zip(const Geometry& g, R*& p, ZipBufs<R>& zb, R* wm_smem, 
   zb.gism = gism;
   zb.gsm_reals = (int)(reals_region_bytes(g, sizeof(R), true, wm_smem != nullptr) / sizeof(R));
   zb.tw.wv = wv;
+  zb.tw.gsm_reals = zb.gsm_reals;
   zb.tw.gsm = gsm;
   zb.tw.gism = gism;
   const size_t Dc = g.Dc, D = g.D, P = Dc * D;

@@ -723,35 +723,53 @@ __device__ __noinline__ void back_transform(const R* W, int ld, bool tall, int P
   }
 }
 
-// CH rows of the carry for one column of X: C[q ck] = sum_i U[i K + q] X[i n], q < nq.
+// CH rows of the carry for one column of X: C[q ck] = sum_i U[i K + q] X[i n], q < nq
+// (FP32: compensated, two rows at once in packed instructions).
 template <typename R, int CH, bool VEC>
 __device__ __forceinline__ void carry_rows(const R* U, const R* X, int m, int n, int K, R* C, int ck, int nq) {
-  R s[CH], c[CH];
+  if constexpr (sizeof(R) == 4) {
+    float2 s[CH / 2], c[CH / 2];
 #pragma unroll
-  for (int q = 0; q < CH; ++q) s[q] = c[q] = R(0);
+    for (int q = 0; q < CH / 2; ++q) s[q] = c[q] = make_float2(0.f, 0.f);
 #pragma unroll 4
-  for (int i = 0; i < m; ++i) {
-    const R x = X[i * n];
-    R u[CH];
-    if constexpr (VEC && sizeof(R) == 4) {
+    for (int i = 0; i < m; ++i) {
+      const float x = X[i * n];
+      float u[CH];
 #pragma unroll
       for (int q = 0; q < CH; q += 4) {
-        const float4 a = *reinterpret_cast<const float4*>(U + i * K + q);
-        u[q] = a.x; u[q + 1] = a.y; u[q + 2] = a.z; u[q + 3] = a.w;
+        if constexpr (VEC) {
+          const float4 a = *reinterpret_cast<const float4*>(U + i * K + q);
+          u[q] = a.x; u[q + 1] = a.y; u[q + 2] = a.z; u[q + 3] = a.w;
+        } else {
+#pragma unroll
+          for (int z = q; z < q + 4; ++z) u[z] = z < nq ? U[i * K + z] : 0.f;
+        }
       }
-    } else {
 #pragma unroll
-      for (int q = 0; q < CH; ++q) u[q] = (VEC || q < nq) ? U[i * K + q] : R(0);
+      for (int q = 0; q < CH / 2; ++q)
+        dot2_step2(make_float2(u[2 * q], u[2 * q + 1]), make_float2(x, x), s[q], c[q]);
     }
 #pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      if constexpr (sizeof(R) == 4) dot2_step(u[q], x, s[q], c[q]);
-      else s[q] = fma(u[q], x, s[q]);
+    for (int q = 0; q < CH / 2; ++q) {
+      const float2 v = __fadd2_rn(s[q], c[q]);
+      if (VEC || 2 * q < nq) C[2 * q * ck] = v.x;
+      if (VEC || 2 * q + 1 < nq) C[(2 * q + 1) * ck] = v.y;
     }
+  } else {
+    R s[CH];
+#pragma unroll
+    for (int q = 0; q < CH; ++q) s[q] = R(0);
+#pragma unroll 4
+    for (int i = 0; i < m; ++i) {
+      const R x = X[i * n];
+#pragma unroll
+      for (int q = 0; q < CH; ++q)
+        if (VEC || q < nq) s[q] = fma(U[i * K + q], x, s[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < CH; ++q)
+      if (VEC || q < nq) C[q * ck] = s[q];
   }
-#pragma unroll
-  for (int q = 0; q < CH; ++q)
-    if (VEC || q < nq) C[q * ck] = sizeof(R) == 4 ? s[q] + c[q] : s[q];
 }
 
 // One Newton-Schulz step on U (m x K), U to global memory through (uo, uk), and the
