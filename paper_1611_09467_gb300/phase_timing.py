@@ -37,25 +37,35 @@ def measure(workload: str = "16x16_D8_Dc16", n: int = 1216, prec: str = "mixed_t
         raise RuntimeError("the library is already loaded in this process; run the diagnostic in its own process")
     peps.LIB_PATH = path
     lib = peps.lib()
-    lib.peps_phase_read.argtypes = [ctypes.c_void_p, ctypes.c_int]
-    lib.peps_phase_read.restype = ctypes.c_int
+    # one set of counters per translation unit: the FP32 and FP64 CTA sweeps, the one-warp sweeps
+    readers = [lib.peps_phase_read, lib.peps_phase_read_f64, lib.peps_phase_read_small]
+    for f in readers:
+        f.argtypes = [ctypes.c_void_p, ctypes.c_int]
+        f.restype = ctypes.c_int
+
+    def read():
+        total = [0] * 16
+        for f in readers:
+            counts = (ctypes.c_ulonglong * 16)()
+            if f(counts, 1) != 0:
+                raise RuntimeError("reading the phase counters failed")
+            total = [a + b for a, b in zip(total, counts)]
+        return total
+
     w = inputs.WORKLOADS[workload]
     L, D, Dc = w["L"], w["D"], w["Dc"]
     A, _ = inputs.workload_inputs(workload, n=1)
     S = torch.from_numpy(inputs.pack_spins(inputs.random_sz0(n, L * L, seed)).view(np.int64)).cuda()
     p = peps.PEPS(A, L, L, D, Dc, J1=1.0, J2=w["J2"], prec=prec)
     try:
-        counts = (ctypes.c_ulonglong * 16)()
         p.evaluate(S, logabs=True, eloc=False)
-        if lib.peps_phase_read(counts, 1) != 0:
-            raise RuntimeError("reading the phase counters failed")
+        read()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record()
         p.evaluate(S, logabs=True, eloc=False)
         e1.record()
         torch.cuda.synchronize()
-        if lib.peps_phase_read(counts, 1) != 0:
-            raise RuntimeError("reading the phase counters failed")
+        counts = read()
     finally:
         p.close()
     return {name: counts[k] / n / 1e6 for k, name in PHASES.items()}, e0.elapsed_time(e1)
