@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kThreads) k_mc(KArgs<R> a, uint64_t* S, int ns
 }
 
 // One warp per chain (models small.cuh takes).  304 chains of 8x8 D = 4 Dc = 8 in
-// FP64 take 126 ms a sweep against 397 ms with a CTA each, whose time went to the
+// FP64 take 105 ms a sweep against 397 ms with a CTA each, whose time went to the
 // truncation's barriers and FP64 sections and to the tiled engine's offset
 // tables on products of a few hundred outputs.
 template <typename R>

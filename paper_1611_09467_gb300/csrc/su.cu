@@ -308,6 +308,8 @@ struct Args {
   size_t slot;
 };
 
+constexpr int kMaxD = 16;
+
 // Shared memory: Theta and V (n2max^2 each, n2max = 4D), sigma and its inverse,
 // tau, the leg weights and their inverses ([2 sites][4 legs][D] each), the gate;
 // then M_i, M_j, N_i, N_j (D^3 x 2D each) where they fit.
@@ -556,7 +558,7 @@ extern "C" {
 
 peps_status peps_su_create(const peps_params* p, void* stream, peps_su** out) {
   if (!p || !out) return su_fail(PEPS_EINVAL, "null argument");
-  if (p->Lx < 2 || p->Ly < 2 || p->Lx > kMaxL || p->Ly > kMaxL || p->D < 1 || p->D > 16 || p->d != 2)
+  if (p->Lx < 2 || p->Ly < 2 || p->Lx > kMaxL || p->Ly > kMaxL || p->D < 1 || p->D > su::kMaxD || p->d != 2)
     return su_fail(PEPS_EINVAL, "need 2 <= Lx, Ly <= 64, 1 <= D <= 16, d = 2");
   if (!std::isfinite(p->J1) || !std::isfinite(p->J2)) return su_fail(PEPS_EINVAL, "non-finite coupling");
   peps_su* s = new peps_su();
@@ -625,7 +627,10 @@ peps_status peps_su_create(const peps_params* p, void* stream, peps_su** out) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->A0, sizeof(double) * N * 2 * D4);
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->A1, sizeof(double) * N * 2 * D4);
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->chg, 2 * sizeof(unsigned long long));
-  const size_t smem = su::smem_doubles(D) * sizeof(double);
+  // the limit belongs to the kernel, not to this state: always the largest over
+  // all D, so that a state of another D does not lower it under this one
+  size_t smem = 0;
+  for (int d = 1; d <= su::kMaxD; ++d) smem = std::max(smem, su::smem_doubles(d) * sizeof(double));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(su::k_su_bond, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) {

@@ -32,3 +32,21 @@ def test_su_weights_by_bond_dimension(D):
     ref = np.stack([lam[b] for b in h + v])
     assert np.abs(s.lam.cpu().numpy() - ref).max() < 1e-10
     s.close()
+
+
+def test_su_states_of_two_bond_dimensions():
+    """A state of a smaller D made in between does not lower the shared memory
+    that the first one's launches may ask for."""
+    from paper_1611_09467_gb300.peps import SimpleUpdate
+    h, v = O.nn_bonds(2, 2)
+    states = []
+    for D in (7, 2):
+        Gam, lam = SU.init_state(2, 2, D, 78)
+        s = SimpleUpdate(Gam, np.stack([lam[b] for b in h + v]), 2, 2, D, J1=1.0, J2=0.5)
+        states.append((s, Gam, lam, D))
+    for s, Gam, lam, D in states:
+        s.evolve(0.05, 1, measure=False)
+        SU.trotter_step(Gam, lam, 2, 2, 1.0, 0.5, 0.05, D)
+        ref = np.stack([lam[b] for b in h + v])
+        assert np.abs(s.lam.cpu().numpy() - ref).max() < 1e-10
+        s.close()
