@@ -425,9 +425,12 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
   }
   __syncthreads();
   const int K = min(D, min(m2, n2));
+  // ordered by the bits (norms are not negative), NaN before all: s_order is
+  // filled whatever the tensors hold
+  auto key = [&](int c) { return __double_as_longlong(sig[c]) & 0x7fffffffffffffffLL; };
   for (int c = threadIdx.x; c < n2; c += blockDim.x) {
     int rank = 0;
-    for (int q = 0; q < n2; ++q) rank += sig[q] > sig[c] || (sig[q] == sig[c] && q < c) ? 1 : 0;
+    for (int q = 0; q < n2; ++q) rank += key(q) > key(c) || (key(q) == key(c) && q < c) ? 1 : 0;
     if (rank < K) s_order[rank] = c;
   }
   __syncthreads();

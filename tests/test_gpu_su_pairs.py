@@ -50,3 +50,15 @@ def test_su_states_of_two_bond_dimensions():
         ref = np.stack([lam[b] for b in h + v])
         assert np.abs(s.lam.cpu().numpy() - ref).max() < 1e-10
         s.close()
+
+
+def test_su_nan_tensors():
+    """NaN tensors give NaN weights and leave the device usable."""
+    from paper_1611_09467_gb300.peps import SimpleUpdate
+    Gam, lam = SU.init_state(2, 2, 3, 79)
+    h, v = O.nn_bonds(2, 2)
+    lam0 = np.stack([lam[b] for b in h + v])
+    s = SimpleUpdate(np.full_like(Gam, np.nan), lam0, 2, 2, 3, J1=1.0, J2=0.5)
+    s.evolve(0.05, 1, measure=False)
+    assert np.isnan(s.lam.cpu().numpy()).all()
+    s.close()
