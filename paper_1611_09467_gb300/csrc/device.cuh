@@ -620,6 +620,12 @@ struct TruncWork {
   int Kmax;        // Ubs and Uks hold Qmax x Kmax
   int gsm_reals;   // size of the shared region
   int wm_shared;   // Wm is in shared memory
+  // Whether blocks of the register-tiled path with at most 16 columns apply
+  // their reflectors one at a time: models whose shared region is at most 200 KB.
+  // Above (D = 10, Dc = 20) such blocks are the few next to an edge, and take
+  // the compact WY form as the others do; the two differ in the last FP32 bits,
+  // 6e-9 of an energy.
+  int one_by_one;
 };
 
 // Element counts of the truncation workspace for P, Q <= pq and K <= kmax.
@@ -1940,7 +1946,7 @@ __device__ void cta_topk_left(const R* X, int m, int n, int K, TruncWork<R>& w, 
     const int nref = tall ? Q : Q - 1;
     bool applied = false;
     if constexpr (sizeof(R) == 4) {
-      if (tiled && w.wm_shared && Q <= 128 && rowsU <= 128 && K <= 2 * kWarps) {
+      if (tiled && w.one_by_one && Q <= 128 && rowsU <= 128 && K <= 2 * kWarps) {
         // Reflectors in shared memory, at most 128 rows and 16 columns: one
         // column of U per half-warp (lane l holds rows l, l + 16, ...), the
         // reflectors applied one at a time, last first.  Each is a dot

@@ -378,6 +378,7 @@ __device__ void carve_zip(const Geometry& g, R*& p, ZipBufs<R>& zb, R* wm_smem, 
   w.Qmax = (int)P;
   w.Kmax = (int)Dc;
   w.wm_shared = wm_smem != nullptr;
+  w.one_by_one = wm_smem && reals_region_bytes(g, sizeof(R), true, true) + kGemmSmemInts * sizeof(int) <= 200 * 1024;
   w.tau = p; p += 4 * P;
   w.t = p; p += 2 * P;
   w.t2 = p; p += 2 * P;
