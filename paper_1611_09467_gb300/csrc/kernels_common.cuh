@@ -39,10 +39,20 @@ __device__ __forceinline__ TDims tdims(const Geometry& g, int row, int col) {
 }
 
 // Kernels with large shared-memory footprints ask for the maximum carve-out so
-// the occupancy the grids are sized for is the one the hardware grants.
+// the occupancy the grids are sized for is the one the hardware grants.  The
+// limit belongs to the kernel, not to the launch, and host threads may launch
+// one kernel for models of different sizes: it is always set to all that the
+// device leaves beside the static part, so no thread lowers it under another.
 template <typename F>
 static cudaError_t prefer_shared(F* f, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, f);
+  if (e != cudaSuccess) return e;
+  const size_t most = (size_t)optin - fa.sharedSizeBytes;
+  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem > most ? smem : most));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   return e;
