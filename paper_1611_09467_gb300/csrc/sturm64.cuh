@@ -24,17 +24,23 @@ namespace peps {
 
 // Number of eigenvalues below x > 0 of the zero-diagonal symmetric
 // tridiagonal with squared off-diagonals t2 (scaled so that they are below 4).
-// A zero minor counts as a negative pivot, as a clamped pivot does.
+// A zero minor counts as a negative pivot, as a clamped pivot does: it is
+// replaced by -2^-100 times the minor before it (the pivot -2^-100, a change of a
+// diagonal entry far below an ulp).  Left at zero it would make every later minor
+// zero where the next off-diagonal is zero too.
 __device__ __forceinline__ int sturm_count_minors(const double* t2, int n2, double x) {
   double p0 = 1.0, p1 = -x;
   int cnt = 1;
   unsigned sg = 1u;
   auto row = [&](double tv) {
-    const double p2 = fma(-x, p1, -(tv * p0));
-    const unsigned h = (unsigned)__double2hiint(p2), lo = (unsigned)__double2loint(p2);
-    const unsigned s = ((h & 0x7fffffffu) | lo) == 0u ? (sg ^ 1u) : (h >> 31);
+    const double m = fma(-x, p1, -(tv * p0));
+    const unsigned h = (unsigned)__double2hiint(m), lo = (unsigned)__double2loint(m);
+    const bool zero = ((h & 0x7fffffffu) | lo) == 0u;
+    const unsigned s = zero ? (sg ^ 1u) : (h >> 31);
     cnt += (int)(s ^ sg);
     sg = s;
+    const int tiny = max((__double2hiint(p1) & 0x7ff00000) - (100 << 20), 1 << 20);
+    const double p2 = __hiloint2double(zero ? (int)(s << 31) | tiny : (int)h, (int)lo);
     p0 = p1;
     p1 = p2;
   };
