@@ -129,8 +129,25 @@ __device__ __forceinline__ void jacobi_pair(int round, int k, int np, int& p, in
   }
 }
 
+// Squared column norms whose products and squares stay in range: zero, or
+// 2^-400 .. 2^400.
+__device__ __forceinline__ bool plain_norm2(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return (h | (unsigned)__double2loint(x)) == 0u || h - 0x26f00000u < 0x32000000u;
+}
+
+// The rotation of columns of any other norms, as a function of ratios only: (c, s),
+// or (1, 0) where the pair is orthogonal to working precision.
+__device__ __noinline__ double2 jacobi_rotation_any(double al, double be, double ga, double tol) {
+  if (!(fabs(ga) > tol * sqrt(al) * sqrt(be))) return make_double2(1.0, 0.0);
+  const double zeta = (be - al) / (2.0 * ga);
+  const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+  const double c = 1.0 / sqrt(1.0 + t * t);
+  return make_double2(c, c * t);
+}
+
 template <int RP>
-__device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int round, int np, int npair, double tol2,
+__device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int round, int np, int npair, double tol,
                                                double2* cs) {
   const int gl = threadIdx.x & 7, k = threadIdx.x >> 3;
   int p = 0, q = 0;
@@ -157,8 +174,13 @@ __device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int ro
     be += __shfl_xor_sync(0xffffffffu, be, o);
     ga += __shfl_xor_sync(0xffffffffu, ga, o);
   }
-  const bool rot = on && ga * ga > tol2 * al * be;
+  bool rot = on && ga * ga > tol * tol * al * be;
   double2 cn = make_double2(1.0, 0.0);
+  const bool plain = plain_norm2(al) && plain_norm2(be);
+  if (!plain) {
+    if (on) cn = jacobi_rotation_any(al, be, ga, tol);
+    rot = cn.y != 0.0;
+  }
   if (__any_sync(0xffffffffu, rot)) {
     // the rotation with t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
     // zeta = (be - al) / (2 ga): cos^2 = (1 + |be - al| / h) / 2 and
@@ -167,10 +189,15 @@ __device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int ro
     const double rh = quick_rsqrt(fma(d, d, g2 * g2));
     const double c2 = fma(0.5 * fabs(d), rh, 0.5);
     const double rc = quick_rsqrt(c2);
-    const double c = c2 * rc;
-    const double sn = (d == 0.0 ? fabs(g2) : (d > 0.0 ? g2 : -g2)) * (0.5 * rh) * rc;
+    double c = c2 * rc;
+    double sn = (d == 0.0 ? fabs(g2) : (d > 0.0 ? g2 : -g2)) * (0.5 * rh) * rc;
     if (rot) {
-      cn = make_double2(c, sn);
+      if (plain) {
+        cn = make_double2(c, sn);
+      } else {
+        c = cn.x;
+        sn = cn.y;
+      }
 #pragma unroll
       for (int x = 0; x < RP; ++x) {
         const int r = gl + x * 8;
@@ -195,7 +222,7 @@ __device__ void jacobi_svd(double* T, int m2, int n2, double* V, double2* cs, in
   const int warp = threadIdx.x >> 5, rp = (m2 + 7) / 8;
   const bool is_t = warp < nt, is_v = warp >= v0 && warp < v1;
   const int busy = v1 > nt ? v1 : nt;             // the warps that meet at the barrier: 0 .. busy - 1
-  const double tol = 1e-15 * (double)m2, tol2 = tol * tol;
+  const double tol = 1e-15 * (double)m2;
   __syncthreads();
   for (int sweep = 0; sweep < 40; ++sweep) {
     if (threadIdx.x == 0) *s_rot = 0;
@@ -206,11 +233,11 @@ __device__ void jacobi_svd(double* T, int m2, int n2, double* V, double2* cs, in
         if (is_t && round < np - 1) {
           double2* c = cs + (round & 1) * 32;
           bool r;
-          if (rp <= 1) r = jacobi_round_t<1>(T, m2, n2, round, np, npair, tol2, c);
-          else if (rp <= 2) r = jacobi_round_t<2>(T, m2, n2, round, np, npair, tol2, c);
-          else if (rp <= 3) r = jacobi_round_t<3>(T, m2, n2, round, np, npair, tol2, c);
-          else if (rp <= 4) r = jacobi_round_t<4>(T, m2, n2, round, np, npair, tol2, c);
-          else r = jacobi_round_t<8>(T, m2, n2, round, np, npair, tol2, c);
+          if (rp <= 1) r = jacobi_round_t<1>(T, m2, n2, round, np, npair, tol, c);
+          else if (rp <= 2) r = jacobi_round_t<2>(T, m2, n2, round, np, npair, tol, c);
+          else if (rp <= 3) r = jacobi_round_t<3>(T, m2, n2, round, np, npair, tol, c);
+          else if (rp <= 4) r = jacobi_round_t<4>(T, m2, n2, round, np, npair, tol, c);
+          else r = jacobi_round_t<8>(T, m2, n2, round, np, npair, tol, c);
           rotated = rotated || r;
         }
         if (is_v && round > 0) {
