@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(32) k_pair_small(KArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t sp[kMaxWords];
   __shared__ int eH[kMaxL + 1];
-  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw));
+  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw), sandwich_in_fused_order<R>(a.g));
   pair_items<R>(a, ops, a.scratch + (size_t)blockIdx.x * a.slot_elems, sp, eH);
 }
 

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(32) k_row_small(KArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t sp[kMaxWords];
   __shared__ int eG[kMaxL + 1];
-  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw));
+  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw), sandwich_in_fused_order<R>(a.g));
   row_items<R>(a, ops, a.scratch + (size_t)blockIdx.x * a.slot_elems, sp, eG);
 }
 

@@ -4,8 +4,8 @@
 // models with Dc D <= 32, small.cuh).  A CTA of a WarpOps kernel is one warp.
 //
 // WarpOps keeps the multiply-add chains of the contraction programs
-// (contract.cuh) and the 256-thread partition of the dot products, so FP32
-// results equal the CTA's bit for bit.  Two-row steps are split over the
+// (contract.cuh) and the 256-thread partition of the dot products, so results
+// equal the CTA's bit for bit (or, asked to, those of the fused kernels).  Two-row steps are split over the
 // out-bond of the upper environment: every step of the program is independent
 // between out-bonds, so a slice needs three temporaries of D^3 Dc reals instead
 // of Dc^2 D^3 and no sum is cut.  Rows that are read as the left operand are
@@ -148,6 +148,26 @@ PEPS_HD GemmDesc site_slice(int s, int D, int Dc) {
   return gemm(D3, D, Dc, ix1(1), kx(Dc, 0, D3), kx(Dc, 0, 1), ix1(Dc), ix2(D, 1, DD), ix1(D3));   // rows (u,d,r), cols l
 }
 
+// The order of row_fused.cuh and pair_fused.cuh.  Left steps sum in the same
+// order there; right steps take the horizontal index before the vertical one
+// and L's in-bond before its physical index.  The site environment pairs F with
+// Mu and Md with G (Z of site_env_step) and sums their product over (a', b).
+PEPS_HD GemmDesc fused_right(GemmDesc g, bool site_step, int D, int Dc) {
+  if (site_step) {   // k = (r, u) of T and of rows [u][r]
+    g.ak = kx(D, 1, D);
+    g.bk = kx(D, D * D, D);
+  } else {           // k = (b', d) of Md and of rows [d][b']
+    g.ak = g.bk = kx(D, 1, Dc);
+  }
+  return g;
+}
+PEPS_HD GemmDesc site_fused(int s, int D, int Dc) {
+  const int DD = D * D, D3 = DD * D;
+  if (s == 0)   // X[b][l][u]: rows l of F[a][l][a'] at a', cols (u,b) of Mu
+    return gemm(D, D * Dc, Dc, ix1(Dc), kx(Dc, 0, D * Dc), kx(Dc, 0, D * Dc), ix1(1), ix1(D), ix2(Dc, 1, DD));
+  return gemm(DD, DD, Dc, ix1(1), kx(Dc, 0, DD), kx(Dc, 0, D), ix2(D, Dc * D, 1), ix2(D, D3, D), ix2(D, 1, DD));
+}
+
 // Reals of shared memory the contractions need; the zip-up's region is reused.
 PEPS_HD int ops_reals(int D, int Dc) {
   const int DD = D * D, envT = Dc * D * Dc, p = DD + 1, q = Dc * D + 1;
@@ -172,13 +192,25 @@ __device__ __forceinline__ R* stage(R*& p, const R* src, int n) {
 
 }  // namespace small
 
+// The small models whose sandwiches run in the fused kernels or on warps, by the
+// size of the batch: in FP64 D = 4, Dc = 8 (FP32 always takes the fused kernels where
+// there are any, FP64 D = 2, Dc = 4 always warps).
+template <typename R>
+PEPS_HD bool sandwich_in_fused_order(const Geometry& g) {
+  return sizeof(R) == 8 && g.D == 4 && g.Dc == 8;
+}
+
+// fused: sums in the order of the fused kernels, for the models whose sandwiches
+// run in either (dispatch by batch size), so that results do not depend on it.
 template <typename R>
 struct WarpOps {
   const KArgs<R>& a;
   R* sm;
   small::Layout L;
+  const bool fused;
 
-  __device__ WarpOps(const KArgs<R>& a_, R* sm_) : a(a_), sm(sm_), L(small::layout(a_.g.D, a_.g.Dc)) {}
+  __device__ WarpOps(const KArgs<R>& a_, R* sm_, bool fused_ = false)
+      : a(a_), sm(sm_), L(small::layout(a_.g.D, a_.g.Dc)), fused(fused_) {}
   __device__ double absorb(const R* Min, R* Mout, int row, int dir, bool lr, const int* bdin, const uint64_t* sp) {
     __syncwarp();
     return small::absorb_row<R>(a, Min, Mout, row, dir, lr, bdin, sp, sm, L);
@@ -197,7 +229,8 @@ struct WarpOps {
     if (right) small::desc_gemm<R>(col1_right_step(0, D, Dc), u, f, t0);
     else small::desc_gemm<R>(col1_left_step(0, D, Dc), f, u, t0);
     for (int s = 1; s < 3; ++s) {
-      const GemmDesc g = right ? col1_right_step(s, D, Dc) : col1_left_step(s, D, Dc);
+      GemmDesc g = right ? col1_right_step(s, D, Dc) : col1_left_step(s, D, Dc);
+      if (fused && right) g = small::fused_right(g, s == 1, D, Dc);
       small::desc_gemm<R>(g, s == 1 ? t0 : t1, s == 1 ? t : d, s == 1 ? t1 : out);
     }
   }
@@ -219,7 +252,8 @@ struct WarpOps {
     for (int k = nx * DD * Dc + small::lane_id(); k < Dc * DD * Dc; k += 32) out[k] = R(0);
     for (int x = 0; x < nx; ++x)
       for (int s = 0; s < 4; ++s) {
-        const GemmDesc g = right ? small::right2_slice(s, D, Dc) : small::left2_slice(s, D, Dc);
+        GemmDesc g = right ? small::right2_slice(s, D, Dc) : small::left2_slice(s, D, Dc);
+        if (fused && right && (s & 1)) g = small::fused_right(g, s == 1, D, Dc);
         const R* A = s == 0 ? e : (s == 1 ? x0 : (s == 2 ? x1 : x2));
         const R* B = s == 0 ? u + (right ? x * D * Dc : x) : (s == 1 ? t1 : (s == 2 ? t2 : d));
         small::desc_gemm<R>(g, A, B, s == 0 ? x0 : (s == 1 ? x1 : (s == 2 ? x2 : out + x * DD * Dc)));
@@ -238,20 +272,36 @@ struct WarpOps {
     R* b = r + small::up4(Dc * DD * D);
     __syncwarp();
     small::desc_gemm<R>(site_env_step(0, D, Dc), d, gg, z);
-    for (int x = 0; x < Dc; ++x) {
+    for (int x = 0; fused && x < Dc; ++x) {
+      small::desc_gemm<R>(small::site_fused(0, D, Dc), f + x, u, r);
+      small::desc_gemm<R>(small::site_fused(1, D, Dc), r, z + x * D * Dc * D, b, x > 0);
+    }
+    for (int x = 0; !fused && x < Dc; ++x) {
       small::desc_gemm<R>(small::site_slice(0, D, Dc), z, u + x * D * Dc, r);
       small::desc_gemm<R>(small::site_slice(1, D, Dc), r, f + x * D * Dc, b, x > 0);
     }
     for (int k = small::lane_id(); k < DD * DD; k += 32) out[k] = b[k];
     __syncwarp();
   }
-  // block_dot and normalize_pow2
+  // block_dot and normalize_pow2.  In the fused kernels a thread owns one row (all
+  // but the last index) of a two-row transfer, or one entry of a single-row one, the
+  // last index slowest.
   __device__ __noinline__ R dot(const R* x, const R* y, int n) {
     R v[8];
+    const int Dc = a.g.Dc, rows = n / Dc;
     __syncwarp();
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
       R s = R(0);
+      if (fused) {
+        const bool one = rows * Dc <= 256;
+        const int row = one ? (32 * w + small::lane_id()) % rows : 32 * w + small::lane_id();
+        const int k0 = one ? (32 * w + small::lane_id()) / rows : 0, k1 = one ? k0 + 1 : Dc;
+        if (row < rows && k1 <= Dc)
+          for (int k = k0; k < k1; ++k) s = fma(x[row * Dc + k], y[row * Dc + k], s);
+        v[w] = s;
+        continue;
+      }
       for (int e = 32 * w + small::lane_id(); e < n; e += 256) s = fma(x[e], y[e], s);
       v[w] = s;
     }
