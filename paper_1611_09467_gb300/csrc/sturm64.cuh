@@ -24,23 +24,25 @@ namespace peps {
 
 // Number of eigenvalues below x > 0 of the zero-diagonal symmetric
 // tridiagonal with squared off-diagonals t2 (scaled so that they are below 4).
-// A zero minor counts as a negative pivot, as a clamped pivot does: it is
-// replaced by -2^-100 times the minor before it (the pivot -2^-100, a change of a
-// diagonal entry far below an ulp).  Left at zero it would make every later minor
-// zero where the next off-diagonal is zero too.
-__device__ __forceinline__ int sturm_count_minors(const double* t2, int n2, double x) {
+// A zero minor counts as a negative pivot, as a clamped pivot does.  Where the
+// next off-diagonal is zero too, all later minors are zero and nothing can be
+// counted from them: with `replace` a zero minor becomes -2^-100 times the one
+// before it (the pivot -2^-100, a change of a diagonal entry far below an ulp).
+// zeros: whether the minors ended that way.
+template <bool replace>
+__device__ __forceinline__ int count_minors(const double* t2, int n2, double x, bool& zeros) {
   double p0 = 1.0, p1 = -x;
   int cnt = 1;
   unsigned sg = 1u;
+  auto is_zero = [](double v) { return ((unsigned)(__double2hiint(v) & 0x7fffffff) | (unsigned)__double2loint(v)) == 0u; };
   auto row = [&](double tv) {
-    const double m = fma(-x, p1, -(tv * p0));
-    const unsigned h = (unsigned)__double2hiint(m), lo = (unsigned)__double2loint(m);
-    const bool zero = ((h & 0x7fffffffu) | lo) == 0u;
-    const unsigned s = zero ? (sg ^ 1u) : (h >> 31);
+    double p2 = fma(-x, p1, -(tv * p0));
+    const bool z = is_zero(p2);
+    const unsigned s = z ? (sg ^ 1u) : ((unsigned)__double2hiint(p2) >> 31);
     cnt += (int)(s ^ sg);
     sg = s;
-    const int tiny = max((__double2hiint(p1) & 0x7ff00000) - (100 << 20), 1 << 20);
-    const double p2 = __hiloint2double(zero ? (int)(s << 31) | tiny : (int)h, (int)lo);
+    if (replace && z)
+      p2 = __hiloint2double((int)(s << 31) | max((__double2hiint(p1) & 0x7ff00000) - (100 << 20), 1 << 20), 0);
     p0 = p1;
     p1 = p2;
   };
@@ -55,7 +57,20 @@ __device__ __forceinline__ int sturm_count_minors(const double* t2, int n2, doub
     p1 *= f;
   }
   for (; i < n2; ++i) row(t2[i - 1]);
+  zeros = is_zero(p0) && is_zero(p1);
   return cnt;
+}
+static __device__ __noinline__ int count_minors_again(const double* t2, int n2, double x) {
+  bool zeros;
+  return count_minors<true>(t2, n2, x, zeros);
+}
+// The replacement is a second pass for the points that need it (a root of a
+// leading block, met exactly): in every row it would lengthen the dependent chain
+// of the minors (8x8 D = 4 FP64 sweep: 1.3%).
+__device__ __forceinline__ int sturm_count_minors(const double* t2, int n2, double x) {
+  bool zeros;
+  const int cnt = count_minors<false>(t2, n2, x, zeros);
+  return zeros ? count_minors_again(t2, n2, x) : cnt;
 }
 
 // Half-width of the FP64 start interval around an FP32 value, in units where

@@ -20,6 +20,7 @@ SHIM = r"""
 using std::fma; using std::fmax; using std::max; using std::min;
 #define __device__
 #define __forceinline__ inline
+#define __noinline__
 inline int __double2hiint(double x) { int64_t b; std::memcpy(&b, &x, 8); return (int)(b >> 32); }
 inline int __double2loint(double x) { int64_t b; std::memcpy(&b, &x, 8); return (int)b; }
 inline double __hiloint2double(int h, int l) {
