@@ -129,25 +129,8 @@ __device__ __forceinline__ void jacobi_pair(int round, int k, int np, int& p, in
   }
 }
 
-// Squared column norms whose products and squares stay in range: zero, or
-// 2^-400 .. 2^400.
-__device__ __forceinline__ bool plain_norm2(double x) {
-  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
-  return (h | (unsigned)__double2loint(x)) == 0u || h - 0x26f00000u < 0x32000000u;
-}
-
-// The rotation of columns of any other norms, as a function of ratios only: (c, s),
-// or (1, 0) where the pair is orthogonal to working precision.
-__device__ __noinline__ double2 jacobi_rotation_any(double al, double be, double ga, double tol) {
-  if (!(fabs(ga) > tol * sqrt(al) * sqrt(be))) return make_double2(1.0, 0.0);
-  const double zeta = (be - al) / (2.0 * ga);
-  const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-  const double c = 1.0 / sqrt(1.0 + t * t);
-  return make_double2(c, c * t);
-}
-
 template <int RP>
-__device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int round, int np, int npair, double tol,
+__device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int round, int np, int npair, double tol2,
                                                double2* cs) {
   const int gl = threadIdx.x & 7, k = threadIdx.x >> 3;
   int p = 0, q = 0;
@@ -174,30 +157,29 @@ __device__ __forceinline__ bool jacobi_round_t(double* T, int m2, int n2, int ro
     be += __shfl_xor_sync(0xffffffffu, be, o);
     ga += __shfl_xor_sync(0xffffffffu, ga, o);
   }
-  bool rot = on && ga * ga > tol * tol * al * be;
+  const bool rot = on && ga * ga > tol2 * al * be;
   double2 cn = make_double2(1.0, 0.0);
-  const bool plain = plain_norm2(al) && plain_norm2(be);
-  if (!plain) {
-    if (on) cn = jacobi_rotation_any(al, be, ga, tol);
-    rot = cn.y != 0.0;
-  }
   if (__any_sync(0xffffffffu, rot)) {
+    double d = be - al, g2 = 2.0 * ga, h2 = fma(d, d, g2 * g2);
+    if (rot && (unsigned)__double2hiint(h2) < 0x07b00000u) {
+      // squares near the end of the exponent range (below 2^-900: columns past an
+      // exact rank, which shrink by 1e-16 a sweep): the larger norm brought to about one
+      const int k = min(1022, 1023 - (max(__double2hiint(al), __double2hiint(be)) >> 20));
+      const double f = __hiloint2double((1023 + k) << 20, 0);
+      d *= f;
+      g2 *= f;
+      h2 = fma(d, d, g2 * g2);
+    }
     // the rotation with t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
     // zeta = (be - al) / (2 ga): cos^2 = (1 + |be - al| / h) / 2 and
     // sin = 2 ga / (2 h cos), h^2 = (be - al)^2 + (2 ga)^2
-    const double d = be - al, g2 = 2.0 * ga;
-    const double rh = quick_rsqrt(fma(d, d, g2 * g2));
+    const double rh = quick_rsqrt(h2);
     const double c2 = fma(0.5 * fabs(d), rh, 0.5);
     const double rc = quick_rsqrt(c2);
-    double c = c2 * rc;
-    double sn = (d == 0.0 ? fabs(g2) : (d > 0.0 ? g2 : -g2)) * (0.5 * rh) * rc;
+    const double c = c2 * rc;
+    const double sn = (d == 0.0 ? fabs(g2) : (d > 0.0 ? g2 : -g2)) * (0.5 * rh) * rc;
     if (rot) {
-      if (plain) {
-        cn = make_double2(c, sn);
-      } else {
-        c = cn.x;
-        sn = cn.y;
-      }
+      cn = make_double2(c, sn);
 #pragma unroll
       for (int x = 0; x < RP; ++x) {
         const int r = gl + x * 8;
@@ -222,7 +204,7 @@ __device__ void jacobi_svd(double* T, int m2, int n2, double* V, double2* cs, in
   const int warp = threadIdx.x >> 5, rp = (m2 + 7) / 8;
   const bool is_t = warp < nt, is_v = warp >= v0 && warp < v1;
   const int busy = v1 > nt ? v1 : nt;             // the warps that meet at the barrier: 0 .. busy - 1
-  const double tol = 1e-15 * (double)m2;
+  const double tol = 1e-15 * (double)m2, tol2 = tol * tol;
   __syncthreads();
   for (int sweep = 0; sweep < 40; ++sweep) {
     if (threadIdx.x == 0) *s_rot = 0;
@@ -233,11 +215,11 @@ __device__ void jacobi_svd(double* T, int m2, int n2, double* V, double2* cs, in
         if (is_t && round < np - 1) {
           double2* c = cs + (round & 1) * 32;
           bool r;
-          if (rp <= 1) r = jacobi_round_t<1>(T, m2, n2, round, np, npair, tol, c);
-          else if (rp <= 2) r = jacobi_round_t<2>(T, m2, n2, round, np, npair, tol, c);
-          else if (rp <= 3) r = jacobi_round_t<3>(T, m2, n2, round, np, npair, tol, c);
-          else if (rp <= 4) r = jacobi_round_t<4>(T, m2, n2, round, np, npair, tol, c);
-          else r = jacobi_round_t<8>(T, m2, n2, round, np, npair, tol, c);
+          if (rp <= 1) r = jacobi_round_t<1>(T, m2, n2, round, np, npair, tol2, c);
+          else if (rp <= 2) r = jacobi_round_t<2>(T, m2, n2, round, np, npair, tol2, c);
+          else if (rp <= 3) r = jacobi_round_t<3>(T, m2, n2, round, np, npair, tol2, c);
+          else if (rp <= 4) r = jacobi_round_t<4>(T, m2, n2, round, np, npair, tol2, c);
+          else r = jacobi_round_t<8>(T, m2, n2, round, np, npair, tol2, c);
           rotated = rotated || r;
         }
         if (is_v && round > 0) {
@@ -356,6 +338,7 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
   extern __shared__ __align__(16) double sm[];
   __shared__ int s_rot, s_order[64];
   __shared__ double s_nrm;
+  __shared__ int s_top;
   __shared__ double2 cs[64];
   const Geom& g = a.g;
   const int D = g.D, n = 2 * D, m = D * D * D, D4 = D * D * D * D;
@@ -383,6 +366,7 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
   double* Mj = Mi + (size_t)m * n;
   double* Ni = Mj + (size_t)m * n;
   double* Nj = Ni + (size_t)m * n;
+  if (threadIdx.x == 0) s_top = 0;
   // ---- tables
   for (int e = threadIdx.x; e < 8 * D; e += blockDim.x) {
     const int site = e / (4 * D), leg = e / D % 4, x = e % D;
@@ -425,6 +409,7 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
   const int ki = min(m, n), kj = min(m, n);
   const int m2 = 2 * ki, n2 = 2 * kj;
   // ---- 3. Theta[(a, s_i'), (s_j', b)]
+  int top = 0;
   for (int e = threadIdx.x; e < m2 * n2; e += blockDim.x) {
     const int r = e / n2, c = e % n2;
     const int ai = r >> 1, sp = r & 1, sq = c / kj, bj = c % kj;
@@ -439,8 +424,21 @@ __global__ void __launch_bounds__(kT) k_su_bond(Args a) {
       v = fma(gate[(sp * 2 + sq) * 4 + q], t, v);
     }
     Th[e] = v;
+    top = max(top, __double2hiint(v) & 0x7fffffff);
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
   __syncthreads();
+  // far from one, Theta is scaled by a power of two: the SVD squares entries of
+  // its Gram matrix, and the scale drops out of the weights.  (Pairs of columns
+  // whose Gram entry is below 2^-538 of the largest, with singular values that are
+  // zero for every use, are left as they are.)
+  const int etop = (s_top >> 20) - 1023;
+  if (etop > 100 || (etop < -100 && etop > -1023)) {
+    const double f = __hiloint2double((1023 - min(etop, 1022)) << 20, 0);
+    for (int e = threadIdx.x; e < m2 * n2; e += blockDim.x) Th[e] *= f;
+    __syncthreads();
+  }
   // ---- 4. SVD; the K largest singular values, in decreasing order (equal ones by column)
   jacobi_svd(Th, m2, n2, V, cs, &s_rot);
   for (int c = threadIdx.x; c < n2; c += blockDim.x) {
