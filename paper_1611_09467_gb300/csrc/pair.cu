@@ -108,16 +108,24 @@ __global__ void __launch_bounds__(kThreads) k_pair(KArgs<R> a) {
 // 4x4 D = 2 Dc = 4 FP64, 64 configurations: 0.33 ms against 0.65 with
 // k_pair_fused (barriers around products of 64 outputs); 8x8 D = 4 Dc = 8 FP64,
 // 304 configurations: 29 against 49 ms.
-template <typename R>
+template <typename R, bool fused>
 __global__ void __launch_bounds__(32) k_pair_small(KArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t sp[kMaxWords];
   __shared__ int eH[kMaxL + 1];
-  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw), sandwich_in_fused_order<R>(a.g));
+  WarpOps<R, fused> ops(a, reinterpret_cast<R*>(smem_raw));
   pair_items<R>(a, ops, a.scratch + (size_t)blockIdx.x * a.slot_elems, sp, eH);
 }
 
 size_t pair_small_slot_elems(const Geometry& g) { return (size_t)(g.Lx + 5) * g.Dc * g.D * g.D * g.Dc; }
+
+// The kernel for a model: in the order of the fused one where both are used.
+template <typename R>
+static auto pair_small_kernel(const Geometry& g) -> void (*)(KArgs<R>) {
+  if constexpr (sizeof(R) == 8)
+    if (sandwich_in_fused_order<R>(g)) return k_pair_small<R, true>;
+  return k_pair_small<R, false>;
+}
 
 template <typename R>
 int max_blocks_pair_small(const Geometry& g) {
@@ -125,17 +133,19 @@ int max_blocks_pair_small(const Geometry& g) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = (size_t)small::ops_reals(g.D, g.Dc) * sizeof(R);
-  prefer_shared(k_pair_small<R>, smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pair_small<R>, 32, smem);
+  const auto kernel = pair_small_kernel<R>(g);
+  prefer_shared(kernel, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 32, smem);
   return nsm * (nb < 1 ? 1 : nb);
 }
 
 template <typename R>
 cudaError_t launch_pair_small(const KArgs<R>& a, int grid, cudaStream_t st) {
   const size_t smem = (size_t)small::ops_reals(a.g.D, a.g.Dc) * sizeof(R);
-  cudaError_t e = prefer_shared(k_pair_small<R>, smem);
+  const auto kernel = pair_small_kernel<R>(a.g);
+  cudaError_t e = prefer_shared(kernel, smem);
   if (e != cudaSuccess) return e;
-  k_pair_small<R><<<grid, 32, smem, st>>>(a);
+  kernel<<<grid, 32, smem, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -93,12 +93,12 @@ __global__ void __launch_bounds__(kThreads) k_row(KArgs<R> a) {
 // One warp per (configuration, row), for the models small.cuh takes: k_row's
 // contractions with each product on one warp in shared memory (small_ops.cuh).
 // 6x6 D = 3 Dc = 6 FP64, 128 configurations with Delta: 0.8 ms against 25 with k_row.
-template <typename R>
+template <typename R, bool fused>
 __global__ void __launch_bounds__(32) k_row_small(KArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t sp[kMaxWords];
   __shared__ int eG[kMaxL + 1];
-  WarpOps<R> ops(a, reinterpret_cast<R*>(smem_raw), sandwich_in_fused_order<R>(a.g));
+  WarpOps<R, fused> ops(a, reinterpret_cast<R*>(smem_raw));
   row_items<R>(a, ops, a.scratch + (size_t)blockIdx.x * a.slot_elems, sp, eG);
 }
 
@@ -107,23 +107,33 @@ size_t row_small_slot_elems(const Geometry& g) {
   return (size_t)(g.Lx + 5) * envT + (size_t)g.D * g.D * g.D * g.D;
 }
 
+// The kernel for a model: in the order of the fused one where both are used.
+template <typename R>
+static auto row_small_kernel(const Geometry& g) -> void (*)(KArgs<R>) {
+  if constexpr (sizeof(R) == 8)
+    if (sandwich_in_fused_order<R>(g)) return k_row_small<R, true>;
+  return k_row_small<R, false>;
+}
+
 template <typename R>
 int max_blocks_row_small(const Geometry& g) {
   int dev = 0, nsm = 0, nb = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = (size_t)small::ops_reals(g.D, g.Dc) * sizeof(R);
-  prefer_shared(k_row_small<R>, smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_row_small<R>, 32, smem);
+  const auto kernel = row_small_kernel<R>(g);
+  prefer_shared(kernel, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 32, smem);
   return nsm * (nb < 1 ? 1 : nb);
 }
 
 template <typename R>
 cudaError_t launch_row_small(const KArgs<R>& a, int grid, cudaStream_t st) {
   const size_t smem = (size_t)small::ops_reals(a.g.D, a.g.Dc) * sizeof(R);
-  cudaError_t e = prefer_shared(k_row_small<R>, smem);
+  const auto kernel = row_small_kernel<R>(a.g);
+  cudaError_t e = prefer_shared(kernel, smem);
   if (e != cudaSuccess) return e;
-  k_row_small<R><<<grid, 32, smem, st>>>(a);
+  kernel<<<grid, 32, smem, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -202,15 +202,13 @@ PEPS_HD bool sandwich_in_fused_order(const Geometry& g) {
 
 // fused: sums in the order of the fused kernels, for the models whose sandwiches
 // run in either (dispatch by batch size), so that results do not depend on it.
-template <typename R>
+template <typename R, bool fused = false>
 struct WarpOps {
   const KArgs<R>& a;
   R* sm;
   small::Layout L;
-  const bool fused;
 
-  __device__ WarpOps(const KArgs<R>& a_, R* sm_, bool fused_ = false)
-      : a(a_), sm(sm_), L(small::layout(a_.g.D, a_.g.Dc)), fused(fused_) {}
+  __device__ WarpOps(const KArgs<R>& a_, R* sm_) : a(a_), sm(sm_), L(small::layout(a_.g.D, a_.g.Dc)) {}
   __device__ double absorb(const R* Min, R* Mout, int row, int dir, bool lr, const int* bdin, const uint64_t* sp) {
     __syncwarp();
     return small::absorb_row<R>(a, Min, Mout, row, dir, lr, bdin, sp, sm, L);
@@ -272,13 +270,14 @@ struct WarpOps {
     R* b = r + small::up4(Dc * DD * D);
     __syncwarp();
     small::desc_gemm<R>(site_env_step(0, D, Dc), d, gg, z);
-    for (int x = 0; fused && x < Dc; ++x) {
-      small::desc_gemm<R>(small::site_fused(0, D, Dc), f + x, u, r);
-      small::desc_gemm<R>(small::site_fused(1, D, Dc), r, z + x * D * Dc * D, b, x > 0);
-    }
-    for (int x = 0; !fused && x < Dc; ++x) {
-      small::desc_gemm<R>(small::site_slice(0, D, Dc), z, u + x * D * Dc, r);
-      small::desc_gemm<R>(small::site_slice(1, D, Dc), r, f + x * D * Dc, b, x > 0);
+    for (int x = 0; x < Dc; ++x) {
+      if constexpr (fused) {
+        small::desc_gemm<R>(small::site_fused(0, D, Dc), f + x, u, r);
+        small::desc_gemm<R>(small::site_fused(1, D, Dc), r, z + x * D * Dc * D, b, x > 0);
+      } else {
+        small::desc_gemm<R>(small::site_slice(0, D, Dc), z, u + x * D * Dc, r);
+        small::desc_gemm<R>(small::site_slice(1, D, Dc), r, f + x * D * Dc, b, x > 0);
+      }
     }
     for (int k = small::lane_id(); k < DD * DD; k += 32) out[k] = b[k];
     __syncwarp();
@@ -293,16 +292,15 @@ struct WarpOps {
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
       R s = R(0);
-      if (fused) {
+      if constexpr (fused) {
         const bool one = rows * Dc <= 256;
         const int row = one ? (32 * w + small::lane_id()) % rows : 32 * w + small::lane_id();
         const int k0 = one ? (32 * w + small::lane_id()) / rows : 0, k1 = one ? k0 + 1 : Dc;
         if (row < rows && k1 <= Dc)
           for (int k = k0; k < k1; ++k) s = fma(x[row * Dc + k], y[row * Dc + k], s);
-        v[w] = s;
-        continue;
+      } else {
+        for (int e = 32 * w + small::lane_id(); e < n; e += 256) s = fma(x[e], y[e], s);
       }
-      for (int e = 32 * w + small::lane_id(); e < n; e += 256) s = fma(x[e], y[e], s);
       v[w] = s;
     }
     return small::sum256(v);
