@@ -266,14 +266,17 @@ peps_status peps_tuned_config(peps_ctx* ctx, int* vals /* [4] */, double* worksp
 
 /* Packed launches.  A packer evaluates requests of several models (contexts
  * of different lattices, D and Dc, all PEPS_FP64 or all of the FP32 family)
- * with the boundary sweeps of all requests in ONE persistent kernel launch:
+ * with the boundary sweeps of all requests in one persistent kernel launch for
+ * the models swept by one warp (Dc D <= 32, 2 <= D <= 6, zip-up truncation) and
+ * one for the others; where a pack has both, the two run side by side.  In each,
  * work items are (request, configuration, sweep direction) numbered request
  * after request, each CTA finds its request by the item's index and lays its
  * scratch slot and shared memory out for that model.  The sandwich and
- * finalisation steps then run per request.  Everything runs on the packer's
- * stream (cudaStream_t, NULL = legacy default) using each context's
- * workspace, so the contexts must have no work in flight on their own
- * streams.  Per request i: S[i] [n[i]][ceil(N_i/64)], outputs as in
+ * finalisation steps then run per request.  Everything is ordered on the
+ * packer's stream (cudaStream_t, NULL = legacy default; the second launch runs
+ * on a stream of the packer, after the work before it and before the work after
+ * it) using each context's workspace, so the contexts must have no work in
+ * flight on their own streams.  Per request i: S[i] [n[i]][ceil(N_i/64)], outputs as in
  * peps_evaluate (each array of pointers, or any of its entries, may be
  * NULL); a request must fit in one chunk of its context's workspace
  * (PEPS_EINVAL otherwise) and a context may appear once per call.  Results

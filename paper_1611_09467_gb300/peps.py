@@ -403,7 +403,8 @@ class PEPS:
 
 class Packer:
     """Packed evaluation of requests of several models (boundary sweeps of all
-    requests in one kernel launch) on the current torch stream."""
+    requests in one kernel launch, or in two side by side where some models are
+    swept by a warp) on the current torch stream."""
 
     def __init__(self):
         import torch
