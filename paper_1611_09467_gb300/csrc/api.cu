@@ -335,29 +335,49 @@ KArgs<R> make_args(peps_ctx* c, const uint64_t* S, int n, const Small& sm) {
   return a;
 }
 
+// Whether a call's sandwiches take a warp per item or a CTA.  Both give the same
+// bits, so the lines only follow the times.  A warp takes up to 2.5 times as long
+// as a CTA on one item, but more of them share an SM than the two generic CTAs (one
+// in FP64).  Two-row steps, time on warps over time on CTAs by items per SM (0.1, 1,
+// 2, 3, 4, 6), 8x8, FP32:
+//   D = 2 Dc = 8   1.02 1.09 0.91 0.53 0.48 0.35 (5x4 0.59 0.58 0.52 0.30 0.28 0.21)
+//   D = 2 Dc = 16  1.35 1.39 1.24 0.71 0.66 0.46
+//   D = 3 Dc = 4   0.85 0.92 0.76 0.45 0.40 0.31    D = 4 Dc = 3  1.01 1.01 0.87 0.50 0.46 0.37
+//   D = 3 Dc = 6   1.28 1.34 1.12 0.66 0.60 0.45    D = 4 Dc = 4  1.30 1.29 1.08 0.63 0.59 0.45
+//   D = 3 Dc = 8   2.05 2.22 1.81 1.05 0.96 0.72    D = 4 Dc = 6  1.82 1.93 1.60 0.92 0.85 0.65
+//   D = 3 Dc = 10  2.55 2.74 2.24 1.29 1.18 0.87    D = 4 Dc = 7  2.39 2.49 1.95 1.15 1.04 0.80
+//   D = 5 Dc = 2   0.91 0.93 0.79 0.47 0.43 0.33    D = 6 Dc = 3  0.96 0.95 0.79 0.47 0.42 0.32
+//   D = 5 Dc = 5   2.07 2.03 1.77 1.04 0.94 0.73    D = 6 Dc = 5  1.64 1.62 1.33 0.78 0.71 0.55
+//   D = 5 Dc = 6   2.28 2.42 2.01 1.18 1.07 0.82
+// FP64: below 0.76 at one item and less above for D = 3, D = 4 Dc = 6, D = 5 and 6 Dc = 4;
+// D = 4 Dc = 7 0.98 1.05 0.64; D = 5 Dc = 6 1.37 1.46 0.89; D = 6 Dc = 5 1.03 1.04 0.62;
+// against the fused kernel at D = 4 Dc = 8 1.48 1.58 1.53 0.92 0.84 0.66.
+bool pair_on_warps(const peps_ctx* c, int items) {
+  const Geometry& g = c->g;
+  if (!small_boundary(c) || !c->res_pair_small || c->pair_mode != 0) return false;
+  const int q = g.D * g.Dc;
+  if (c->elem == 8) {
+    if (sandwich_in_fused_order<double>(g)) return items >= 3 * c->nsm;
+    return g.D <= 4 || q < 25 || items > c->nsm;
+  }
+  if (q <= 12 || (g.D == 2 && g.Dc < 12) || (g.D == 6 && g.Dc <= 3)) return true;
+  return items > (q < 28 || g.D == 2 || g.D == 6 ? 2 : 4) * c->nsm;
+}
+// Single-row steps (8x8, ratio by items per SM, 0.1 and 1): FP32 0.55 0.47 at D = 3 Dc = 4,
+// 0.94 0.76 at D = 4 Dc = 6, 1.07 0.85 at D = 5 Dc = 6, the largest; FP64 below 0.43 and
+// 0.25, against the fused kernel at D = 4 Dc = 8 1.4 up to two items per SM and 0.7 above.
+bool row_on_warps(const peps_ctx* c, int items) {
+  const Geometry& g = c->g;
+  if (!small_boundary(c) || !c->res_row_small || c->row_generic) return false;
+  return c->elem == 4 || !sandwich_in_fused_order<double>(g) || items > 2 * c->nsm;
+}
+
 // Single-row and two-row sandwich steps and the E(S)/status finalisation of
 // one chunk whose environments are in place, on stream st.
 template <typename R>
 peps_status sandwich_chunk(peps_ctx* c, const KArgs<R>& a, const uint64_t* S, int n, bool need_env_l,
                            bool need_pairs, Small& sm, cudaStream_t st) {
-  // One-warp kernels: as many items side by side as are resident and have a slot.
-  // A warp takes two to four times as long as a CTA on one item (8x8 FP32 two-row
-  // D = 5 Dc = 6: 6.8 against 2.4 ms a wave; FP64 D = 4 Dc = 8: 13 against 8.5) but
-  // four times as many run side by side, so they are the better ones from a few
-  // items per SM on (at 152 configurations 7.6 against 9.8 ms and 15 against 29
-  // ms).  Two-row transfers of up to 400 entries are faster on a warp at any
-  // number (FP64 D = 3 Dc = 6, one configuration: 3.5 against 9.7 ms), and so are
-  // single-row ones but for FP64 D = 4 Dc = 8, whose fused kernel is ahead up to
-  // two items per SM (1.8 against 2.3 ms; 3.4 against 2.3 above).
-  const Geometry& g = c->g;
-  const bool warps = small_boundary(c);
-  const bool tiny = g.Dc * g.Dc * g.D * g.D <= 400;
-  const bool row_warps = warps && c->res_row_small && !c->row_generic &&
-                         (tiny || !row_has_fused(g) || n * g.Ly > 2 * c->nsm);
-  // two-row items per SM from which warps are ahead: against the fused kernel in FP64, the generic one in FP64, in FP32
-  const int pair_few = c->elem == 8 ? (row_has_fused(g) ? 3 : 1) : 6;
-  const bool pair_warps = warps && c->res_pair_small && c->pair_mode == 0 &&
-                          (tiny || n * (g.Ly - 1) >= pair_few * c->nsm);
+  // one-warp kernels: as many items side by side as are resident and have a slot
   auto warp_grid = [&](KArgs<R>& b, size_t slot, int items, int res) {
     b.slot_elems = (slot + 31) / 32 * 32;
     const size_t slots = scratch_bytes(c, c->nslots) / c->elem / b.slot_elems;
@@ -366,7 +386,7 @@ peps_status sandwich_chunk(peps_ctx* c, const KArgs<R>& a, const uint64_t* S, in
   if (need_env_l) {
     const int items = n * c->g.Ly;
     Prof pf(c, 1);
-    if (row_warps) {
+    if (row_on_warps(c, items)) {
       KArgs<R> b = a;
       const int grid = warp_grid(b, row_small_slot_elems(c->g), items, c->res_row_small);
       PEPS_CUDA(launch_row_small<R>(b, grid, st));
@@ -384,7 +404,7 @@ peps_status sandwich_chunk(peps_ctx* c, const KArgs<R>& a, const uint64_t* S, in
       tc = c->pair_tc && c->pair_mode == 0;
       if (tc) PEPS_CUDA(launch_pair_tc(a, grid, st));
     }
-    if (!tc && pair_warps) {
+    if (!tc && pair_on_warps(c, items)) {
       KArgs<R> b = a;
       const int wgrid = warp_grid(b, pair_small_slot_elems(c->g), items, c->res_pair_small);
       PEPS_CUDA(launch_pair_small<R>(b, wgrid, st));

@@ -97,6 +97,14 @@ size_t dyn_smem_bytes(const Geometry& g, size_t elem, bool truncates, bool wm_in
 template <typename R> int max_blocks_mc(const Geometry& g);
 // Sandwiches with one warp per item, for the models boundary_small_fits accepts.
 bool row_has_fused(const Geometry& g);
+// The small models whose sandwiches run in the fused kernels or on warps, by the
+// size of the batch: in FP64 D = 4, Dc = 8 (FP32 always takes the fused kernels where
+// there are any, FP64 D = 2, Dc = 4 always warps).  Their one-warp kernels sum in the
+// order of the fused ones.
+template <typename R>
+inline bool sandwich_in_fused_order(const Geometry& g) {
+  return sizeof(R) == 8 && g.D == 4 && g.Dc == 8;
+}
 size_t row_small_slot_elems(const Geometry& g);
 size_t pair_small_slot_elems(const Geometry& g);
 template <typename R> int max_blocks_row_small(const Geometry& g);

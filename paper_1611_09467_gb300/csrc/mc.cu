@@ -168,10 +168,13 @@ __global__ void __launch_bounds__(kThreads) k_mc(KArgs<R> a, uint64_t* S, int ns
   mc_chains<R>(a, ops, p, sp, ones, eH, S, nsweeps, seed, chain0, sweep0, accepted);
 }
 
-// One warp per chain (models small.cuh takes).  304 chains of 8x8 D = 4 Dc = 8 in
-// FP64 take 105 ms a sweep against 397 ms with a CTA each, whose time went to the
-// truncation's barriers and FP64 sections and to the tiled engine's offset
-// tables on products of a few hundred outputs.
+// One warp per chain (models small.cuh takes), at any number of chains: on one
+// chain too a warp is not behind a CTA (8x8, ms a sweep: FP32 10.0 against 20.0 at D = 2
+// Dc = 8, 24.1 against 30.4 at D = 4 Dc = 6, 38.8 against 38.3 at D = 5 Dc = 6, the closest;
+// FP64 101 against 128 at D = 4 Dc = 8, 145 against 156 at D = 5 Dc = 6; alike for 152).  304
+// chains of 8x8 D = 4 Dc = 8 in FP64 take 105 ms a sweep against 397 ms with a CTA each,
+// whose time went to the truncation's barriers and FP64 sections and to the tiled
+// engine's offset tables on products of a few hundred outputs.
 template <typename R>
 __global__ void __launch_bounds__(32) k_mc_small(KArgs<R> a, uint64_t* S, int nsweeps, uint64_t seed, uint64_t chain0,
                                                  uint64_t sweep0, long long* accepted) {

@@ -192,14 +192,6 @@ __device__ __forceinline__ R* stage(R*& p, const R* src, int n) {
 
 }  // namespace small
 
-// The small models whose sandwiches run in the fused kernels or on warps, by the
-// size of the batch: in FP64 D = 4, Dc = 8 (FP32 always takes the fused kernels where
-// there are any, FP64 D = 2, Dc = 4 always warps).
-template <typename R>
-PEPS_HD bool sandwich_in_fused_order(const Geometry& g) {
-  return sizeof(R) == 8 && g.D == 4 && g.Dc == 8;
-}
-
 // fused: sums in the order of the fused kernels, for the models whose sandwiches
 // run in either (dispatch by batch size), so that results do not depend on it.
 template <typename R, bool fused = false>

@@ -23,10 +23,11 @@ def built():
     (4, 4, 4, 8, "fp64"), (5, 2, 4, 8, "fp64"), (4, 4, 4, 7, "fp64"), (3, 4, 5, 6, "fp64"), (4, 3, 3, 10, "fp64"),
     (4, 4, 2, 16, "fp64"), (3, 4, 6, 5, "fp64"), (4, 4, 3, 6, "fp64"),
     (4, 4, 4, 7, "fp32"), (3, 4, 5, 6, "fp32"), (4, 3, 3, 10, "fp32"), (4, 4, 2, 16, "fp32"), (3, 4, 6, 5, "fp32"),
+    (4, 4, 4, 5, "fp32"), (4, 4, 3, 6, "fp32"), (4, 4, 5, 2, "fp32"), (4, 4, 5, 5, "fp64"),
 ])
 def test_results_do_not_depend_on_the_batch(Lx, Ly, D, Dc, prec):
     from paper_1611_09467_gb300.peps import PEPS
-    n = 2100   # the two-row items of a batch of n pass the warps that are resident; six items an SM is the highest line
+    n = 2100   # the two-row items of a batch of n pass the warps that are resident; four items an SM is the highest line
     A = inputs.near_product_tensors(Ly, Lx, D, 97)
     S = torch.from_numpy(inputs.pack_spins(inputs.random_sz0(n, Lx * Ly, 98)).view(np.int64)).cuda()
     m = PEPS(A, Lx, Ly, D, Dc, J1=1.0, J2=0.5, prec=prec)
