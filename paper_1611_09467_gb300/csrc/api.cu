@@ -116,7 +116,7 @@ struct peps_ctx {
   int chunk = 0;  // configurations per pass
   // resident CTAs of the one-warp kernels (0: the model is too large for them,
   // or another kernel is the better one for it)
-  int res_small = 0, res_row_small = 0, res_pair_small = 0;
+  int res_small = 0, res_row_small = 0, res_pair_small = 0, res_mc_small = 0;
   int res_boundary = 0, res_row = 0, res_pair = 0, res_mc = 0;  // resident CTAs per kernel
   bool pair_tc = false;  // two-row step on the tensor cores (PEPS_MIXED_TF32, D = 8, Dc = 16)
   // kernel variants (peps_autotune): row_generic 1 takes the generic single-row
@@ -602,7 +602,7 @@ peps_status mc_impl(peps_ctx* c, uint64_t* S, int n, int nsweeps, uint64_t seed,
     a.slot_elems = (mc_small_slot_elems(c->g) + 31) / 32 * 32;
     // as many chains side by side as are resident and have a slot (a CTA's slot holds two or three)
     const int slots = (int)std::min<size_t>(scratch_bytes(c, c->nslots) / c->elem / a.slot_elems, 1u << 20);
-    const int grid = std::max(1, std::min(n, std::min(slots, max_blocks_mc_small<R>(c->g))));
+    const int grid = std::max(1, std::min(n, std::min(slots, c->res_mc_small)));
     Prof pf(c, 7);
     PEPS_CUDA(launch_mc_small<R>(a, S, nsweeps, seed, chain0, sweep0, (long long*)accepted, grid, c->stream));
     return PEPS_OK;
@@ -918,6 +918,7 @@ peps_ctx* ctx_clone(peps_ctx* c, cudaStream_t stream, double workspace_gb, int s
   k->res_small = c->res_small ? part(c->res_small) : 0;
   k->res_row_small = c->res_row_small ? part(c->res_row_small) : 0;
   k->res_pair_small = c->res_pair_small ? part(c->res_pair_small) : 0;
+  k->res_mc_small = c->res_mc_small ? part(c->res_mc_small) : 0;
   k->res_boundary = part(c->res_boundary);
   k->res_row = part(c->res_row);
   k->res_pair = part(c->res_pair);
@@ -1027,6 +1028,7 @@ peps_status peps_create(const peps_params* p, const double* A_host, void* stream
     const size_t smem = boundary_small_smem(c->g, c->elem);
     c->res_small = c->elem == 8 ? max_blocks_boundary_small<double>(smem)
                                 : max_blocks_boundary_small<float>(smem);
+    c->res_mc_small = c->elem == 8 ? max_blocks_mc_small<double>(c->g) : max_blocks_mc_small<float>(c->g);
     // sandwiches: always in FP64; in FP32 where there is no fused kernel
     if (c->elem == 8) {
       c->res_row_small = max_blocks_row_small<double>(c->g);
