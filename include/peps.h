@@ -242,12 +242,13 @@ peps_status peps_graph_stats(peps_ctx* ctx, long long* stats);
 /* Autotuner.  Times full gradient passes (one untimed, one timed, CUDA
  * events on the context's stream) over the probe batch S_dev [n] for each
  * candidate, one setting after another, and keeps the fastest:
- *   - the two-row kernel: tensor cores (PEPS_MIXED_TF32, D = 8, Dc = 16),
- *     the fused shared-memory kernel (where one exists for (D, Dc)), or the
+ *   - the two-row kernel: tensor cores (PEPS_MIXED_TF32, D = 8, Dc = 16), the
+ *     default (a warp per item where models with Dc D <= 32 have enough items,
+ *     else the fused shared-memory kernel where one exists for (D, Dc)), or the
  *     generic one;
- *   - the single-row kernel: fused (where one exists) or generic;
- *   - the persistent grid of the boundary sweeps: the resident CTA count or
- *     half of it;
+ *   - the single-row kernel: the default (as above) or generic;
+ *   - the persistent grid of the boundary sweeps: the resident CTA count (of
+ *     one-warp CTAs where a warp sweeps) or half of it;
  *   - the workspace budget (configurations per chunk): the current one, x2,
  *     x4 (within 60% of device memory), tried only when the probe batch
  *     spans more than one chunk.
@@ -259,8 +260,9 @@ peps_status peps_graph_stats(peps_ctx* ctx, long long* stats);
 peps_status peps_autotune(peps_ctx* ctx, const uint64_t* S_dev, int n, char* report, size_t report_len);
 
 /* The context's kernel settings: vals[0] two-row kernel (0 tensor cores,
- * 1 fused, 2 generic), vals[1] single-row kernel (0 fused, 1 generic),
- * vals[2] boundary-sweep CTAs, vals[3] configurations per chunk of the last
+ * 1 fused, 2 generic, 3 a warp per item, or 1 / 2 in calls of few items),
+ * vals[1] single-row kernel (0 fused, 1 generic, 2 a warp per item, likewise),
+ * vals[2] boundary-sweep CTAs (or warps), vals[3] configurations per chunk of the last
  * call; *workspace_gb the workspace budget. */
 peps_status peps_tuned_config(peps_ctx* ctx, int* vals /* [4] */, double* workspace_gb);
 

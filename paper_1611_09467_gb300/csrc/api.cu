@@ -123,7 +123,7 @@ struct peps_ctx {
   // kernel; pair_mode 0 the default two-row kernel (tensor cores where
   // pair_tc, else fused where one exists), 1 the fused SIMT kernel, 2 the generic one
   int row_generic = 0, pair_mode = 0;
-  int boundary_ctas = 0;   // 0: the boundary kernel's resident CTA count, else this many (peps_autotune)
+  int boundary_div = 1;   // the boundary sweeps' grid: the resident CTA count divided by this (peps_autotune)
   DevBuf corr_sites, corr_x, corr_scratch;   // correlation functions (peps_correlations)
   // environment cache (peps_set_env_cache): the bits of the configurations
   // whose boundary sweeps are in env, and per configuration which sweeps are
@@ -274,6 +274,13 @@ size_t slot_elems(const peps_ctx* c) {
 
 // Whether the boundary sweeps take the one-warp kernel.
 bool small_boundary(const peps_ctx* c) { return c->res_small > 0 && boundary_small_fits(c->g); }
+
+// Persistent grid of the boundary sweeps: the resident CTAs (of one warp where the
+// sweeps take that kernel) or the autotuner's choice.
+int boundary_grid(const peps_ctx* c) {
+  const int res = small_boundary(c) ? c->res_small : c->res_boundary;
+  return std::max(res / c->boundary_div, 1);
+}
 
 // Scratch of the persistent kernels: a slot per resident CTA; the one-warp
 // sweeps keep one boundary MPS each.
@@ -464,10 +471,9 @@ peps_status evaluate_chunk(peps_ctx* c, const uint64_t* S, int n, bool need_env_
     Prof pf(c, 0);
     PEPS_CUDA(launch_boundary_small<R>(a, nullptr, nullptr, 0, dirs, a.scratch, slot,
                                        boundary_small_smem(c->g, c->elem),
-                                       std::max(std::min(n * dirs, c->res_small), 1), c->stream));
+                                       std::max(std::min(n * dirs, boundary_grid(c)), 1), c->stream));
   } else {
-    const int res = c->boundary_ctas > 0 ? std::min(c->boundary_ctas, c->res_boundary) : c->res_boundary;
-    const int grid = std::min(n * dirs, std::min(c->nslots, res));
+    const int grid = std::min(n * dirs, std::min(c->nslots, boundary_grid(c)));
     Prof pf(c, 0);
     PEPS_CUDA(launch_boundary<R>(a, nullptr, nullptr, 0, dirs, a.scratch, a.slot_elems,
                                  dyn_smem_bytes(c->g, c->elem, true, c->wm_smem), std::max(grid, 1), c->stream));
@@ -727,7 +733,7 @@ struct TuneKey {
   }
 };
 struct TuneVal {
-  int row_generic, pair_mode, boundary_ctas;
+  int row_generic, pair_mode, boundary_div;
   double workspace_gb;
 };
 std::vector<std::pair<TuneKey, TuneVal>> g_tuned;   // choices of peps_autotune in this process
@@ -1060,7 +1066,7 @@ peps_status peps_create(const peps_params* p, const double* A_host, void* stream
       if (kv.first == tune_key(c)) {
         c->row_generic = kv.second.row_generic;
         c->pair_mode = kv.second.pair_mode;
-        c->boundary_ctas = kv.second.boundary_ctas;
+        c->boundary_div = kv.second.boundary_div;
         if (c->p.workspace_gb <= 0) c->p.workspace_gb = kv.second.workspace_gb;
         apply_variants(c);
       }
@@ -1261,9 +1267,11 @@ peps_status peps_tuned_config(peps_ctx* c, int* vals, double* workspace_gb) {
   if (!c) return fail(PEPS_EINVAL, "null context");
   if (vals) {
     const bool fused = c->elem == 8 ? max_blocks_pair_fused<double>(c->g) > 0 : max_blocks_pair_fused<float>(c->g) > 0;
+    const bool warps = small_boundary(c);
     vals[0] = c->pair_tc && c->pair_mode == 0 ? 0 : ((c->pair_mode == 2 || !fused) ? 2 : 1);
-    vals[1] = c->row_generic;
-    vals[2] = c->boundary_ctas > 0 ? std::min(c->boundary_ctas, c->res_boundary) : c->res_boundary;
+    if (warps && c->res_pair_small && c->pair_mode == 0) vals[0] = 3;
+    vals[1] = warps && c->res_row_small && !c->row_generic ? 2 : c->row_generic;
+    vals[2] = boundary_grid(c);
     vals[3] = c->chunk;
   }
   if (workspace_gb) *workspace_gb = c->p.workspace_gb > 0 ? c->p.workspace_gb : 24.0;
@@ -1327,12 +1335,18 @@ peps_status peps_autotune(peps_ctx* c, const uint64_t* S, int n, char* report, s
   };
   const bool fp64 = c->elem == 8;
   const bool fused_pair = fp64 ? max_blocks_pair_fused<double>(c->g) > 0 : max_blocks_pair_fused<float>(c->g) > 0;
+  // what the default setting runs for this batch, where that is a warp per item
+  const int pair_mode = c->pair_mode, row_generic = c->row_generic;
+  c->pair_mode = c->row_generic = 0;
+  const bool pair_warps = pair_on_warps(c, n * (c->g.Ly - 1)), row_warps = row_on_warps(c, n * c->g.Ly);
+  c->pair_mode = pair_mode;
+  c->row_generic = row_generic;
   std::vector<int> pc;
   if (c->pair_tc) pc.push_back(0);
-  if (fused_pair) pc.push_back(1);
+  if (fused_pair || pair_warps) pc.push_back(1);
   pc.push_back(2);
-  static const char* pnames[] = {"tensor-core", "fused", "generic"};
-  static const char* rnames[] = {"fused", "generic"};
+  const char* const pnames[] = {"tensor-core", pair_warps ? "one-warp" : "fused", "generic"};
+  const char* const rnames[] = {row_warps ? "one-warp" : "fused", "generic"};
   if (c->g.Ly > 1 && pc.size() > 1)
     st = pick("two-row kernel", pc, [&](int v) { c->pair_mode = v == 1 && !c->pair_tc ? 0 : v; apply_variants(c); },
               [&](int v) { return pnames[v]; });
@@ -1341,13 +1355,12 @@ peps_status peps_autotune(peps_ctx* c, const uint64_t* S, int n, char* report, s
               [&](int v) { return rnames[v]; });
   std::vector<std::string> bnames;
   if (st == PEPS_OK) {
-    std::vector<int> bc = {c->res_boundary};
-    if (c->res_boundary / 2 >= c->nsm) bc.push_back(c->res_boundary / 2);
-    for (int v : bc) bnames.push_back(std::to_string(v) + " CTAs");
-    std::vector<int> idx;
-    for (size_t i = 0; i < bc.size(); ++i) idx.push_back((int)i);
-    st = pick("boundary grid", idx, [&](int i) { c->boundary_ctas = bc[i]; },
-              [&](int i) { return bnames[i].c_str(); });
+    c->boundary_div = 1;
+    std::vector<int> divs = {1};
+    if (boundary_grid(c) / 2 >= c->nsm) divs.push_back(2);
+    for (int d : divs) bnames.push_back(std::to_string(boundary_grid(c) / d) + (small_boundary(c) ? " warps" : " CTAs"));
+    st = pick("boundary grid", divs, [&](int d) { c->boundary_div = d; },
+              [&](int d) { return bnames[d - 1].c_str(); });
   }
   if (st == PEPS_OK) {
     // a larger workspace budget means fewer chunks (fewer partial last waves)
@@ -1374,7 +1387,7 @@ peps_status peps_autotune(peps_ctx* c, const uint64_t* S, int n, char* report, s
   if (st != PEPS_OK) return st;
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    TuneVal v{c->row_generic, c->pair_mode, c->boundary_ctas, c->p.workspace_gb};
+    TuneVal v{c->row_generic, c->pair_mode, c->boundary_div, c->p.workspace_gb};
     bool found = false;
     for (auto& kv : g_tuned)
       if (kv.first == tune_key(c)) {

@@ -371,8 +371,8 @@ class PEPS:
         v = np.zeros(4, dtype=np.int32)
         ws = ctypes.c_double()
         check(lib().peps_tuned_config(self.h, _ptr(v), ctypes.byref(ws)))
-        return dict(two_row_kernel=["tensor-core", "fused", "generic"][v[0]],
-                    single_row_kernel=["fused", "generic"][v[1]], boundary_ctas=int(v[2]),
+        return dict(two_row_kernel=["tensor-core", "fused", "generic", "one-warp"][v[0]],
+                    single_row_kernel=["fused", "generic", "one-warp"][v[1]], boundary_ctas=int(v[2]),
                     configs_per_chunk=int(v[3]), workspace_gb=ws.value)
 
     def mc_sweep(self, S, nsweeps, seed, chain0=0, sweep0=0):
