@@ -1,5 +1,5 @@
 // One boundary sweep of one configuration (Fig. 1d), shared by the kernels that
-// absorb rows with a CTA (kernels.cu) and with a warp (small.cu).
+// absorb rows with a CTA (boundary.cuh) and with a warp (small.cu).
 #pragma once
 
 #include "kernels_common.cuh"

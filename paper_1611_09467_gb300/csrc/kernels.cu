@@ -1,29 +1,16 @@
-// CUDA kernels of the PEPS sampling path (sm_103a): layouts, the boundary
-// sweeps, E_loc and gradient reductions, the GO update and the
-// allocation-free amplitudes.  The sandwich kernels are in row.cu and pair.cu,
-// the Metropolis kernel in mc.cu.
+// Layouts and sizes of the scratch slots, the environment cache's check, the
+// reductions over sandwiches and configurations, and the GO update (sm_103a).  The
+// boundary sweeps are in boundary.cuh (a CTA each) and small.cu (a warp each), the
+// allocation-free amplitudes in static.cu, the sandwiches in row.cu and pair.cu,
+// the Metropolis chains in mc.cu, the correlations in corr.cu.
 //
-//   k_boundary : boundary-MPS sweeps (Fig. 1d): top-down U_r (gives ln|psi|,
-//                sign) and bottom-up L_r, alternating zip-up with truncation
-//                to Dc.  One CTA per (configuration, sweep direction).
-//   k_row      : single-row sandwiches <U_{r-1}| row r |L_{r+1}>: W_r,
-//                amplitude ratios of horizontal spin exchanges, Delta = B/W
-//                (Sec. II).  One CTA per (configuration, row).  k_row_fused
-//                is the same with every intermediate in shared memory, for
-//                (D, Dc) = (2,4), (4,8), (6,12), (8,16).
-//   k_pair     : two-row sandwiches <U_{r-1}| rows r,r+1 |L_{r+2}>: ratios
-//                of vertical and diagonal exchanges.  One CTA per
-//                (configuration, row pair).
 //   k_finalize : E(S) = diagonal + sum of (J/2) ratios (Sec. II with the
 //                Hamiltonian of Sec. IV), status.
 //   k_grad_*   : sums of O and E*O over configurations for
 //                dE/dA = 2<Delta E> - 2<Delta><E> (Sec. II).
-//   k_mc       : Metropolis sweeps over nearest-neighbour spin exchanges.
 //
 // Kernels are persistent over work items (grid-stride), so the per-CTA
 // scratch slots bound the workspace.
-#include <mutex>
-
 #include "kernels_common.cuh"
 
 namespace peps {

@@ -61,10 +61,6 @@ PEPS_HD Layout layout(int D, int Dc) {
   l.total = l.vb + kP;
   return l;
 }
-template <typename R>
-size_t smem_bytes(const Geometry& g) {
-  return (size_t)layout(g.D, g.Dc).total * sizeof(R);
-}
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 

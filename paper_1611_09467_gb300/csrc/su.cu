@@ -7,8 +7,9 @@
 // A two-site gate on bond (i, j) is applied by one CTA:
 //   1. M_i = Gamma_i with the weights of its three other bonds and of the
 //      bond itself absorbed, as a matrix [(outer legs), (s, x)]; M_j likewise
-//      (without the bond's weight).  Column-major in the CTA's scratch slot.
-//   2. Householder QR of each (m = D^3 rows, n = 2D columns): M = Q R (qr.cuh).
+//      (without the bond's weight).  Column-major, in shared memory for D <= 7, else
+//      in the CTA's scratch slot.
+//   2. Householder QR of each (m = D^3 rows, n = 2D columns): M = Q R.
 //   3. Theta[(a, s_i'), (s_j', b)] = sum G[s_i' s_j', s_i s_j] R_i[a, (s_i, x)] R_j[b, (s_j, x)].
 //   4. One-sided Jacobi SVD of Theta (columns rotated until orthogonal):
 //      the D largest singular values, normalised, are the new weight; the
@@ -313,7 +314,7 @@ struct Args {
   double* lam;             // [nbonds][D]
   const Upd* ups;          // this launch's updates, one per CTA
   double J1, J2, dtau;
-  double* scratch;         // per CTA: 4 m n doubles (M_i, M_j, N_i, N_j)
+  double* scratch;         // D > 7, per CTA: 4 m n doubles (M_i, M_j, N_i, N_j)
   size_t slot;
 };
 
@@ -644,14 +645,14 @@ peps_status peps_su_create(const peps_params* p, void* stream, peps_su** out) {
         }
   }
   const int D = p->D, m = D * D * D, n = 2 * D;
-  s->slot = (size_t)4 * m * n;
+  s->slot = su::mats_in_smem(D) ? 0 : (size_t)4 * m * n;
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&s->nsm, cudaDevAttrMultiProcessorCount, dev);
   const size_t N = (size_t)Lx * Ly, D4 = (size_t)D * D * D * D;
   cudaError_t e = cudaMalloc((void**)&s->ups, sizeof(su::Upd) * ups.size());
   if (e == cudaSuccess) e = cudaMemcpy(s->ups, ups.data(), sizeof(su::Upd) * ups.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&s->scratch, sizeof(double) * s->slot * s->max_count);
+  if (e == cudaSuccess && s->slot) e = cudaMalloc((void**)&s->scratch, sizeof(double) * s->slot * s->max_count);
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->A0, sizeof(double) * N * 2 * D4);
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->A1, sizeof(double) * N * 2 * D4);
   if (e == cudaSuccess) e = cudaMalloc((void**)&s->chg, 2 * sizeof(unsigned long long));
