@@ -36,12 +36,13 @@ UNIT = "configs/s"
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per configuration
 # of a kernel, from one ncu capture of 32 configurations of the same kernel
-# build (two launches: two-row tensor-core kernel 1766.7 and 1767.2 MB);
-# traffic grows in proportion to the configurations a launch processes.  It
-# describes that build only: re-measure it, or drop the entry, when the
-# kernel changes.  The boundary kernel has changed since its last capture,
-# so it has no entry (its traffic is reported as null).
-DRAM_BYTES_PER_CONFIG = {("16x16_D8_Dc16", "float", "pair_sandwich"): 5.52e7}
+# build (two launches each: boundary 174.1 and 171.0 MB, single-row 424.9 and
+# 424.9, two-row on the tensor cores 1694.9 and 1694.2); traffic grows in
+# proportion to the configurations a launch processes.  It describes that
+# build only: re-measure it, or drop the entry, when the kernel changes.
+DRAM_BYTES_PER_CONFIG = {("16x16_D8_Dc16", "float", "boundary"): 5.39e6,
+                         ("16x16_D8_Dc16", "float", "row_sandwich"): 1.328e7,
+                         ("16x16_D8_Dc16", "float", "pair_tc"): 5.30e7}
 
 
 def parse():
@@ -305,7 +306,7 @@ def run_ours(args, rank, world, local_rank):
             peak, bound, src = peaks["fp64_simt"], "alu", "measured: FP64 FMA on the SIMT pipe (peps_measure_peaks)"
         else:
             peak, bound, src = peaks["fp32_simt"], "alu", "measured: FP32 FMA on the SIMT pipe (peps_measure_peaks)"
-        bpc = DRAM_BYTES_PER_CONFIG.get((args.workload, fp, kname))
+        bpc = DRAM_BYTES_PER_CONFIG.get((args.workload, fp, "pair_tc" if kname == "pair_sandwich" and tc else kname))
         out = {"bound": bound, "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                "frac": achieved / peak, "traffic": bpc * n * args.steps / launches_k if bpc else None,
                "traffic_unit": "bytes per launch (DRAM read + write, ncu)", "peak_source": src,
